@@ -415,7 +415,14 @@ int mat_get_plan(gbs_mat A, int32_t *spmv_rows, int32_t *update_rows, int32_t *k
  *   GBS_SOLVER_AUTO (default): CTA when the largest system solved has at
  *     most 40000 nonzeros plus eight per row (the FP64 work of one iteration
  *     that one SM does faster than the phase kernels' fixed cost per
- *     iteration), or a batched solve has at least 2 systems per SM.
+ *     iteration), or a batched solve has at least 2 systems per SM; else
+ *     PHASES.  One system of at most 3,145,728 rows whose plan is automatic
+ *     runs FP64 CG (textbook form, no host_loop) as one launch of a team of
+ *     CTAs -- a thread-block cluster, or one CTA per SM launched
+ *     cooperatively, whose bounded waits (about a second) end the solve with
+ *     GBS_ERR_TIMEOUT -- with the same iteration up to reduction order;
+ *     ksp_result.solver names the solver it stands in for, and phase times
+ *     are reported as for the phase kernels.
  * ksp_result.solver tells which one ran.  No synchronisation.
  */
 int mat_set_solver(gbs_mat A, int32_t solver);
@@ -472,7 +479,8 @@ int mat_get_tuning(gbs_mat A, int32_t *solver, int32_t *cg_form, int64_t *split_
  *
  * mat_autotune_file: the same, persisted.  path names a text file (created if
  * missing) of one line per tuned key: "<key> | Ra Re kernel ctas_per_sm
- * solver cg_form split_rows patterns | <time>" (lines without the last one
+ * solver cg_form split_rows patterns | <time>" (patterns: 0 or 1, plus 2 where one
+ * system's CG runs on the team of CTAs; lines without the last one
  * or two fields leave those settings as they are).  The key holds the handle's sizes, a hash of its
  * systems' sizes and of 257 sampled entries each of row_ptr and col, the
  * device name and SM count, and "fp64".  A matching line is applied without

@@ -476,6 +476,7 @@ int mat_set_solver(gbs_mat A, int32_t solver) {
   if (solver != A->solver) drop_graphs(A);  // a split loop's graph skips the small systems
   A->solver = solver;
   A->solver_batched_only = false;
+  A->team_tuned = false;
   return GBS_OK;
 }
 
@@ -522,6 +523,7 @@ struct Tuning {
   int32_t Ra, Re, kernel, cpsm, solver, cg_form;
   int64_t split_rows;
   int32_t patterns;  // column patterns of the sliced copy (1 / 0; -1: as they are)
+  int32_t team;      // one system: the team of CTAs instead of the phase kernels
 };
 
 // Makes t the handle's plan (rebuilt only when it differs from the current
@@ -535,13 +537,15 @@ int apply_tuning(gbs_mat A, const Tuning &t, cudaStream_t s) {
   A->solver_batched_only = A->nsys > 1;  // tuned on the batched solve
   A->cg_form = t.cg_form;
   A->split_rows = t.split_rows;
+  A->team_tuned = t.team != 0 && A->nsys == 1;
   return GBS_OK;
 }
 
 // The resolved plan of the handle with its solver and form.
 Tuning current_tuning(gbs_mat A) {
   return Tuning{A->Ra,     A->Re,         A->lanes,      A->ctas_per_sm,
-                A->solver, A->cg_form,    A->split_rows, A->sell_patterns ? 1 : 0};
+                A->solver, A->cg_form,    A->split_rows, A->sell_patterns ? 1 : 0,
+                A->team_tuned ? 1 : 0};
 }
 
 // 257 evenly spaced entries each of row_ptr and col (the cache key's sample).
@@ -579,7 +583,7 @@ static int autotune(gbs_mat A, cudaStream_t s, Tuning *out, float *out_ms) {
   cudaEventCreate(&e1);
   const int32_t pat = A->sell_patterns ? 1 : 0;
   Tuning best{A->Ra, A->Re, A->lanes, A->ctas_per_sm, GBS_SOLVER_PHASES, GBS_CG_TEXTBOOK,
-              A->split_rows, pat};
+              A->split_rows, pat, 0};
   float best_ms = 1e30f;
   int st = GBS_OK;
   std::vector<std::pair<float, Tuning>> tried;
@@ -618,7 +622,7 @@ static int autotune(gbs_mat A, cudaStream_t s, Tuning *out, float *out_ms) {
       if (pass == 1 && c[2] != GBS_SPMV_SELL) continue;  // patterns concern the sliced copy
       for (int32_t form : {GBS_CG_TEXTBOOK, GBS_CG_SINGLE_REDUCTION}) {
         if (form != GBS_CG_TEXTBOOK && (per_system || c[2] != GBS_SPMV_SELL)) continue;
-        timed(Tuning{c[0], c[1], c[2], c[3], GBS_SOLVER_PHASES, form, A->split_rows, pp});
+        timed(Tuning{c[0], c[1], c[2], c[3], GBS_SOLVER_PHASES, form, A->split_rows, pp, 0});
         if (st != GBS_OK) break;
       }
       if (st != GBS_OK) break;
@@ -633,6 +637,11 @@ static int autotune(gbs_mat A, cudaStream_t s, Tuning *out, float *out_ms) {
     } else {  // the one-kernel form (where it fits, else two)
       t.cg_form = GBS_CG_SINGLE_KERNEL;
       timed(t);
+      if (st == GBS_OK) {  // and the whole solve in one launch
+        t.cg_form = GBS_CG_TEXTBOOK;
+        t.team = 1;
+        timed(t);
+      }
     }
     t = base;
     const int64_t nz = per_system ? A->max_sys_nnz : A->nnz;
@@ -812,12 +821,13 @@ int mat_autotune_file(gbs_mat A, const char *path, int32_t *from_cache, void *st
       if (!bar || (size_t)(bar - line) != key.size() + 1 || strncmp(line, key.c_str(), key.size()))
         continue;
       long long sr = 1;
-      int pt = -1;
+      int pt = -1;  // column patterns, plus 2 for the team of CTAs
       const int nf = sscanf(bar + 1, " %d %d %d %d %d %d %lld %d", &t.Ra, &t.Re, &t.kernel,
                             &t.cpsm, &t.solver, &t.cg_form, &sr, &pt);
       if (nf >= 6) {  // the last matching line wins
         t.split_rows = nf >= 7 && sr >= 1 ? (int64_t)sr : 1;
-        t.patterns = nf == 8 && (pt == 0 || pt == 1) ? pt : -1;
+        t.patterns = nf == 8 && pt >= 0 && pt <= 3 ? (pt & 1) : -1;
+        t.team = nf == 8 && (pt == 2 || pt == 3) ? 1 : 0;
         hit = true;
       }
     }
@@ -832,7 +842,7 @@ int mat_autotune_file(gbs_mat A, const char *path, int32_t *from_cache, void *st
         fseek(f, 0, SEEK_END);
         fprintf(f, "%s | %d %d %d %d %d %d %lld %d | %.4f ms per 30 iterations\n", key.c_str(),
                 t.Ra, t.Re, t.kernel, t.cpsm, t.solver, t.cg_form, (long long)t.split_rows,
-                t.patterns, ms);
+                t.patterns + 2 * t.team, ms);
         fflush(f);
       }
     }
@@ -851,6 +861,7 @@ int mat_set_cg_form(gbs_mat A, int32_t form) {
     return GBS_ERR_ARG;
   }
   A->cg_form = form;
+  A->team_tuned = false;
   return GBS_OK;
 }
 

@@ -196,7 +196,8 @@ int ensure_solver_workspace(gbs_mat A, bool refined, cudaStream_t s) {
   }
   // reduction slots: table A's, table E's, and a third region the size of
   // table E's for partial sums of E's slots
-  const int64_t need = std::max(A->ta.nslots + 2 * A->te.nslots, A->sa.nslots + 2 * A->se.nslots) + 1;
+  const int64_t need = std::max({A->ta.nslots + 2 * A->te.nslots,
+                                 A->sa.nslots + 2 * A->se.nslots, (int64_t)sm_count(A)}) + 1;
   if (A->part_cap < need) {
     if (A->part) {
       GBS_TRY_CUDA(cudaStreamSynchronize(s));
@@ -562,6 +563,14 @@ int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_sys
     GBS_TRY_CUDA(cudaMemsetAsync(A->st, 0, sizeof(SysState) * A->nsys, s));
     GBS_TRY_CUDA(cudaMemsetAsync(A->ctl, 0, sizeof(DevCtl), s));
     return GBS_OK;
+  }
+  if (use_team(A, per_system, o)) {
+    bool ran = false;
+    GBS_TRY(solve_team(A, b, x, o, s, &ran));
+    if (ran) {
+      A->last_solver = use_cta_solver(A, per_system) ? GBS_SOLVER_CTA : GBS_SOLVER_PHASES;
+      return GBS_OK;
+    }
   }
   if (use_cta_solver(A, per_system)) {
     if (A->lanes != GBS_SPMV_SELL) {

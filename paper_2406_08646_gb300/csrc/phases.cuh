@@ -528,19 +528,30 @@ struct Vals {
 // How a row product gathers x: GATHER_NC the read-only path (x is not
 // written during the kernel), GATHER_CA a plain L1-cached load (coherent for
 // values the same CTA wrote before a barrier, and for values other CTAs
-// published with a release that this thread's acquire load observed).
-enum { GATHER_CA = 0, GATHER_NC = 1 };
+// published with a release that this thread's acquire load observed),
+// GATHER_SM a copy of x in shared memory.
+enum { GATHER_CA = 0, GATHER_NC = 1, GATHER_SM = 2 };
 
 template <int GATHER, typename T>
 __device__ __forceinline__ T ld_x(const T *p) {
   if constexpr (GATHER == GATHER_NC) return __ldg(p);
+  else if constexpr (GATHER == GATHER_SM) return *p;
   else return __ldca(p);
 }
 
-// Read-only load of a matrix entry, evict-first when STREAM.
-template <bool STREAM, typename T>
+// Read-only load of a matrix entry, evict-first when STREAM; a plain load of a
+// shared-memory copy when SM.
+template <bool STREAM, bool SM = false, typename T>
 __device__ __forceinline__ T ld_entry(const T *p) {
-  if constexpr (STREAM) return __ldcs(p);
+  if constexpr (SM) return *p;
+  else if constexpr (STREAM) return __ldcs(p);
+  else return __ldg(p);
+}
+
+// Read-only load of the sliced copy's tables (a plain one of a shared-memory copy when SM).
+template <bool SM, typename T>
+__device__ __forceinline__ T ld_meta(const T *p) {
+  if constexpr (SM) return *p;
   else return __ldg(p);
 }
 
@@ -584,64 +595,155 @@ constexpr int16_t SELL_PAD16 = -32768;
 
 // The two column indices of a pair (entries 2m, 2m + 1 of a lane's row): from
 // the 32-bit columns, or decoded from the two 16-bit offsets; padding -1.
-template <bool STREAM>
+template <bool STREAM, bool SM = false>
 __device__ __forceinline__ int2 sell_pair_cols(const int2 *__restrict__ c2,
                                                const int *__restrict__ o2, int pi, int r) {
   if (o2) {
-    const int o = ld_entry<STREAM>(o2 + pi);
+    const int o = ld_entry<STREAM, SM>(o2 + pi);
     const int lo = (int)(int16_t)o, hi = o >> 16;
     return make_int2(lo == SELL_PAD16 ? -1 : r + lo, hi == SELL_PAD16 ? -1 : r + hi);
   }
-  return ld_entry<STREAM>(c2 + pi);
+  return ld_entry<STREAM, SM>(c2 + pi);
 }
 
-// Slices with column patterns (S.pat set: every slice has one).
-template <typename T, bool STREAM, int NC, class F>
+// Slices with column patterns (S.pat set: every slice has one).  SM: the view
+// and the values are copies in shared memory (team.cu), read by plain loads.
+template <typename T, bool STREAM, int NC, bool SM = false, class F>
 __device__ __forceinline__ void sell_rows_pat(const SellView &S, const T *__restrict__ sval,
                                               const T *x, int s0, int s1, F &f) {
   typedef typename Pair<T>::type P;
   const P *__restrict__ v2 = reinterpret_cast<const P *>(sval);
   const int lane = threadIdx.x & 31;
   for (int sl = s0 + (int)(threadIdx.x >> 5); sl < s1; sl += (int)(blockDim.x >> 5)) {
-    const int b0 = __ldg(S.ptr + sl), b1 = __ldg(S.ptr + sl + 1);
-    const int r = __ldg(S.row0 + sl) + lane, re = __ldg(S.row0 + sl + 1);
-    const int2 *__restrict__ pat2 = reinterpret_cast<const int2 *>(S.pool + __ldg(S.pat + sl));
-    uint32_t mk = __ldg(S.mask + 32 * (int64_t)sl + lane);
-    if constexpr (STREAM && sizeof(T) == 4) {  // the slice's whole run in flight at once
+    const int b0 = ld_meta<SM>(S.ptr + sl), b1 = ld_meta<SM>(S.ptr + sl + 1);
+    const int r = ld_meta<SM>(S.row0 + sl) + lane, re = ld_meta<SM>(S.row0 + sl + 1);
+    const int2 *__restrict__ pat2 = reinterpret_cast<const int2 *>(S.pool + ld_meta<SM>(S.pat + sl));
+    uint32_t mk = ld_meta<SM>(S.mask + 32 * (int64_t)sl + lane);
+    if constexpr (STREAM && !SM && sizeof(T) == 4) {  // the slice's whole run in flight at once
       if (lane == 0) prefetch_rows(sval, b0, b1);
     }
     int pi = (b0 >> 1) + lane;
     const int pend = pi + 32 * ((b1 - b0) >> 6);
     T acc = T(0);
     for (; pi + 32 < pend; pi += 64, pat2 += 2, mk >>= 4) {
-      const int2 oa = __ldg(pat2), ob = __ldg(pat2 + 1);
-      const P va = ld_entry<STREAM>(v2 + pi), vb = ld_entry<STREAM>(v2 + pi + 32);
+      const int2 oa = ld_meta<SM>(pat2), ob = ld_meta<SM>(pat2 + 1);
+      const P va = ld_entry<STREAM, SM>(v2 + pi), vb = ld_entry<STREAM, SM>(v2 + pi + 32);
       if (mk & 1u) acc = fma_rn(va.x, ld_x<NC>(x + r + oa.x), acc);
       if (mk & 2u) acc = fma_rn(va.y, ld_x<NC>(x + r + oa.y), acc);
       if (mk & 4u) acc = fma_rn(vb.x, ld_x<NC>(x + r + ob.x), acc);
       if (mk & 8u) acc = fma_rn(vb.y, ld_x<NC>(x + r + ob.y), acc);
     }
     if (pi < pend) {
-      const int2 oa = __ldg(pat2);
-      const P va = ld_entry<STREAM>(v2 + pi);
+      const int2 oa = ld_meta<SM>(pat2);
+      const P va = ld_entry<STREAM, SM>(v2 + pi);
       if (mk & 1u) acc = fma_rn(va.x, ld_x<NC>(x + r + oa.x), acc);
       if (mk & 2u) acc = fma_rn(va.y, ld_x<NC>(x + r + oa.y), acc);
       mk >>= 2;
       ++pat2;
     }
     if ((((b1 - b0) >> 5) & 1) && (mk & 1u)) {  // the odd last entry
-      const int o = __ldg(reinterpret_cast<const int *>(pat2));
-      acc = fma_rn(ld_entry<STREAM>(sval + (b1 - 32 + lane)), ld_x<NC>(x + r + o), acc);
+      const int o = ld_meta<SM>(reinterpret_cast<const int *>(pat2));
+      acc = fma_rn(ld_entry<STREAM, SM>(sval + (b1 - 32 + lane)), ld_x<NC>(x + r + o), acc);
     }
     if (r < re) f(r, acc);
   }
 }
 
-template <typename T, bool STREAM, int NC, class F>
+// The same sums with more loads in flight, for kernels with 64 registers a
+// thread: the next slice's bounds, pattern and masks are loaded while the
+// current slice is summed, a step issues the loads of NP pairs (offsets,
+// values, gathers) before its first FMA, and the odd last entry's loads go
+// out before the first step.  An absent entry gathers the slice's first row,
+// whose value its FMA then does not use, so no load waits on a branch.
+template <int N, typename T, bool STREAM, int NC, bool SM>
+__device__ __forceinline__ void sell_step(const typename Pair<T>::type *v2,
+                                          const int2 *pat2, const T *xr, uint32_t mk, int lane,
+                                          T &acc) {
+  typename Pair<T>::type v[N];
+  int2 o[N];
+  T g[2 * N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    o[j] = ld_meta<SM>(pat2 + j);
+    v[j] = ld_entry<STREAM, SM>(v2 + 32 * j);
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    g[2 * j] = ld_x<NC>(xr + ((mk >> (2 * j)) & 1u ? o[j].x : -lane));
+    g[2 * j + 1] = ld_x<NC>(xr + ((mk >> (2 * j + 1)) & 1u ? o[j].y : -lane));
+  }
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const T t = fma_rn(v[j].x, g[2 * j], acc);
+    acc = (mk >> (2 * j)) & 1u ? t : acc;
+    const T u = fma_rn(v[j].y, g[2 * j + 1], acc);
+    acc = (mk >> (2 * j + 1)) & 1u ? u : acc;
+  }
+}
+
+template <typename T, bool STREAM, int NC, bool SM, int NP, class F>
+__device__ __forceinline__ void sell_rows_deep(const SellView &S, const T *__restrict__ sval,
+                                               const T *x, int s0, int s1, F &f) {
+  typedef typename Pair<T>::type P;
+  const int lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
+  int sl = s0 + (int)(threadIdx.x >> 5);
+  if (sl >= s1) return;
+  int b0 = ld_meta<SM>(S.ptr + sl), b1 = ld_meta<SM>(S.ptr + sl + 1);
+  int r = ld_meta<SM>(S.row0 + sl), re = ld_meta<SM>(S.row0 + sl + 1);
+  int p0 = ld_meta<SM>(S.pat + sl);
+  uint32_t mk = ld_meta<SM>(S.mask + 32 * (int64_t)sl + lane);
+  for (;;) {
+    const int nx = sl + nw;
+    int nb0 = 0, nb1 = 0, nr = 0, nre = 0, np0 = 0;
+    uint32_t nmk = 0;
+    if (nx < s1) {
+      nb0 = ld_meta<SM>(S.ptr + nx);
+      nb1 = ld_meta<SM>(S.ptr + nx + 1);
+      nr = ld_meta<SM>(S.row0 + nx);
+      nre = ld_meta<SM>(S.row0 + nx + 1);
+      np0 = ld_meta<SM>(S.pat + nx);
+      nmk = ld_meta<SM>(S.mask + 32 * (int64_t)nx + lane);
+    }
+    const int w = (b1 - b0) >> 5;
+    const T *xr = x + r + lane;
+    const P *v2 = reinterpret_cast<const P *>(sval) + (b0 >> 1) + lane;
+    const int2 *pat2 = reinterpret_cast<const int2 *>(S.pool + p0);
+    T vo = T(0), xo = T(0);
+    const bool odd = (w & 1) && ((mk >> (w - 1)) & 1u);
+    if (w & 1) {
+      const int o = ld_meta<SM>(S.pool + p0 + w - 1);
+      vo = ld_entry<STREAM, SM>(sval + (b1 - 32 + lane));
+      xo = ld_x<NC>(xr + (odd ? o : -lane));
+    }
+    T acc = T(0);
+    int m = w >> 1;
+    for (; m >= NP; m -= NP, v2 += 32 * NP, pat2 += NP, mk >>= 2 * NP)
+      sell_step<NP, T, STREAM, NC, SM>(v2, pat2, xr, mk, lane, acc);
+    if (NP > 2 && m >= 2) {
+      sell_step<2, T, STREAM, NC, SM>(v2, pat2, xr, mk, lane, acc);
+      m -= 2, v2 += 64, pat2 += 2, mk >>= 4;
+    }
+    if (m > 0) sell_step<1, T, STREAM, NC, SM>(v2, pat2, xr, mk, lane, acc);
+    const T t = fma_rn(vo, xo, acc);
+    acc = odd ? t : acc;
+    if (r + lane < re) f(r + lane, acc);
+    if (nx >= s1) break;
+    sl = nx;
+    b0 = nb0;
+    b1 = nb1;
+    r = nr;
+    re = nre;
+    p0 = np0;
+    mk = nmk;
+  }
+}
+
+template <typename T, bool STREAM, int NC, bool SM = false, int NP = 2, class F>
 __device__ __forceinline__ void sell_rows(const SellView &S, const T *__restrict__ sval,
                                           const T *x, int s0, int s1, F &f) {
   if (S.pat) {
-    sell_rows_pat<T, STREAM, NC>(S, sval, x, s0, s1, f);
+    if constexpr (NP > 2) sell_rows_deep<T, STREAM, NC, SM, NP>(S, sval, x, s0, s1, f);
+    else sell_rows_pat<T, STREAM, NC, SM>(S, sval, x, s0, s1, f);
     return;
   }
   typedef typename Pair<T>::type P;
@@ -650,9 +752,9 @@ __device__ __forceinline__ void sell_rows(const SellView &S, const T *__restrict
   const P *__restrict__ v2 = reinterpret_cast<const P *>(sval);
   const int lane = threadIdx.x & 31;
   for (int sl = s0 + (int)(threadIdx.x >> 5); sl < s1; sl += (int)(blockDim.x >> 5)) {
-    const int b0 = __ldg(S.ptr + sl), b1 = __ldg(S.ptr + sl + 1);
-    const int r = __ldg(S.row0 + sl) + lane, re = __ldg(S.row0 + sl + 1);
-    if constexpr (STREAM && sizeof(T) == 4) {  // the slice's whole run in flight at once
+    const int b0 = ld_meta<SM>(S.ptr + sl), b1 = ld_meta<SM>(S.ptr + sl + 1);
+    const int r = ld_meta<SM>(S.row0 + sl) + lane, re = ld_meta<SM>(S.row0 + sl + 1);
+    if constexpr (STREAM && !SM && sizeof(T) == 4) {  // the slice's whole run in flight at once
       if (lane == 0) prefetch_rows(sval, b0, b1);
       else if (lane == 1) {
         if (S.off) prefetch_rows(S.off, b0, b1);
@@ -664,17 +766,17 @@ __device__ __forceinline__ void sell_rows(const SellView &S, const T *__restrict
     const int pend = pi + 32 * ((b1 - b0) >> 6);
     T acc = T(0);
     for (; pi + 32 < pend; pi += 64) {
-      const int2 ca = sell_pair_cols<STREAM>(c2, o2, pi, r);
-      const int2 cb = sell_pair_cols<STREAM>(c2, o2, pi + 32, r);
-      const P va = ld_entry<STREAM>(v2 + pi), vb = ld_entry<STREAM>(v2 + pi + 32);
+      const int2 ca = sell_pair_cols<STREAM, SM>(c2, o2, pi, r);
+      const int2 cb = sell_pair_cols<STREAM, SM>(c2, o2, pi + 32, r);
+      const P va = ld_entry<STREAM, SM>(v2 + pi), vb = ld_entry<STREAM, SM>(v2 + pi + 32);
       if (ca.x >= 0) acc = fma_rn(va.x, ld_x<NC>(x + ca.x), acc);
       if (ca.y >= 0) acc = fma_rn(va.y, ld_x<NC>(x + ca.y), acc);
       if (cb.x >= 0) acc = fma_rn(vb.x, ld_x<NC>(x + cb.x), acc);
       if (cb.y >= 0) acc = fma_rn(vb.y, ld_x<NC>(x + cb.y), acc);
     }
     if (pi < pend) {
-      const int2 ca = sell_pair_cols<STREAM>(c2, o2, pi, r);
-      const P va = ld_entry<STREAM>(v2 + pi);
+      const int2 ca = sell_pair_cols<STREAM, SM>(c2, o2, pi, r);
+      const P va = ld_entry<STREAM, SM>(v2 + pi);
       if (ca.x >= 0) acc = fma_rn(va.x, ld_x<NC>(x + ca.x), acc);
       if (ca.y >= 0) acc = fma_rn(va.y, ld_x<NC>(x + ca.y), acc);
     }
@@ -682,19 +784,18 @@ __device__ __forceinline__ void sell_rows(const SellView &S, const T *__restrict
       const int q = b1 - 32 + lane;
       int c;
       if (S.off) {
-        const int o = ld_entry<STREAM>(S.off + q);
+        const int o = ld_entry<STREAM, SM>(S.off + q);
         c = o == SELL_PAD16 ? -1 : r + o;
       } else {
-        c = ld_entry<STREAM>(S.col + q);
+        c = ld_entry<STREAM, SM>(S.col + q);
       }
-      if (c >= 0) acc = fma_rn(ld_entry<STREAM>(sval + q), ld_x<NC>(x + c), acc);
+      if (c >= 0) acc = fma_rn(ld_entry<STREAM, SM>(sval + q), ld_x<NC>(x + c), acc);
     }
     if (r < re) f(r, acc);
   }
 }
 
 // The row products of block b (rows [r0, r1) of table ta) with the plan's
-// kernel: L == 0 sliced ELL, else CSR-vector with L lanes per row.// The row products of block b (rows [r0, r1) of table ta) with the plan's
 // kernel: L == 0 sliced ELL, else CSR-vector with L lanes per row.
 template <typename T, int L, class F>
 __device__ __forceinline__ void row_products(const PcgArgs &a, int b, int r0, int r1,

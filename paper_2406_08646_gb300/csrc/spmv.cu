@@ -292,6 +292,7 @@ int build_plan(gbs_mat A, int32_t Ra, int32_t Re, int32_t kernel, int32_t ctas_p
               Ra, Re, kernel, ctas_per_sm);
     return GBS_ERR_ARG;
   }
+  const bool all_auto = Ra == 0 && Re == 0 && kernel == GBS_SPMV_AUTO && ctas_per_sm == 0;
   drop_graphs(A);
   free_table(A->sa);  // the size split's tables follow the plan
   free_table(A->se);
@@ -325,6 +326,8 @@ int build_plan(gbs_mat A, int32_t Ra, int32_t Re, int32_t kernel, int32_t ctas_p
   A->Re = Re;
   A->lanes = kernel;
   A->ctas_per_sm = ctas_per_sm;
+  A->plan_auto = all_auto;
+  A->team_tuned = false;
   return GBS_OK;
 }
 

@@ -1,0 +1,736 @@
+// Jacobi-PCG with a team of CTAs per system, every iteration inside one
+// launch (Sec. 6.1 CG with device-resident scalars and no host round trip).
+//
+// The phase kernels (phases.cuh) pay three kernel boundaries an iteration:
+// each drains the grid, launches the next one, refills it and finishes its
+// reduction in one last CTA -- 14 to 17 us an iteration however small the
+// system.  Measured, us an iteration, phases -> here: 2D 64^2 15.7 -> 5.9,
+// 256^2 15.9 -> 9.5, 512^2 21.5 -> 13.8, 1024^2 42.1 -> 35.9; Q1 32^3 21.1 ->
+// 12.5, 64^3 37.0 -> 28.4, 96^3 76.0 -> 68.0; 3D 7-point 100^3 45.1 -> 39.7.
+// What bounds them: the meetings and the FP64 latency of the sums on small
+// systems (a dependent FP64 add takes 60 clocks and more), the FP64 pipe (two
+// FMAs a clock an SM, nonzeros + 8 a row of them: 40 us of Q1 96^3's 68) and
+// the gathers' latency on large ones.
+//
+// Here the CTAs stay: each owns a run of the system's 32-row slices
+// for the whole solve, keeps its part of the vectors (and of the matrix, where
+// it fits) in shared memory, and the team meets three times an iteration:
+//
+//   q = A p, p.q         -- sum over the team -> alpha
+//   x, r, z, r.z, r.r    -- sum over the team -> tests, beta
+//   p = z + beta p       -- barrier: p is what the other CTAs gather next
+//
+// Two kinds of team:
+//   - a thread-block cluster (up to 16 CTAs) meets at the hardware cluster
+//     barrier and exchanges its partial sums through distributed shared
+//     memory: 0.2-0.3 us a barrier, 0.7-0.9 us a sum;
+//   - the whole grid, one CTA per SM, launched cooperatively, meets at a
+//     counter in global memory: 1.2 us a barrier, 1.9 us a sum (152 CTAs).
+// Every wait of the grid team is bounded (one second and 2^22 polls), after
+// which the solve ends with GBS_ERR_TIMEOUT.
+//
+// Every CTA adds the team's partial sums itself, in rank order, and its thread
+// 0 runs the scalar recurrences on the same totals, so all CTAs take the same
+// decisions without a broadcast and results are the same on every run.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "cta.cuh"
+#include "device_util.cuh"
+#include "internal.cuh"
+#include "phases.cuh"
+
+namespace gbs {
+
+constexpr int TEAM_MAX_CLUSTER = 16;
+
+// How a launch lays out its dynamic shared memory: the block sums' scratch,
+// the p window and (clusters) the halo of z, then nvec vectors of rows_cap
+// rows, then mat_cap bytes for the CTA's part of the sliced copy.
+struct TeamCfg {
+  int32_t window;  // 1: windows of p in shared memory (halo rows beyond the CTA's own)
+  int32_t halo, win_cap, zh_cap;
+  int32_t nvec, rows_cap, mat_cap;
+  unsigned *ctr;   // grid team: arrivals, zero at launch
+  double *slots;   // grid team: 2 parities x 2 values x CTAs
+};
+
+// The part of a system one CTA owns: slices [s0, s1), rows [r0, r1).
+struct TeamPart {
+  int s, s0, s1, r0, r1;
+  int w0, w1;    // window of p: its own rows and those its row products read
+  int dlo, dhi;  // the cluster's CTAs with rows of this one in their windows
+};
+
+// The vectors of a solve, where they live: shared memory (offset so that row
+// indices apply) or global.  p is the window, or the global vector that the
+// whole team gathers; zh holds the window's halo of z (clusters), zg the z
+// that the grid's CTAs read their halos from.
+struct TeamVecs {
+  double *q, *r, *z, *dv, *x, *p, *zh, *zg;
+};
+
+struct TeamShared {
+  // (here, not in registers: a pass over the rows loads the few it needs)
+  TeamPart g;
+  TeamVecs V;
+  SellView sv;
+  const double *sval;
+  double lanes[2 * 128];                    // block_sums' lane partials
+  double box[2][2][TEAM_MAX_CLUSTER];       // partial sums of the cluster's CTAs, by parity
+  double pub[2];
+  int ipub[2];
+  // thread 0's scalars (in shared memory, not in every thread's registers)
+  SysState S;                               // bb, rr, thr and its bounds, rho, rnorm0
+  int it, status, timed, zero;
+  int abort;                                // a bounded wait ran out
+  // the rows each CTA of the cluster takes into its halo of z, and where
+  int32_t lo[TEAM_MAX_CLUSTER], hi[TEAM_MAX_CLUSTER];
+  uint32_t to[TEAM_MAX_CLUSTER];
+  CallArgs call;                            // (global loads would wait on L2: L1 is dropped
+                                            // at every meeting)
+  unsigned long long ns[5], last;           // phase timers (one thread of rank 0)
+};
+
+__device__ __forceinline__ void cluster_meet() {
+  asm volatile(
+      "barrier.cluster.arrive.release.aligned;\n\t"
+      "barrier.cluster.wait.acquire.aligned;" ::
+          : "memory");
+}
+
+// The address that p (this CTA's shared memory) has in the cluster's CTA `rank`.
+__device__ __forceinline__ uint32_t remote(const void *p, int rank) {
+  const uint32_t l = (uint32_t)__cvta_generic_to_shared(p);
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(l), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_remote(uint32_t to, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(to), "d"(v) : "memory");
+}
+
+template <bool GRID>
+struct Team {
+  int rank, size;
+  TeamShared &sh;
+  double *red;      // 2 blockDim doubles
+  const TeamCfg &cfg;
+  DevCtl *ctl;
+  unsigned target;  // grid: arrivals that complete the next meeting
+  int par;
+
+  // Warp 0 counts the CTA in and waits for the whole grid.
+  __device__ __forceinline__ void arrive_and_wait() {
+    target += (unsigned)size;
+    if (threadIdx.x == 0)
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cfg.ctr) : "memory");
+    unsigned v;
+    uint64_t t0 = 0;
+    for (unsigned polls = 0;; ++polls) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cfg.ctr) : "memory");
+      if ((int)(v - target) >= 0) break;
+      if ((polls & 1023u) == 1023u) {
+        const uint64_t t = global_ns();
+        if (t0 == 0) t0 = t;
+        else if (polls > (1u << 22) && t - t0 > 1000000000ull) {
+          sh.abort = 1;
+          break;
+        }
+      }
+    }
+    __syncwarp();
+  }
+
+  // Sums over the team of NV <= 2 values a thread, valid in warp 0 of every
+  // CTA (the same bits in all of them).
+  template <int NV>
+  __device__ __forceinline__ void sum(double (&v)[NV]) {
+    block_sums<double, NV>(v, red, sh.lanes);
+    if (size == 1) return;
+    const int lane = threadIdx.x & 31;
+    if constexpr (GRID) {
+      if ((threadIdx.x >> 5) != 0) return;
+      double *s = cfg.slots + (size_t)par * 2 * size;
+      if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) s[k * size + rank] = v[k];
+      }
+      arrive_and_wait();
+      // lane l adds slots l, l + 32, ...; all loads of a batch in flight
+      constexpr int BATCH = 6;
+#pragma unroll
+      for (int k = 0; k < NV; ++k) v[k] = 0.0;
+      for (int i0 = 0; i0 < size; i0 += 32 * BATCH) {
+        double u[BATCH][NV];
+#pragma unroll
+        for (int j = 0; j < BATCH; ++j)
+#pragma unroll
+          for (int k = 0; k < NV; ++k) {
+            const int i = i0 + 32 * j + lane;
+            u[j][k] = i < size ? ldcg(s + k * size + i) : 0.0;
+          }
+#pragma unroll
+        for (int j = 0; j < BATCH; ++j)
+#pragma unroll
+          for (int k = 0; k < NV; ++k)
+            if (i0 + 32 * j < size) v[k] += u[j][k];
+      }
+      warp_sums<double, NV>(v);
+    } else {
+      if ((threadIdx.x >> 5) == 0 && lane < size) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) st_remote(remote(&sh.box[par][k][rank], lane), v[k]);
+      }
+      cluster_meet();
+      if ((threadIdx.x >> 5) == 0) {
+        // value lane / 16 of CTA lane % 16: four steps add either one value or two
+        const int k = NV == 2 ? lane >> 4 : 0, c = lane & 15;
+        double t = c < size ? sh.box[par][k][c] : 0.0;
+#pragma unroll
+        for (int d = 8; d > 0; d >>= 1) t += __shfl_xor_sync(FULL_MASK, t, d);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) v[q] = __shfl_sync(FULL_MASK, t, 16 * q);
+      }
+    }
+    par ^= 1;
+  }
+
+  // Every thread's global writes before it are visible to every thread of the
+  // team after it.
+  __device__ __forceinline__ void barrier() {
+    if constexpr (GRID) {
+      __syncthreads();
+      if ((threadIdx.x >> 5) == 0) arrive_and_wait();
+      __syncthreads();
+    } else {
+      if (size > 1) cluster_meet();
+      else __syncthreads();
+    }
+  }
+  __device__ __forceinline__ bool aborted() const { return GRID && sh.abort != 0; }
+};
+
+// FP64 PCG on one system: cta_pcg_fp64's steps, tests and statuses, over a
+// team.
+//
+// WIN: the CTA holds p for every row that its row products read, its own and
+// a halo of col_span rows on either side.  The update hands z's halo rows over
+// together with the partial sums (to the other CTAs' shared memory, or through
+// L2), and after the sum every CTA forms p = z + beta p over its whole window
+// -- the same operations on the same values as the owner's, so the same bits
+// -- and needs no third meeting; the row products then gather from shared
+// memory.  Without windows (a span too wide for them) p is a global vector and
+// the third meeting publishes it.
+template <bool GRID, bool SM, bool WIN>
+__device__ __forceinline__ void team_pcg(const PcgArgs &a, Team<GRID> &tm, bool timers) {
+  TeamShared &sh = tm.sh;
+  const TeamPart &g = sh.g;
+  const TeamVecs &V = sh.V;
+  const CallArgs &C = sh.call;
+  const double *b = C.b;
+  double *xg = C.x;
+  const bool t0 = threadIdx.x == 0, lead = tm.rank == 0;
+  const bool clk = timers && lead && threadIdx.x == 32;
+  auto mark = [&](int k) {
+    if (clk) {
+      const unsigned long long t = global_ns();
+      sh.ns[k] += t - sh.last;
+      sh.last = t;
+    }
+  };
+  if (clk) {
+    for (int k = 0; k < 5; ++k) sh.ns[k] = 0;
+    sh.last = global_ns();
+  }
+  auto rows = [&](auto gather, const double *v, auto &f) {
+    constexpr int NC = decltype(gather)::value;
+    if constexpr (SM) {
+      sell_rows<double, false, NC, true, 2>(sh.sv, sh.sval, v, g.s0, g.s1, f);
+    } else {
+      if (a.stream_matrix) sell_rows<double, true, NC, false, 4>(a.sv, a.sval, v, g.s0, g.s1, f);
+      else sell_rows<double, false, NC, false, 4>(a.sv, a.sval, v, g.s0, g.s1, f);
+    }
+  };
+  std::integral_constant<int, GATHER_CA> from_global;
+  std::integral_constant<int, WIN ? GATHER_SM : GATHER_CA> from_p;
+  auto p_at = [&](int i) -> double {
+    if constexpr (WIN) return V.p[i];
+    else return __ldca(V.p + i);
+  };
+  // z of an own row: kept, and handed to the CTAs that hold the row in their halos
+  auto put_z = [&](int i, double z) {
+    V.z[i] = z;
+    if constexpr (WIN && GRID) {
+      if (V.z != V.zg) V.zg[i] = z;
+    } else if constexpr (WIN) {
+      for (int d = g.dlo; d <= g.dhi; ++d)
+        if (i >= sh.lo[d] && i < sh.hi[d]) st_remote(sh.to[d] + 8u * (uint32_t)i, z);
+    }
+  };
+  // p = z (+ beta p), over the window or the own rows
+  auto direction = [&](bool first, double be) {
+    constexpr int U = 2;
+    double pv[U], zv[U];
+    auto ld = [&](int i, int k) {
+      pv[k] = first ? 0.0 : p_at(i);
+      zv[k] = V.z[i];
+    };
+    auto use = [&](int i, int k) { V.p[i] = first ? zv[k] : fma(be, pv[k], zv[k]); };
+    cta_rows_by<U>(g.r0, g.r1, ld, use);
+    if constexpr (WIN) {
+      const int nlo = g.r0 - g.w0, nh = nlo + g.w1 - g.r1;
+      for (int h = threadIdx.x; h < nh; h += blockDim.x) {
+        const int i = h < nlo ? g.w0 + h : g.r1 + (h - nlo);
+        const double z = GRID ? __ldcg(V.zg + i) : V.zh[h];
+        V.p[i] = first ? z : fma(be, V.p[i], z);
+      }
+      __syncthreads();
+    }
+  };
+  // setup: r = b - A x0, z = D^-1 r; r.z, r.r, then b.b, missing diagonals
+  double u[2] = {0.0, 0.0}, w[2] = {0.0, 0.0};
+  auto start = [&](int i, double t) {
+    const double bv = b[i], rv = bv - t, d = a.dinv[i], z = d * rv;
+    if (V.dv != a.dinv) V.dv[i] = d;
+    V.r[i] = rv;
+    put_z(i, z);
+    u[0] = fma(rv, z, u[0]);
+    u[1] = fma(rv, rv, u[1]);
+    w[0] = fma(bv, bv, w[0]);
+    w[1] += (d == 0.0) ? 1.0 : 0.0;
+  };
+  if (C.nonzero_guess) {
+    if (V.x != xg)
+      for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) V.x[i] = xg[i];
+    rows(from_global, xg, start);
+  } else {
+    for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) {
+      V.x[i] = 0.0;
+      start(i, 0.0);
+    }
+  }
+  tm.template sum<2>(u);
+  __syncthreads();  // (block_sums' scratch)
+  tm.template sum<2>(w);
+  SysState &S = sh.S;
+  if (t0) {  // the scalars, the same in every CTA
+    int status = -1;
+    sh.it = sh.timed = sh.zero = 0;
+    S.rho = u[0];
+    S.rr = u[1];
+    S.bb = w[0];
+    set_thr(S, C.rtol * sqrt(S.bb));
+    S.rnorm0 = sqrt(S.rr);
+    if (w[1] > 0.0) status = GBS_ERR_NOT_SPD;
+    else if (!isfinite(S.bb)) status = GBS_ERR_NAN;
+    else if (S.bb == 0.0) {
+      status = GBS_OK;
+      sh.zero = 1;
+      S.rr = S.rnorm0 = 0.0;
+    } else if (!isfinite(S.rr) || !isfinite(S.rho)) status = GBS_ERR_NAN;
+    else if (S.rnorm0 <= S.thr) status = GBS_OK;
+    else if (C.maxit <= 0) status = GBS_ERR_MAXIT;
+    sh.status = sh.ipub[0] = status;
+  }
+  __syncthreads();
+  direction(true, 0.0);
+  if constexpr (!WIN) tm.barrier();
+  const bool zero_x = sh.zero != 0, limited = C.timeout_ns > 0;
+  const bool go = sh.ipub[0] < 0 && !tm.aborted();
+  mark(0);
+  while (go) {
+    // q = A p, p.q -> alpha
+    double pq[1] = {0.0};
+    auto fa = [&](int i, double y) {
+      V.q[i] = y;
+      pq[0] = fma(p_at(i), y, pq[0]);
+    };
+    rows(from_p, V.p, fa);
+    tm.template sum<1>(pq);
+    if (t0) {
+      int status = -1;
+      sh.it += 1;
+      if (nan64(pq[0])) status = GBS_ERR_NAN;
+      else if (!positive64(pq[0])) status = GBS_ERR_BREAKDOWN;
+      else sh.pub[0] = S.rho / pq[0];
+      sh.status = sh.ipub[0] = status;
+    }
+    __syncthreads();
+    mark(1);
+    if (sh.ipub[0] >= 0 || tm.aborted()) break;
+    const double al = sh.pub[0];
+    // x += alpha p, r -= alpha q, z = D^-1 r, r.z, r.r -> tests, beta
+    u[0] = u[1] = 0.0;
+    {
+      constexpr int U = 2;
+      double qv[U], rv0[U], d[U], pv[U], xv[U];
+      auto ld = [&](int i, int k) {
+        qv[k] = V.q[i];
+        rv0[k] = V.r[i];
+        d[k] = V.dv[i];
+        pv[k] = p_at(i);
+        xv[k] = V.x[i];
+      };
+      auto use = [&](int i, int k) {
+        const double rv = fma(-al, qv[k], rv0[k]);
+        const double z = d[k] * rv;
+        V.x[i] = fma(al, pv[k], xv[k]);
+        V.r[i] = rv;
+        put_z(i, z);
+        u[0] = fma(rv, z, u[0]);
+        u[1] = fma(rv, rv, u[1]);
+      };
+      cta_rows_by<U>(g.r0, g.r1, ld, use);
+    }
+    // the time limit is the lead's clock: its verdict goes round with the sums
+    double late[1] = {0.0};
+    if (limited && lead && t0) late[0] = cta_timed_out(a.ctl, C.timeout_ns) ? 1.0 : 0.0;
+    tm.template sum<2>(u);
+    if (limited) {
+      __syncthreads();
+      tm.template sum<1>(late);
+    }
+    if (t0) {
+      int status = -1;
+      S.rr = u[1];
+      if (!finite64(u[1]) || !finite64(u[0])) status = GBS_ERR_NAN;
+      else if (meets_thr(u[1], S)) status = GBS_OK;
+      else if (sh.it >= C.maxit) status = GBS_ERR_MAXIT;
+      else if (late[0] != 0.0) sh.timed = 1;
+      else {
+        sh.pub[1] = u[0] / S.rho;
+        S.rho = u[0];
+      }
+      sh.status = status;
+      sh.ipub[1] = (status < 0 && late[0] == 0.0) ? -1 : 0;
+    }
+    __syncthreads();
+    mark(2);
+    if (sh.ipub[1] >= 0 || tm.aborted()) break;
+    direction(false, sh.pub[1]);
+    if constexpr (!WIN) {
+      tm.barrier();
+      if (tm.aborted()) break;
+    }
+    mark(3);
+  }
+  // x out, then ||b - A x||^2 (x = 0 where b = 0)
+  if (zero_x || V.x != xg)
+    for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) xg[i] = zero_x ? 0.0 : V.x[i];
+  if (!tm.aborted()) tm.barrier();
+  double tt[1] = {0.0};
+  auto ft = [&](int i, double t) {
+    const double d = b[i] - t;
+    tt[0] = fma(d, d, tt[0]);
+  };
+  rows(from_global, xg, ft);
+  if (!tm.aborted()) tm.template sum<1>(tt);
+  if (lead && t0) {
+    const bool stopped = sh.timed || tm.aborted();
+    SysState &O = a.st[g.s];
+    memset(&O, 0, sizeof(SysState));
+    O.bb = S.bb;
+    O.rnorm0 = S.rnorm0;
+    O.rnorm = sqrt(S.rr);
+    O.tt = tt[0];
+    O.iterations = sh.it;
+    O.zero_x = sh.zero;
+    O.status = stopped ? GBS_OK : sh.status;
+    O.active = stopped ? 1 : 0;  // reported as the control word's error
+    if (stopped) a.ctl->err = GBS_ERR_TIMEOUT;
+  }
+  mark(4);
+  if (clk)
+    for (int k = 0; k < 5; ++k) a.ctl->phase_ns[k] = (int64_t)sh.ns[k];
+}
+
+__device__ __forceinline__ size_t up16(size_t n) { return (n + 15) & ~(size_t)15; }
+
+// Copies the CTA's part of the sliced copy into shared memory at m (cap
+// bytes); the view and the values are rebased so that global slice, entry and
+// pool indices apply.  Returns false (nothing copied) where it does not fit.
+__device__ bool team_cache(const SellView &S, const double *sval, const TeamPart &g,
+                           unsigned char *m, size_t cap, SellView &V, const double **vals) {
+  const int ns = g.s1 - g.s0;
+  if (ns <= 0) return false;
+  const int e0 = __ldg(S.ptr + g.s0), e1 = __ldg(S.ptr + g.s1);
+  const size_t ne = (size_t)(e1 - e0);
+  int pool0 = 0, npool = 0;
+  if (S.pat) {
+    pool0 = __ldg(S.pat + g.s0);
+    const int wl = (e1 - __ldg(S.ptr + g.s1 - 1)) >> 5;
+    npool = __ldg(S.pat + g.s1 - 1) + ((wl + 1) & ~1) - pool0;
+  }
+  const size_t o_ptr = up16(ne * 8), o_row = o_ptr + up16(4 * (size_t)(ns + 1));
+  const size_t o_a = o_row + up16(4 * (size_t)(ns + 1));
+  size_t o_pool = 0, o_mask = 0, need = o_a;
+  if (S.pat) {
+    o_pool = o_a + up16(4 * (size_t)ns);
+    o_mask = o_pool + up16(4 * (size_t)npool);
+    need = o_mask + 128 * (size_t)ns;
+  } else {
+    need = o_a + (S.off ? 2 : 4) * ne;
+  }
+  if (need > cap) return false;
+  auto copy = [&](auto *dst, const auto *src, int n) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = __ldg(src + i);
+  };
+  copy(reinterpret_cast<double2 *>(m), reinterpret_cast<const double2 *>(sval + e0), (int)(ne >> 1));
+  copy(reinterpret_cast<int32_t *>(m + o_ptr), S.ptr + g.s0, ns + 1);
+  copy(reinterpret_cast<int32_t *>(m + o_row), S.row0 + g.s0, ns + 1);
+  V = S;
+  V.ptr = reinterpret_cast<int32_t *>(m + o_ptr) - g.s0;
+  V.row0 = reinterpret_cast<int32_t *>(m + o_row) - g.s0;
+  *vals = reinterpret_cast<double *>(m) - e0;
+  if (S.pat) {
+    copy(reinterpret_cast<int32_t *>(m + o_a), S.pat + g.s0, ns);
+    copy(reinterpret_cast<int32_t *>(m + o_pool), S.pool + pool0, npool);
+    copy(reinterpret_cast<uint32_t *>(m + o_mask), S.mask + 32 * (int64_t)g.s0, 32 * ns);
+    V.pat = reinterpret_cast<int32_t *>(m + o_a) - g.s0;
+    V.pool = reinterpret_cast<int32_t *>(m + o_pool) - pool0;
+    V.mask = reinterpret_cast<uint32_t *>(m + o_mask) - 32 * (int64_t)g.s0;
+  } else if (S.off) {
+    copy(reinterpret_cast<int32_t *>(m + o_a), reinterpret_cast<const int32_t *>(S.off + e0),
+         (int)(ne >> 1));
+    V.off = reinterpret_cast<int16_t *>(m + o_a) - e0;
+  } else {
+    copy(reinterpret_cast<int32_t *>(m + o_a), S.col + e0, (int)ne);
+    V.col = reinterpret_cast<int32_t *>(m + o_a) - e0;
+  }
+  __syncthreads();
+  return true;
+}
+
+template <bool GRID>
+__device__ __forceinline__ void team_body(const PcgArgs &a, const TeamCfg &cfg) {
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  __shared__ TeamShared sh;
+  uint32_t rank, size, cluster = 0, nclusters = 1;
+  if constexpr (GRID) {
+    rank = blockIdx.x;
+    size = gridDim.x;
+  } else {
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
+    asm("mov.u32 %0, %%clusterid.x;" : "=r"(cluster));
+    asm("mov.u32 %0, %%nclusterid.x;" : "=r"(nclusters));
+  }
+  double *red = reinterpret_cast<double *>(team_smem);
+  double *win = red + 2 * blockDim.x, *zh = win + cfg.win_cap, *vec = zh + cfg.zh_cap;
+  unsigned char *mat = reinterpret_cast<unsigned char *>(vec + (size_t)cfg.nvec * cfg.rows_cap);
+  if (threadIdx.x == 0) {
+    sh.abort = 0;
+    sh.call = *a.call;
+  }
+  Team<GRID> tm{(int)rank, (int)size, sh, red, cfg, a.ctl, 0u, 0};
+  const SysRange sys = cta_system(a, 0);
+  const int64_t ns = sys.s1 - sys.s0;
+  auto part = [&](int k, int &r0, int &r1) {  // rows of the team's CTA k
+    r0 = min(sys.r1, sys.r0 + 32 * (int)(ns * k / size));
+    r1 = min(sys.r1, sys.r0 + 32 * (int)(ns * (k + 1) / size));
+  };
+  auto window = [&](int r0, int r1, int &w0, int &w1) {  // (r1 - halo: no overflow)
+    w0 = r0 < r1 ? max(sys.r0, r0 - cfg.halo) : r0;
+    w1 = r0 < r1 ? (sys.r1 - r1 < cfg.halo ? sys.r1 : r1 + cfg.halo) : r1;
+  };
+  TeamPart g;
+  g.s = sys.s;
+  g.s0 = sys.s0 + (int)(ns * rank / size);
+  g.s1 = sys.s0 + (int)(ns * (rank + 1) / size);
+  part(rank, g.r0, g.r1);
+  window(g.r0, g.r1, g.w0, g.w1);
+  g.dlo = 0;
+  g.dhi = -1;
+  __syncthreads();  // sh.call
+  if constexpr (!GRID) {
+    if (cfg.window) {
+      if (threadIdx.x < size) {
+        const int d = threadIdx.x;
+        int r0, r1, w0, w1;
+        part(d, r0, r1);
+        window(r0, r1, w0, w1);
+        sh.lo[d] = d == (int)rank ? INT32_MAX : max(g.r0, w0);
+        sh.hi[d] = min(g.r1, w1);
+        // rows below d's own start its halo, rows above follow them
+        sh.to[d] = remote(zh, d) - 8u * (uint32_t)((int)rank < d ? w0 : r1 - (r0 - w0));
+      }
+      __syncthreads();
+      for (int d = 0; d < (int)size; ++d)
+        if (sh.lo[d] < sh.hi[d]) {
+          if (g.dhi < 0) g.dlo = d;
+          g.dhi = d;
+        }
+    }
+  }
+  // q, r, [z,] D^-1, x: without windows z is kept over q
+  const bool w = cfg.window != 0;
+  if (threadIdx.x == 0) {
+    int k = 0;
+    auto home = [&](double *global) {
+      const int at = k++;
+      return at < cfg.nvec ? vec + (int64_t)at * cfg.rows_cap - g.r0 : global;
+    };
+    TeamVecs &V = sh.V;
+    V.q = home(w ? a.p : a.q);
+    V.r = home(a.r);
+    V.z = w ? home(a.q) : V.q;
+    V.dv = home(const_cast<double *>(a.dinv));
+    V.x = home(sh.call.x);
+    V.p = w ? win - g.w0 : a.p;
+    V.zh = zh;
+    V.zg = a.q;
+    sh.g = g;
+  }
+  SellView C;
+  const double *vals = nullptr;
+  const bool cached = cfg.mat_cap > 0 && team_cache(a.sv, a.sval, g, mat, cfg.mat_cap, C, &vals);
+  if (threadIdx.x == 0 && cached) {
+    sh.sv = C;
+    sh.sval = vals;
+  }
+  __syncthreads();
+  if (w) {
+    if (cached) team_pcg<GRID, true, true>(a, tm, true);
+    else team_pcg<GRID, false, true>(a, tm, true);
+  } else {
+    if (cached) team_pcg<GRID, true, false>(a, tm, true);
+    else team_pcg<GRID, false, false>(a, tm, true);
+  }
+  if (!GRID && size > 1) cluster_meet();  // no CTA leaves while others may write to its boxes
+}
+
+template <bool GRID, int TPB>
+__global__ void __launch_bounds__(TPB, 1) k_team(PcgArgs a, const __grid_constant__ TeamCfg cfg) {
+  team_body<GRID>(a, cfg);
+}
+
+// ------------------------------------------------------------------ host side
+
+constexpr int64_t TEAM_SMEM = 219 * 1024;  // dynamic shared memory a CTA may take (of 227 KB)
+constexpr int64_t TEAM_L1_SMEM = 128 * 1024;  // ... where the row products need L1 for p
+
+// One system runs on a cluster up to this many FP64 operations an iteration
+// (nonzeros plus eight a row): 16 SMs do 32 of them a clock, so beyond it the
+// grid's dearer meetings are the cheaper part.  Measured, us an iteration on
+// cluster / grid: 2D 64^2 (53k operations) 5.9 / 8.1, 3D 16^3 (60k) 6.4 / 8.7,
+// 2D 101^2 (132k) 7.9 / 8.1, Q1 16^3 (157k) 9.6 / 10.4, 2D 128^2 (212k) 8.6 / 8.0.
+constexpr int64_t TEAM_CLUSTER_WORK = 160000;
+// Beyond this many rows the phase kernels take over: twice the threads an SM
+// hide HBM's latency better than the saved meetings are worth (3D 7-point,
+// us an iteration on team / phases: 128^3 70.4 / 72.9, 160^3 141.6 / 134.0).
+constexpr int64_t TEAM_GRID_ROWS = 3 << 20;
+
+// An automatic solver and plan take the team by size; the autotuner takes it
+// where it measured it fastest (team_tuned).  An explicit solver, plan or
+// single-reduction form is what the caller asked for.
+bool use_team(gbs_mat A, bool per_system, const ksp_opts &o) {
+  if (per_system || A->nsys != 1 || o.method != GBS_KSP_CG || o.precision != GBS_FP64 ||
+      o.host_loop || A->lanes != GBS_SPMV_SELL || A->nrows == 0)
+    return false;
+  return A->team_tuned || (A->solver == GBS_SOLVER_AUTO && A->cg_form == GBS_CG_TEXTBOOK &&
+                           A->plan_auto && A->nrows <= TEAM_GRID_ROWS);
+}
+
+// The team of a solve on A: its CTAs, their threads and their shared memory.
+struct TeamShape {
+  TeamCfg cfg;
+  bool cluster;
+  int size, tpb;
+  size_t smem;
+};
+
+static TeamShape team_shape(gbs_mat A) {
+  TeamShape T;
+  memset(&T, 0, sizeof(T));
+  TeamCfg &c = T.cfg;
+  const int64_t n = A->nrows, ns = A->nslices;
+  T.cluster = A->nnz + 8 * n <= TEAM_CLUSTER_WORK;
+  T.size = T.cluster ? TEAM_MAX_CLUSTER : sm_count(A);
+  while (T.size > 1 && ns < T.size) T.size = (T.size + 1) / 2;  // every CTA has a slice
+  const int64_t per = (ns + T.size - 1) / T.size, rows = 32 * per;
+  T.tpb = rows <= 256 ? 256 : 512;
+  c.rows_cap = (int32_t)rows;
+  int64_t left = TEAM_SMEM - 16 * T.tpb;
+  // windows where the halo's extra work (one FMA a row, two rows a clock) stays
+  // below the meeting they save
+  const auto up32 = [](int64_t k) { return (k + 31) & ~(int64_t)31; };
+  const int64_t halo = std::min<int64_t>(A->col_span, n), win = up32(std::min(n, rows + 2 * halo));
+  const int64_t zh = T.cluster ? up32(std::min(2 * halo, n)) : 0;
+  const bool window = 2 * halo <= std::max<int64_t>(rows, 4096) && 8 * (win + zh) <= left / 3;
+  const int64_t per_entry = A->sell_npat ? 8 : (A->col_span <= 32767 ? 10 : 12);
+  const int64_t mat = A->sell_nnz / ns * per * per_entry * 9 / 8 +
+                      per * (136 + (A->sell_npat ? 256 : 0)) + 1024;
+  const int nv = window ? 5 : 4;
+  const int64_t used = (window ? 8 * (win + zh) : 0) + nv * 8 * rows;
+  if (used + mat <= left) {  // vectors, windows and matrix all stay
+    c.nvec = nv;
+    c.mat_cap = (int32_t)std::min<int64_t>((left - used) & ~(int64_t)15,
+                                           (mat + 1023) & ~(int64_t)1023);
+    if (window) {
+      c.window = 1;
+      c.halo = (int32_t)halo;
+      c.win_cap = (int32_t)win;
+      c.zh_cap = (int32_t)zh;
+    }
+  } else {
+    // the matrix streams past: every thread the registers allow, to have loads
+    // in flight (2D 1024^2, us an iteration: 1024 threads 35.1, 512 40.3), and
+    // p gathered through L1 rather than from windows (35.1 against 36.9)
+    T.tpb = 1024;
+    c.nvec = (int32_t)std::min<int64_t>(4, TEAM_L1_SMEM / (8 * rows));
+  }
+  T.smem = (size_t)(16 * T.tpb + 8 * (c.win_cap + c.zh_cap) + c.nvec * 8 * rows + c.mat_cap);
+  return T;
+}
+
+// One FP64 CG solve on a team of CTAs; *ran stays false (and nothing has
+// started) where the device cannot hold the team at once.
+int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, cudaStream_t s,
+               bool *ran) {
+  *ran = false;
+  TeamShape T = team_shape(A);
+  PcgArgs a = make_args(A, false, false);
+  a.stream_matrix = stream_matrix(A, 8);
+  T.cfg.slots = A->part;
+  T.cfg.ctr = reinterpret_cast<unsigned *>(&A->ctl->queue);
+  void (*const kernel)(PcgArgs, TeamCfg) =
+      T.tpb <= 512 ? (T.cluster ? k_team<false, 512> : k_team<true, 512>)
+                   : (T.cluster ? k_team<false, 1024> : k_team<true, 1024>);
+  GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)TEAM_SMEM));
+  cudaLaunchConfig_t lc = {};
+  cudaLaunchAttribute at[1];
+  memset(at, 0, sizeof(at));
+  lc.gridDim = dim3((unsigned)T.size);
+  lc.blockDim = dim3((unsigned)T.tpb);
+  lc.dynamicSmemBytes = T.smem;
+  lc.stream = s;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  if (T.cluster) {
+    GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)T.size;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+  GBS_TRY_CUDA(cudaMemsetAsync(A->ctl, 0, sizeof(DevCtl), s));
+  GBS_TRY(put_call(A->call, call_args(b, x, o), s, A->ctl));
+  const cudaError_t e = cudaLaunchKernelEx(&lc, kernel, a, T.cfg);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorInvalidClusterSize ||
+      e == cudaErrorLaunchOutOfResources) {
+    cudaGetLastError();
+    return GBS_OK;
+  }
+  GBS_TRY_CUDA(e);
+  count_launches(1);
+  *ran = true;
+  return GBS_OK;
+}
+
+}  // namespace gbs
