@@ -921,6 +921,10 @@ int vec_create_coo(int64_t n, int64_t ncoo, const int32_t *i, void *stream, gbs_
       A->nsys = 1;
       A->row_off_h = {0, n};
       st = symbolic(A, i, zeros, nullptr, s);
+      if (st == GBS_OK && cudaStreamSynchronize(s) != cudaSuccess) {
+        set_error("vec_create_coo: synchronising the stream failed");
+        st = GBS_ERR_CUDA;
+      }
       if (st == GBS_OK) V->A = A;
       else free_handle(A);
     }

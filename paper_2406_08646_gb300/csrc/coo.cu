@@ -3,6 +3,8 @@
 // refined solve (Sec. 2, A7) and the adjoint scatter over the pattern.
 //
 // Symbolic stage, all on the GPU:
+//   (patterns with a row of more than 4096 entries; the others: the row-bucketed
+//   stage below)
 //   1. keep flags (negative index -> ignored; out of range -> error) and an
 //      exclusive scan, compaction into 64-bit keys i*ncols + j with the
 //      original COO index as payload;
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_down(const uint32_t *in, int64_
 // sums are scanned by one CTA when they fit one tile, else recursively.
 // tmp: scan_tmp_words(n) words.  Grand total written to *total (device) when
 // non-null.
-static int exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp,
+int exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp,
                           uint32_t *total, cudaStream_t s) {
   const int64_t ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
   if (ntiles == 0) {
@@ -148,7 +150,7 @@ static int exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t
   return GBS_OK;
 }
 
-static int64_t scan_tmp_words(int64_t n) {
+int64_t scan_tmp_words(int64_t n) {
   int64_t w = 1, t = (n + SCAN_TILE - 1) / SCAN_TILE;
   for (;;) {
     w += t + 1;
@@ -169,9 +171,8 @@ struct KeepArgs {
   int32_t nsys;
 };
 
-__device__ __forceinline__ bool keep_entry(const KeepArgs &a, int64_t k, int64_t &gi,
-                                           int64_t &gj, bool &bad) {
-  const int32_t li = a.i[k], lj = a.j[k];
+__device__ __forceinline__ bool keep_entry(const KeepArgs &a, int64_t k, int32_t li, int32_t lj,
+                                           int64_t &gi, int64_t &gj, bool &bad) {
   bad = false;
   if (li < 0 || lj < 0) return false;
   if (a.coo_off) {
@@ -196,6 +197,11 @@ __device__ __forceinline__ bool keep_entry(const KeepArgs &a, int64_t k, int64_t
     gj = lj;
   }
   return true;
+}
+
+__device__ __forceinline__ bool keep_entry(const KeepArgs &a, int64_t k, int64_t &gi,
+                                           int64_t &gj, bool &bad) {
+  return keep_entry(a, k, a.i[k], a.j[k], gi, gj, bad);
 }
 
 __global__ void k_keep_flags(KeepArgs a, uint32_t *flags, int32_t *err) {
@@ -347,6 +353,29 @@ __global__ void __launch_bounds__(RS_T) k_radix_scatter(const uint64_t *keys_in,
   }
 }
 
+// The CTA's largest value to *out: one atomic a CTA, and none where it would
+// not raise the maximum (an atomic per warp on one address, a million of them,
+// took 0.6 ms).
+__device__ __forceinline__ void block_atomic_max(int32_t m, int32_t *out) {
+  __shared__ int32_t wm[32];
+  m = (int32_t)__reduce_max_sync(FULL_MASK, (unsigned)m);
+  if ((threadIdx.x & 31) == 0) wm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max(m, wm[w]);
+    if (m > *(volatile int32_t *)out) atomicMax(out, m);
+  }
+}
+
+// The longest row.
+__global__ void k_max_row(const int32_t *row_ptr, int64_t nrows, int32_t *out) {
+  int32_t m = 0;
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nrows;
+       r += (int64_t)gridDim.x * blockDim.x)
+    m = max(m, row_ptr[r + 1] - row_ptr[r]);
+  block_atomic_max(m, out);
+}
+
 // ------------------------------------------------------------------ segments
 
 __global__ void k_seg_flags(const uint64_t *keys, int64_t n, uint32_t *flags) {
@@ -382,8 +411,7 @@ __global__ void k_csr_cols(const uint64_t *ukey, int64_t nnz, int64_t ncols, int
     const int64_t d = c - r, ad = d < 0 ? -d : d;
     m = max(m, (int32_t)(ad > (1 << 30) ? (1 << 30) : ad));
   }
-  m = (int32_t)__reduce_max_sync(FULL_MASK, (unsigned)m);
-  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(span, m);
+  block_atomic_max(m, span);
 }
 
 // row_ptr[r] = first unique key >= r * ncols, for r in [0, nrows].
@@ -401,22 +429,16 @@ __global__ void k_row_ptr(const uint64_t *ukey, int64_t nnz, int64_t ncols, int6
   }
 }
 
-__global__ void k_max_row(const int32_t *row_ptr, int64_t nrows, int32_t *out) {
-  int32_t m = 0;
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nrows;
-       r += (int64_t)gridDim.x * blockDim.x)
-    m = max(m, row_ptr[r + 1] - row_ptr[r]);
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(FULL_MASK, m, off));
-  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
-}
-
 static unsigned grid_for(int64_t n, int tpb) {
   int64_t g = (n + tpb - 1) / tpb;
   if (g < 1) g = 1;
   if (g > 1048576) g = 1048576;
   return (unsigned)g;
 }
+
+// A grid that keeps every SM busy and no more: for kernels that end in one
+// atomic a CTA, or loop anyway.
+static unsigned wave_for(int64_t n, int tpb) { return std::min(grid_for(n, tpb), 8u * 160u); }
 
 // Error exits of the symbolic stages: set status and jump to cleanup.
 #define SYM_CUDA(call)                                                            \
@@ -438,141 +460,284 @@ static unsigned grid_for(int64_t n, int tpb) {
 //
 // The symbolic stage for patterns whose rows hold at most ROW_SORT_CTA COO
 // entries (finite-element, stencil and graph matrices): no global sort.
-//   1. per-row counts of the kept entries (warp-aggregated atomics: one
-//      atomic per distinct row in a warp);
+//   1. per-row counts of the kept entries (one atomic per run of equal rows on
+//      a warp's lanes); the old count plus the lane's place in its run is the
+//      entry's slot in its row, kept as 16 bits;
 //   2. their exclusive scan -> each row's range of the kept entries;
-//   3. every kept entry placed in its row's range as the 64-bit key
-//      (j << 32) | k (the order inside a row depends on atomic timing);
-//   4. each row sorted by that key (a warp's register bitonic sort up to
-//      ROW_SORT_WARP entries, a CTA's shared-memory one up to ROW_SORT_CTA):
-//      the keys are distinct, so the result is the same on every run, and it
+//   3. every kept entry placed at its slot of its row's range as the 64-bit key
+//      (j << 32) | k (the slots depend on the atomics' timing);
+//   4. each row sorted by that key (register bitonic networks, four rows a
+//      warp, up to ROW_SORT_WARP entries; a CTA's shared-memory one up to
+//      ROW_SORT_CTA): the keys are distinct, so the result is the same on every run, and it
 //      is the order of the radix path -- rows ascending, columns ascending,
-//      equal (i, j) by increasing COO index; the low halves are perm, and
-//      each row's distinct columns are counted;
-//   5. the scan of those counts is row_ptr (and nnz), and one pass writes
-//      col, jmap and the diagonal positions.
-// Traffic: about 56 bytes per kept entry, against about 140 for the 5-pass
+//      equal (i, j) by increasing COO index; written out as perm and the
+//      column with a head bit (first entry of its column), with each row's
+//      count of distinct columns and the place of its diagonal among them;
+//   5. the scan of those counts is row_ptr (and nnz); a pass over the sorted
+//      entries writes col and jmap, one over the rows the diagonal positions.
+// Traffic: about 40 bytes per kept entry, against about 140 for the 5-pass
 // radix sort of 40-bit keys.  A longer row sends the pattern to the radix
-// path.
+// path.  Measured on the Q1 96^3 pattern (56.6M entries, 62 a row) and the
+// 2D 1024^2 edges (8.4M, 8 a row), us, against one warp to a row, an atomic a
+// warp for the largest |col - row| and match-aggregated atomics with one entry
+// a thread in flight:
+//   counts 240 / 79 -> 139 / 24, placement 314 / 80 -> 169 / 30, sorts 589 /
+//   669 -> 410 / 80, emission 628 / 675 -> 144 / 28.
+// The long rows' sort is held by the ALU (64-bit compares), the short rows' by
+// the latency of its loads, the others by HBM and the stores' scatter.
 constexpr int ROW_SORT_WARP = 64, ROW_SORT_CTA = 4096, ROW_SORT_TPB = 512;
 
-// The lanes in `active` that share `key` add their count to cnt[key] with one
-// atomic; returns the old value, and in rank each lane's position among them.
-__device__ __forceinline__ uint32_t warp_agg_add(uint32_t *cnt, uint32_t key, unsigned active,
-                                                 uint32_t &rank) {
-  const int lane = threadIdx.x & 31;
-  const unsigned peers = __match_any_sync(active, key);
-  const int leader = __ffs(peers) - 1;
-  uint32_t base = 0;
-  if (lane == leader) base = atomicAdd(cnt + key, (uint32_t)__popc(peers));
-  base = __shfl_sync(peers, base, leader);
-  rank = (uint32_t)__popc(peers & ((1u << lane) - 1u));
-  return base;
-}
-
-// mode 0: count the kept entries per row (and flag out-of-range indices);
-// mode 1: place each at rstart[row] + its slot as (j << 32) | k.
-template <int MODE>
-__global__ void k_row_bucket(KeepArgs a, uint32_t *cnt, const uint32_t *__restrict__ rstart,
-                             uint64_t *keys, int32_t *err) {
+// Counts the kept entries per row (and flags out-of-range indices); slot[k]
+// is entry k's place in its row (rows of up to ROW_SORT_CTA entries need 13
+// bits; a longer row leaves the pattern to the radix path).
+// A warp takes 32 BUCKET_U consecutive entries at a time, all their loads in
+// flight before the first use (one entry a thread kept 8 bytes a thread in
+// flight: 1.6 TB/s).
+constexpr int BUCKET_U = 4;
+__global__ void k_row_count(KeepArgs a, uint32_t *cnt, uint16_t *__restrict__ slot, int32_t *err) {
   const int lane = threadIdx.x & 31;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < a.ncoo;
-       base += nw * 32) {
-    const int64_t k = base + lane;
-    int64_t gi = 0, gj = 0;
-    bool bad = false;
-    const bool keep = k < a.ncoo && keep_entry(a, k, gi, gj, bad);
-    if (MODE == 0 && bad) atomicExch(err, GBS_ERR_INDEX);
-    const unsigned active = __ballot_sync(FULL_MASK, keep);
-    if (keep) {
-      uint32_t rank;
-      const uint32_t b = warp_agg_add(cnt, (uint32_t)gi, active, rank);
-      if (MODE == 1)
-        keys[rstart[gi] + b + rank] = ((uint64_t)(uint32_t)gj << 32) | (uint32_t)k;
+  for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32 * BUCKET_U;
+       base < a.ncoo; base += nw * 32 * BUCKET_U) {
+    int32_t li[BUCKET_U], lj[BUCKET_U];
+    uint32_t old[BUCKET_U];
+    int first[BUCKET_U];
+#pragma unroll
+    for (int u = 0; u < BUCKET_U; ++u) {
+      const int64_t k = base + 32 * u + lane;
+      li[u] = k < a.ncoo ? __ldg(a.i + k) : -1;
+      lj[u] = k < a.ncoo ? __ldg(a.j + k) : -1;
+    }
+#pragma unroll
+    for (int u = 0; u < BUCKET_U; ++u) {
+      int64_t gi = 0, gj = 0;
+      bool bad = false;
+      const bool keep = keep_entry(a, base + 32 * u + lane, li[u], lj[u], gi, gj, bad);
+      if (bad) atomicExch(err, GBS_ERR_INDEX);
+      const int32_t row = keep ? (int32_t)gi : -1;
+      const int32_t before = __shfl_up_sync(FULL_MASK, row, 1);
+      const bool head = keep && (lane == 0 || before != row);
+      const unsigned heads = __ballot_sync(FULL_MASK, head), kept = __ballot_sync(FULL_MASK, keep);
+      // the head of my run: the last one up to my lane
+      first[u] = keep ? 31 - __clz(heads & (0xffffffffu >> (31 - lane))) : lane;
+      old[u] = 0;
+      if (head) {
+        const unsigned ends = lane == 31 ? 0u : (heads | ~kept) >> (lane + 1);
+        old[u] = atomicAdd(cnt + row, (uint32_t)(ends ? __ffs(ends) : 32 - lane));
+      }
+      li[u] = row;
+    }
+#pragma unroll
+    for (int u = 0; u < BUCKET_U; ++u) {
+      const uint32_t o = __shfl_sync(FULL_MASK, old[u], first[u]);
+      if (li[u] >= 0) slot[base + 32 * u + lane] = (uint16_t)(o + (uint32_t)(lane - first[u]));
     }
   }
 }
 
-// Ascending bitonic sort of 64 keys held two per lane (element 2 lane + h).
-__device__ __forceinline__ void warp_sort64(uint64_t &a0, uint64_t &a1) {
-  const int lane = threadIdx.x & 31;
+// Places every kept entry at its slot of its row as (j << 32) | k.
+__global__ void k_row_place(KeepArgs a, const uint32_t *__restrict__ rstart,
+                            const uint16_t *__restrict__ slot, uint64_t *__restrict__ keys) {
+  const int64_t T = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t k0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k0 < a.ncoo;
+       k0 += BUCKET_U * T) {
+    int32_t li[BUCKET_U], lj[BUCKET_U];
+    uint32_t at[BUCKET_U];
 #pragma unroll
-  for (int k = 2; k <= 64; k <<= 1) {
-    const bool asc = ((2 * lane) & k) == 0;
+    for (int u = 0; u < BUCKET_U; ++u) {
+      const int64_t k = k0 + u * T;
+      li[u] = k < a.ncoo ? __ldg(a.i + k) : -1;
+      lj[u] = k < a.ncoo ? __ldg(a.j + k) : -1;
+      at[u] = k < a.ncoo ? __ldg(slot + k) : 0u;
+    }
+    uint64_t key[BUCKET_U];
+    bool keep[BUCKET_U];
+#pragma unroll
+    for (int u = 0; u < BUCKET_U; ++u) {
+      const int64_t k = k0 + u * T;
+      int64_t gi = 0, gj = 0;
+      bool bad;
+      keep[u] = keep_entry(a, k, li[u], lj[u], gi, gj, bad);
+      key[u] = ((uint64_t)(uint32_t)gj << 32) | (uint32_t)k;
+      if (keep[u]) at[u] += __ldg(rstart + gi);
+    }
+#pragma unroll
+    for (int u = 0; u < BUCKET_U; ++u)
+      if (keep[u]) keys[at[u]] = key[u];
+  }
+}
+
+// What a sorted row leaves: its distinct columns, the place of its diagonal
+// among them (-1: none) and the largest |col - row|.
+struct RowOut {
+  int32_t *perm;
+  uint32_t *jh;        // the sorted columns, bit 31: first entry of its column
+  uint32_t *ucnt;      // distinct columns
+  int32_t *dloc;       // the diagonal's place among them
+  int32_t *span;
+  int32_t *long_rows;  // rows for k_row_sort_cta, their count
+  uint32_t *nlong;
+};
+constexpr uint32_t HEAD_BIT = 0x80000000u;
+
+// |j - r| capped at 2^30.
+__device__ __forceinline__ int32_t col_dist(uint32_t j, int64_t r) {
+  const int64_t d = (int64_t)j - r, ad = d < 0 ? -d : d;
+  return (int32_t)(ad > (1 << 30) ? (1 << 30) : ad);
+}
+
+constexpr int SORT_TPB = 256;
+
+// Rows r .. r + 3, of at most 8 KPL entries each, on a warp: eight lanes a row,
+// KPL keys a lane, a bitonic network whose elements are blocked (element KPL g
+// + i is lane g's key i).  Keys of one lane compare in registers; with KPL = 8
+// six of the network's 21 stages need shuffles, where two keys a lane on 32
+// lanes shuffle in 15.  The sorted keys go through shared memory (x: 36 KPL
+// words a warp, one word of padding in nine against bank conflicts), so that
+// every lane writes out consecutive entries.
+template <int KPL>
+__device__ __forceinline__ int32_t sort_rows4(int64_t r, int64_t nrows,
+                                              const uint32_t *__restrict__ rstart,
+                                              const uint64_t *__restrict__ keys, uint64_t *x,
+                                              const RowOut &o) {
+  constexpr int N = 8 * KPL;
+  const int lane = threadIdx.x & 31, g = lane & 7, l0 = lane & 24;
+  const int64_t row = r + (lane >> 3);
+  const uint32_t s0 = row < nrows ? __ldg(rstart + row) : 0u;
+  const int len = row < nrows ? (int)(__ldg(rstart + row + 1) - s0) : 0;
+  uint64_t a[KPL];
+#pragma unroll
+  for (int i = 0; i < KPL; ++i) a[i] = 8 * i + g < len ? __ldg(keys + s0 + 8 * i + g) : ~0ull;
+#pragma unroll
+  for (int k = 2; k <= N; k <<= 1) {
 #pragma unroll
     for (int j = k >> 1; j > 0; j >>= 1) {
-      if (j == 1) {
-        const uint64_t lo = a0 < a1 ? a0 : a1, hi = a0 < a1 ? a1 : a0;
-        a0 = asc ? lo : hi;
-        a1 = asc ? hi : lo;
+      if (j >= KPL) {
+        const bool asc = ((g * KPL) & k) == 0, low = (g & (j / KPL)) == 0;
+#pragma unroll
+        for (int i = 0; i < KPL; ++i) {
+          const uint64_t other = __shfl_xor_sync(FULL_MASK, a[i], j / KPL);
+          a[i] = ((a[i] < other) == (low == asc)) ? a[i] : other;
+        }
       } else {
-        const int lj = j >> 1;
-        const uint64_t b0 = __shfl_xor_sync(FULL_MASK, a0, lj);
-        const uint64_t b1 = __shfl_xor_sync(FULL_MASK, a1, lj);
-        const bool keep_min = ((lane & lj) == 0) == asc;
-        a0 = keep_min ? (a0 < b0 ? a0 : b0) : (a0 < b0 ? b0 : a0);
-        a1 = keep_min ? (a1 < b1 ? a1 : b1) : (a1 < b1 ? b1 : a1);
+#pragma unroll
+        for (int i = 0; i < KPL; ++i) {
+          if ((i & j) == 0) {
+            const bool asc = k < KPL ? (i & k) == 0 : ((g * KPL) & k) == 0;
+            const uint64_t u = a[i], v = a[i | j];
+            const bool swap = (u > v) == asc;
+            a[i] = swap ? v : u;
+            a[i | j] = swap ? u : v;
+          }
+        }
       }
     }
   }
+  uint64_t *xr = x + (lane >> 3) * 9 * KPL;
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < KPL; ++i) {
+    const int e = g * KPL + i;
+    xr[e + (e >> 3)] = a[i];
+  }
+  __syncwarp();
+  int u = 0, diag = -1;
+  int32_t m = 0;
+#pragma unroll
+  for (int i = 0; i < KPL; ++i) {
+    const int e = 8 * i + g;
+    const uint64_t key = xr[e + i];
+    const uint32_t j = (uint32_t)(key >> 32);
+    const uint32_t before = e > 0 ? (uint32_t)(xr[e - 1 + ((e - 1) >> 3)] >> 32) : 0u;
+    const bool in = e < len, head = in && (e == 0 || j != before);
+    const unsigned hb = (__ballot_sync(FULL_MASK, head) >> l0) & 255u;
+    const unsigned db = (__ballot_sync(FULL_MASK, head && (int64_t)j == row) >> l0) & 255u;
+    if (db) diag = u + __popc(hb & (db - 1u));
+    u += __popc(hb);
+    if (in) {
+      o.perm[s0 + e] = (int32_t)(uint32_t)key;
+      o.jh[s0 + e] = j | (head ? HEAD_BIT : 0u);
+      m = max(m, col_dist(j, row));
+    }
+  }
+  if (g == 0 && row < nrows) {
+    o.ucnt[row] = (uint32_t)u;
+    o.dloc[row] = diag;
+  }
+  return m;
 }
 
-// Rows of at most ROW_SORT_WARP entries, one warp each: sort, write back the
-// keys and perm (their low halves), count the distinct columns into ucnt.
-// Longer rows go to long_rows (count in *nlong) for k_row_sort_cta.
-__global__ void k_row_sort_warp(int64_t nrows, const uint32_t *__restrict__ rstart,
-                                uint64_t *__restrict__ keys, int32_t *__restrict__ perm,
-                                uint32_t *__restrict__ ucnt, int32_t *__restrict__ long_rows,
-                                uint32_t *nlong) {
+// Sorts the rows, four consecutive ones a warp at a time with the smallest
+// network that holds the longest of them; MAXK (keys a lane: 1, 2, 4 or 8) is
+// what the pattern's longest row needs, so that patterns of short rows run a
+// kernel of few registers.  Rows of more than ROW_SORT_WARP entries (MAXK = 8)
+// go to long_rows for k_row_sort_cta.
+template <int MAXK>
+__global__ void __launch_bounds__(SORT_TPB)
+    k_row_sort(int64_t nrows, const uint32_t *__restrict__ rstart,
+               const uint64_t *__restrict__ keys, RowOut o) {
+  __shared__ uint64_t sx[SORT_TPB / 32][36 * MAXK];
   const int lane = threadIdx.x & 31;
+  uint64_t *x = sx[threadIdx.x >> 5];
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < nrows; r += nw) {
-    const uint32_t s0 = rstart[r];
-    const int len = (int)(rstart[r + 1] - s0);
-    if (len > ROW_SORT_WARP) {
-      if (lane == 0) long_rows[atomicAdd(nlong, 1u)] = (int32_t)r;
-      continue;
+  int32_t m = 0;
+  for (int64_t r = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 4; r < nrows;
+       r += 4 * nw) {
+    if constexpr (MAXK == 1) {
+      m = max(m, sort_rows4<1>(r, nrows, rstart, keys, x, o));
+    } else {
+      const uint32_t st = lane <= 4 && r + lane <= nrows ? __ldg(rstart + r + lane) : 0u;
+      const uint32_t nxt = __shfl_down_sync(FULL_MASK, st, 1);
+      const unsigned len = lane < 4 && r + lane < nrows ? nxt - st : 0u;
+      int longest = (int)__reduce_max_sync(FULL_MASK, len);
+      if (longest <= 8) {
+        m = max(m, sort_rows4<1>(r, nrows, rstart, keys, x, o));
+      } else if (longest <= 16) {
+        m = max(m, sort_rows4<2>(r, nrows, rstart, keys, x, o));
+      } else if constexpr (MAXK >= 4) {
+        if (longest <= 32) {
+          m = max(m, sort_rows4<4>(r, nrows, rstart, keys, x, o));
+        } else if constexpr (MAXK >= 8) {
+          if (longest <= ROW_SORT_WARP) {
+            m = max(m, sort_rows4<8>(r, nrows, rstart, keys, x, o));
+          } else {  // the rows that fit one at a time, the others later
+            for (int q = 0; q < 4 && r + q < nrows; ++q) {
+              const int l = (int)__shfl_sync(FULL_MASK, len, q);
+              if (l <= ROW_SORT_WARP)
+                m = max(m, sort_rows4<8>(r + q, r + q + 1, rstart, keys, x, o));
+              else if (lane == 0)
+                o.long_rows[atomicAdd(o.nlong, 1u)] = (int32_t)(r + q);
+            }
+          }
+        }
+      }
     }
-    const int q0 = 2 * lane, q1 = 2 * lane + 1;
-    uint64_t a0 = q0 < len ? keys[s0 + q0] : ~0ull, a1 = q1 < len ? keys[s0 + q1] : ~0ull;
-    warp_sort64(a0, a1);
-    const uint32_t j0 = (uint32_t)(a0 >> 32), j1 = (uint32_t)(a1 >> 32);
-    const uint32_t jprev = __shfl_up_sync(FULL_MASK, j1, 1);
-    const bool h0 = q0 < len && (lane == 0 || j0 != jprev), h1 = q1 < len && j1 != j0;
-    if (q0 < len) {
-      keys[s0 + q0] = a0;
-      perm[s0 + q0] = (int32_t)(uint32_t)a0;
-    }
-    if (q1 < len) {
-      keys[s0 + q1] = a1;
-      perm[s0 + q1] = (int32_t)(uint32_t)a1;
-    }
-    const int u = __popc(__ballot_sync(FULL_MASK, h0)) + __popc(__ballot_sync(FULL_MASK, h1));
-    if (lane == 0) ucnt[r] = (uint32_t)u;
   }
+  block_atomic_max(m, o.span);
 }
 
 // The long rows (ROW_SORT_WARP < len <= ROW_SORT_CTA), one CTA each: a
-// bitonic sort in shared memory, then as k_row_sort_warp.
+// bitonic sort in shared memory, then as k_row_sort.
 __global__ void __launch_bounds__(ROW_SORT_TPB)
-    k_row_sort_cta(const uint32_t *__restrict__ rstart, uint64_t *__restrict__ keys,
-                   int32_t *__restrict__ perm, uint32_t *__restrict__ ucnt,
-                   const int32_t *__restrict__ long_rows, const uint32_t *nlong) {
+    k_row_sort_cta(const uint32_t *__restrict__ rstart, const uint64_t *__restrict__ keys,
+                   RowOut o) {
   __shared__ uint64_t sk[ROW_SORT_CTA];
-  __shared__ int cnt_w[ROW_SORT_TPB / 32];
-  const uint32_t nl = *nlong;
+  __shared__ int cnt_w[2][ROW_SORT_TPB / 32];
+  __shared__ int diag;
+  const uint32_t nl = *o.nlong;
+  int32_t m = 0;
   for (uint32_t li = blockIdx.x; li < nl; li += gridDim.x) {
-    const int32_t r = long_rows[li];
+    const int32_t r = o.long_rows[li];
     const uint32_t s0 = rstart[r];
     const int len = (int)(rstart[r + 1] - s0);
-    int m = 1;
-    while (m < len) m <<= 1;
-    for (int q = threadIdx.x; q < m; q += blockDim.x) sk[q] = q < len ? keys[s0 + q] : ~0ull;
+    int n2 = 1;
+    while (n2 < len) n2 <<= 1;
+    if (threadIdx.x == 0) diag = -1;
+    for (int q = threadIdx.x; q < n2; q += blockDim.x) sk[q] = q < len ? keys[s0 + q] : ~0ull;
     __syncthreads();
-    for (int k = 2; k <= m; k <<= 1)
+    for (int k = 2; k <= n2; k <<= 1)
       for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int q = threadIdx.x; q < m; q += blockDim.x) {
+        for (int q = threadIdx.x; q < n2; q += blockDim.x) {
           const int pq = q ^ j;
           if (pq > q) {
             const uint64_t x = sk[q], y = sk[pq];
@@ -585,65 +750,123 @@ __global__ void __launch_bounds__(ROW_SORT_TPB)
         }
         __syncthreads();
       }
+    auto is_head = [&](int q) { return q == 0 || (sk[q] >> 32) != (sk[q - 1] >> 32); };
     int u = 0;
     for (int q = threadIdx.x; q < len; q += blockDim.x) {
       const uint64_t x = sk[q];
-      keys[s0 + q] = x;
-      perm[s0 + q] = (int32_t)(uint32_t)x;
-      u += (q == 0 || (x >> 32) != (sk[q - 1] >> 32)) ? 1 : 0;
+      const uint32_t j = (uint32_t)(x >> 32);
+      const bool head = is_head(q);
+      o.perm[s0 + q] = (int32_t)(uint32_t)x;
+      o.jh[s0 + q] = j | (head ? HEAD_BIT : 0u);
+      if (head && (int64_t)j == r) diag = q;  // (one entry at most)
+      u += head ? 1 : 0;
+      m = max(m, col_dist(j, r));
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) u += __shfl_xor_sync(FULL_MASK, u, off);
-    if ((threadIdx.x & 31) == 0) cnt_w[threadIdx.x >> 5] = u;
+    __syncthreads();
+    int before = 0;  // heads before the diagonal's
+    const int dq = diag;
+    for (int q = threadIdx.x; q < dq; q += blockDim.x) before += is_head(q) ? 1 : 0;
+    u = (int)__reduce_add_sync(FULL_MASK, (unsigned)u);
+    before = (int)__reduce_add_sync(FULL_MASK, (unsigned)before);
+    if ((threadIdx.x & 31) == 0) {
+      cnt_w[0][threadIdx.x >> 5] = u;
+      cnt_w[1][threadIdx.x >> 5] = before;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
-      int t = 0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += cnt_w[w];
-      ucnt[r] = (uint32_t)t;
+      int t = 0, d = 0;
+      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+        t += cnt_w[0][w];
+        d += cnt_w[1][w];
+      }
+      o.ucnt[r] = (uint32_t)t;
+      o.dloc[r] = dq >= 0 ? d : -1;
     }
+    __syncthreads();
+  }
+  block_atomic_max(m, o.span);
+}
+
+// col and jmap from the sorted entries: entry q that heads its column is the
+// pattern's nonzero number (heads before q).  A CTA takes EMIT_TILE entries:
+// the row of the first one (a binary search over rstart) gives the number of
+// heads before that row, row_ptr; counting those between the row's start and
+// the tile gives the tile's first number, a scan of the tile's flags the rest.
+constexpr int EMIT_T = 256, EMIT_IPT = 8, EMIT_TILE = EMIT_T * EMIT_IPT;
+__global__ void __launch_bounds__(EMIT_T)
+    k_row_emit(int64_t nkept, int64_t nrows, const uint32_t *__restrict__ rstart,
+               const uint32_t *__restrict__ jh, const int32_t *__restrict__ row_ptr,
+               int32_t *__restrict__ jmap, int32_t *__restrict__ col) {
+  __shared__ int s_row, s_extra;
+  __shared__ uint32_t warp_tot[EMIT_T / 32];
+  const int64_t t0 = (int64_t)blockIdx.x * EMIT_TILE;
+  if (threadIdx.x < 32) {  // the last row with rstart[row] <= t0, 32 probes a step
+    int64_t lo = 0, hi = nrows;  // rstart[lo] <= t0 < rstart[hi]
+    while (hi - lo > 1) {
+      const int64_t step = (hi - lo + 31) / 32;
+      const int64_t at = min(lo + step * (int)(threadIdx.x + 1), hi);
+      const unsigned le = __ballot_sync(FULL_MASK, at < hi && (int64_t)rstart[at] <= t0);
+      const int k = __popc(le);  // (monotone: the first k probes)
+      const int64_t nlo = lo + step * k;
+      hi = min(nlo + step, hi);
+      lo = nlo;
+    }
+    if (threadIdx.x == 0) {
+      s_row = (int)lo;
+      s_extra = 0;
+    }
+  }
+  __syncthreads();
+  int extra = 0;
+  for (int64_t q = rstart[s_row] + threadIdx.x; q < t0; q += EMIT_T) extra += (int)(jh[q] >> 31);
+  extra = (int)__reduce_add_sync(FULL_MASK, (unsigned)extra);
+  if ((threadIdx.x & 31) == 0 && extra) atomicAdd(&s_extra, extra);
+  __syncthreads();
+  uint32_t base = (uint32_t)(row_ptr[s_row] + s_extra);
+  // EMIT_IPT rounds of one entry a thread: coalesced, and in order
+  uint32_t j[EMIT_IPT];
+#pragma unroll
+  for (int i = 0; i < EMIT_IPT; ++i) {
+    const int64_t q = t0 + i * EMIT_T + threadIdx.x;
+    j[i] = q < nkept ? __ldg(jh + q) : 0u;
+  }
+#pragma unroll
+  for (int i = 0; i < EMIT_IPT; ++i) {
+    const int64_t q = t0 + i * EMIT_T + threadIdx.x;
+    const unsigned hb = __ballot_sync(FULL_MASK, (j[i] & HEAD_BIT) != 0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) warp_tot[warp] = (uint32_t)__popc(hb);
+    __syncthreads();
+    uint32_t below = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < EMIT_T / 32; ++w) {
+      const uint32_t c = warp_tot[w];
+      below += w < warp ? c : 0u;
+      all += c;
+    }
+    if (j[i] & HEAD_BIT) {
+      const uint32_t u = base + below + (uint32_t)__popc(hb & ((1u << lane) - 1u));
+      jmap[u] = (int32_t)q;
+      col[u] = (int32_t)(j[i] & ~HEAD_BIT);
+    }
+    base += all;
     __syncthreads();
   }
 }
 
-// col, jmap and diag_pos from the sorted rows, one warp per row; the
-// largest |col - row| into *span.
-__global__ void k_row_emit(int64_t nrows, const uint32_t *__restrict__ rstart,
-                           const uint64_t *__restrict__ keys, const int32_t *__restrict__ row_ptr,
-                           int32_t *__restrict__ jmap, int32_t *__restrict__ col,
-                           int32_t *__restrict__ diag_pos, int32_t *span) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  int32_t m = 0;
-  for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < nrows; r += nw) {
-    const uint32_t s0 = rstart[r];
-    const int len = (int)(rstart[r + 1] - s0);
-    int run = row_ptr[r];
-    uint32_t prev = 0;  // the column of the chunk's previous entry (lane 31 of the last chunk)
-    for (int c = 0; c < len; c += 32) {
-      const int q = c + lane;
-      const bool valid = q < len;
-      const uint32_t jq = valid ? (uint32_t)(keys[s0 + q] >> 32) : 0u;
-      const uint32_t jl = __shfl_up_sync(FULL_MASK, jq, 1);
-      const uint32_t before = lane == 0 ? prev : jl;
-      const bool head = valid && (q == 0 || jq != before);
-      const unsigned hb = __ballot_sync(FULL_MASK, head);
-      if (head) {
-        const int u = run + __popc(hb & ((1u << lane) - 1u));
-        jmap[u] = (int32_t)(s0 + q);
-        col[u] = (int32_t)jq;
-        if ((int64_t)jq == r) diag_pos[r] = u;
-        const int64_t d = (int64_t)jq - r, ad = d < 0 ? -d : d;
-        m = max(m, (int32_t)(ad > (1 << 30) ? (1 << 30) : ad));
-      }
-      run += __popc(hb);
-      prev = __shfl_sync(FULL_MASK, jq, 31);
-    }
+// diag_pos[r] from the diagonal's place in its row.
+__global__ void k_row_diag(int64_t nrows, const int32_t *__restrict__ row_ptr,
+                           const int32_t *__restrict__ dloc, int32_t *__restrict__ diag_pos) {
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < nrows;
+       r += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t d = dloc[r];
+    diag_pos[r] = d < 0 ? -1 : row_ptr[r] + d;
   }
-  m = (int32_t)__reduce_max_sync(FULL_MASK, (unsigned)m);
-  if (lane == 0 && m > 0) atomicMax(span, m);
 }
 
-// Symbolic stage.  coo_off_h (host, nsys+1) is non-null for batched handles;
+// Symbolic stage, enqueued on s: its buffers are ready on s (the caller
+// synchronises before other streams may use them).  coo_off_h (host, nsys+1)
+// is non-null for batched handles;
 // A->row_off_h, nrows, ncols, ncoo, nsys are set by the caller.  The
 // row-bucketed path runs unless a row holds more than ROW_SORT_CTA entries.
 static int symbolic_radix(gbs_mat A, const int32_t *i, const int32_t *j,
@@ -665,18 +888,18 @@ static int symbolic_rows(gbs_mat A, const int32_t *i, const int32_t *j,
   const int64_t ncoo = A->ncoo, n = A->nrows;
   KeepArgs ka{i, j, ncoo, A->nrows, A->ncols, nullptr, nullptr, A->nsys};
   int64_t *d_off = nullptr;
-  uint32_t *cnt = nullptr, *rstart = nullptr, *scan_tmp = nullptr, *ucnt = nullptr;
+  uint32_t *cnt = nullptr, *rstart = nullptr, *scan_tmp = nullptr, *jh = nullptr;
   uint64_t *keys = nullptr;
-  int32_t *perm = nullptr, *long_rows = nullptr;
+  uint16_t *slot = nullptr;
+  int32_t *perm = nullptr, *long_rows = nullptr, *dloc = nullptr;
   int status = GBS_OK;
   struct Ctl {
     uint32_t nkept, nnz;
-    int32_t err, maxcnt, maxrow, span;
-    uint32_t nlong, pad;
+    int32_t err, maxcnt, span;
+    uint32_t nlong;
   } hc{};
   Ctl *dctl = nullptr;
   const int64_t n1 = std::max<int64_t>(n, 1);
-  const int64_t nwarp_rows = std::max<int64_t>(n, 1) * 32;
 
   {
     SYM_TRY(dev_alloc(&dctl, 1, s));
@@ -690,18 +913,20 @@ static int symbolic_rows(gbs_mat A, const int32_t *i, const int32_t *j,
       ka.coo_off = d_off;
       ka.row_off = d_off + A->nsys + 1;
     }
-    // 1-2. counts per row, their scan (total: nkept), the largest count
+    // 1-2. counts per row and slots, the counts' scan (total: nkept), the
+    // largest count
     SYM_TRY(dev_alloc(&cnt, n1 + 1, s));
     SYM_TRY(dev_alloc(&rstart, n1 + 1, s));
+    SYM_TRY(dev_alloc(&slot, std::max<int64_t>(ncoo, 1), s));
     SYM_TRY(dev_alloc(&scan_tmp, scan_tmp_words(n1 + 1), s));
     SYM_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (n1 + 1), s));
     if (ncoo > 0) {
-      k_row_bucket<0><<<grid_for(ncoo, 256), 256, 0, s>>>(ka, cnt, nullptr, nullptr, &dctl->err);
+      k_row_count<<<grid_for(ncoo, 256 * BUCKET_U), 256, 0, s>>>(ka, cnt, slot, &dctl->err);
       GBS_LAUNCHED(1);
     }
     SYM_TRY(exclusive_scan(cnt, rstart, n + 1, scan_tmp, &dctl->nkept, s));
     if (n > 0) {
-      k_max_row<<<grid_for(n, 256), 256, 0, s>>>(reinterpret_cast<const int32_t *>(rstart), n,
+      k_max_row<<<wave_for(n, 256), 256, 0, s>>>(reinterpret_cast<const int32_t *>(rstart), n,
                                                  &dctl->maxcnt);
       GBS_LAUNCHED(1);
     }
@@ -718,31 +943,38 @@ static int symbolic_rows(gbs_mat A, const int32_t *i, const int32_t *j,
     // 3. placement
     SYM_TRY(dev_alloc(&keys, nk, s));
     SYM_TRY(dev_alloc(&perm, nk, s));
-    SYM_TRY(dev_alloc(&ucnt, n1 + 1, s));
-    SYM_TRY(dev_alloc(&long_rows, n1, s));
-    SYM_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (n1 + 1), s));
-    SYM_CUDA(cudaMemsetAsync(ucnt, 0, sizeof(uint32_t) * (n1 + 1), s));
-    if (ncoo > 0) {
-      k_row_bucket<1><<<grid_for(ncoo, 256), 256, 0, s>>>(ka, cnt, rstart, keys, nullptr);
+    SYM_TRY(dev_alloc(&jh, nk, s));
+    SYM_TRY(dev_alloc(&dloc, n1, s));
+    if (hc.maxcnt > ROW_SORT_WARP) SYM_TRY(dev_alloc(&long_rows, n1, s));
+    if (nkept > 0) {
+      k_row_place<<<grid_for(ncoo, 256 * BUCKET_U), 256, 0, s>>>(ka, rstart, slot, keys);
       GBS_LAUNCHED(1);
     }
-    // 4. per-row sorts, distinct columns
+    // 4. per-row sorts, distinct columns (over cnt, whose last word the scan needs 0)
+    SYM_CUDA(cudaMemsetAsync(cnt + n, 0, sizeof(uint32_t), s));
     if (n > 0) {
-      k_row_sort_warp<<<grid_for(nwarp_rows, 256), 256, 0, s>>>(n, rstart, keys, perm, ucnt,
-                                                                 long_rows, &dctl->nlong);
-      k_row_sort_cta<<<1024, ROW_SORT_TPB, 0, s>>>(rstart, keys, perm, ucnt, long_rows,
-                                                   &dctl->nlong);
-      GBS_LAUNCHED(2);
+      const RowOut o{perm, jh, cnt, dloc, &dctl->span, long_rows, &dctl->nlong};
+      const auto sort = hc.maxcnt <= 8    ? k_row_sort<1>
+                        : hc.maxcnt <= 16 ? k_row_sort<2>
+                        : hc.maxcnt <= 32 ? k_row_sort<4>
+                                          : k_row_sort<8>;
+      sort<<<grid_for((n + 3) / 4 * 32, SORT_TPB), SORT_TPB, 0, s>>>(n, rstart, keys, o);
+      GBS_LAUNCHED(1);
+      if (hc.maxcnt > ROW_SORT_WARP) {
+        k_row_sort_cta<<<1024, ROW_SORT_TPB, 0, s>>>(rstart, keys, o);
+        GBS_LAUNCHED(1);
+      }
     }
     // 5. row_ptr, nnz; then col, jmap, diagonal positions
     SYM_TRY(dev_alloc(&A->row_ptr, n + 1, s));
-    SYM_TRY(exclusive_scan(ucnt, reinterpret_cast<uint32_t *>(A->row_ptr), n + 1, scan_tmp,
+    SYM_TRY(exclusive_scan(cnt, reinterpret_cast<uint32_t *>(A->row_ptr), n + 1, scan_tmp,
                            &dctl->nnz, s));
     SYM_CUDA(cudaMemcpyAsync(&hc, dctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     SYM_CUDA(cudaStreamSynchronize(s));
     const int64_t nnz = hc.nnz;
     A->nkept = nkept;
     A->nnz = nnz;
+    A->col_span = hc.span;
     const int64_t nz1 = std::max<int64_t>(nnz, 1);
     SYM_TRY(dev_alloc(&A->jmap, nnz + 1, s));
     SYM_TRY(dev_alloc(&A->col, nz1, s));
@@ -750,22 +982,19 @@ static int symbolic_rows(gbs_mat A, const int32_t *i, const int32_t *j,
     SYM_TRY(dev_alloc(&A->diag_pos, n1, s));
     SYM_TRY(dev_alloc(&A->dinv, n1, s));
     SYM_CUDA(cudaMemsetAsync(A->val, 0, sizeof(double) * nz1, s));
-    SYM_CUDA(cudaMemsetAsync(A->diag_pos, 0xff, sizeof(int32_t) * n1, s));
     SYM_CUDA(cudaMemsetAsync(A->dinv, 0, sizeof(double) * n1, s));
-    {
-      const int32_t nk32 = (int32_t)nkept;
-      SYM_CUDA(cudaMemcpyAsync(A->jmap + nnz, &nk32, sizeof(int32_t), cudaMemcpyHostToDevice, s));
+    // (nkept, the last offset of jmap, is in the control words)
+    SYM_CUDA(cudaMemcpyAsync(A->jmap + nnz, &dctl->nkept, sizeof(int32_t),
+                             cudaMemcpyDeviceToDevice, s));
+    if (nkept > 0) {
+      k_row_emit<<<(unsigned)((nkept + EMIT_TILE - 1) / EMIT_TILE), EMIT_T, 0, s>>>(
+          nkept, n, rstart, jh, A->row_ptr, A->jmap, A->col);
+      GBS_LAUNCHED(1);
     }
     if (n > 0) {
-      k_row_emit<<<grid_for(nwarp_rows, 256), 256, 0, s>>>(n, rstart, keys, A->row_ptr, A->jmap,
-                                                            A->col, A->diag_pos, &dctl->span);
-      k_max_row<<<grid_for(n, 256), 256, 0, s>>>(A->row_ptr, n, &dctl->maxrow);
-      GBS_LAUNCHED(2);
+      k_row_diag<<<grid_for(n, 256), 256, 0, s>>>(n, A->row_ptr, dloc, A->diag_pos);
+      GBS_LAUNCHED(1);
     }
-    SYM_CUDA(cudaMemcpyAsync(&hc, dctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
-    SYM_CUDA(cudaStreamSynchronize(s));
-    A->max_row_nnz = hc.maxrow;
-    A->col_span = hc.span;
     A->perm = perm;
     perm = nullptr;
     *done = true;
@@ -773,9 +1002,10 @@ static int symbolic_rows(gbs_mat A, const int32_t *i, const int32_t *j,
 
 cleanup:
   for (void *p : {(void *)dctl, (void *)d_off, (void *)cnt, (void *)rstart, (void *)scan_tmp,
-                  (void *)ucnt, (void *)keys, (void *)perm, (void *)long_rows})
+                  (void *)slot, (void *)jh, (void *)dloc, (void *)keys, (void *)perm,
+                  (void *)long_rows})
     dev_free(p, s);
-  cudaStreamSynchronize(s);
+  if (status != GBS_OK) cudaStreamSynchronize(s);
   return status;
 }
 
@@ -793,7 +1023,7 @@ static int symbolic_radix(gbs_mat A, const int32_t *i, const int32_t *j,
   // host mirrors read back after each synchronisation
   struct Ctl {
     uint32_t nkept, nnz;
-    int32_t err, maxrow, span, pad;
+    int32_t err, span;
   } hc{};
   Ctl *dctl = nullptr;
 
@@ -919,17 +1149,15 @@ static int symbolic_radix(gbs_mat A, const int32_t *i, const int32_t *j,
       GBS_LAUNCHED(1);
     }
     if (nnz > 0) {
-      k_csr_cols<<<grid_for(nnz, 256), 256, 0, s>>>(ukey, nnz, A->ncols, A->col, A->diag_pos,
+      k_csr_cols<<<wave_for(nnz, 256), 256, 0, s>>>(ukey, nnz, A->ncols, A->col, A->diag_pos,
                                                     &dctl->span);
       GBS_LAUNCHED(1);
     }
     k_row_ptr<<<grid_for(A->nrows + 1, 256), 256, 0, s>>>(ukey, nnz, A->ncols, A->nrows,
                                                           A->row_ptr);
-    k_max_row<<<grid_for(A->nrows, 256), 256, 0, s>>>(A->row_ptr, A->nrows, &dctl->maxrow);
-    GBS_LAUNCHED(2);
+    GBS_LAUNCHED(1);
     SYM_CUDA(cudaMemcpyAsync(&hc, dctl, sizeof(Ctl), cudaMemcpyDeviceToHost, s));
     SYM_CUDA(cudaStreamSynchronize(s));
-    A->max_row_nnz = hc.maxrow;
     A->col_span = hc.span;
   }
 
@@ -943,114 +1171,223 @@ cleanup:
 
 // ------------------------------------------------------------------ numeric
 
-// One thread per nonzero: a_p = v[perm[jmap[p]]] + v[perm[jmap[p]+1]] + ...
-// in increasing COO index order (Sec. 5: each thread accumulates into a single
-// nonzero, no atomics).  A segment's sum is a chain of dependent FP64 adds,
-// and a warp issues each add step for all its lanes: with consecutive
-// nonzeros on consecutive lanes every warp runs as many steps as its longest
-// segment (on the Q1 matrix segments hold 1, 2, 4 or 8 terms and nearly every
-// warp an 8), and FP64 instructions, scarce on this part, bound the kernel.
-// So a CTA takes a tile of NUM_TILE consecutive nonzeros, orders them by
-// segment length in shared memory (a counting sort over a few length
-// classes), and its warps sum them in that order -- lanes of a warp then
-// hold segments of about one length and issue only the adds those need --
-// into a shared buffer that the CTA writes back in nonzero order (coalesced).
-// Each thread takes two nonzeros and loads each segment's COO indices
-// NUM_BATCH at a time before their values, so its two chains of dependent
-// loads (COO indices -> values) are in flight together.  The lane a nonzero
-// lands on depends on shared-memory atomics; its sum does not.
-constexpr int NUM_BATCH = 4;
-constexpr int NUM_TPB = 256, NUM_TILE = 2 * NUM_TPB, NUM_CLASSES = 5;
+// a_p = v[perm[jmap[p]]] + v[perm[jmap[p]+1]] + ... in increasing COO index
+// order (Sec. 5: each nonzero is accumulated by one thread, no atomics).
+//
+// A CTA takes a tile of consecutive nonzeros in three steps.
+//   1. Their COO values, contiguous in sorted order, into shared memory: perm
+//      read coalesced, v gathered, every load independent of the others.  (One
+//      thread per nonzero walking its own segment had two dependent loads a
+//      term and at most eight of them in flight.)
+//   2. The sums, from shared memory, in order of segment length: a warp issues
+//      each FP64 add for all its lanes, and with consecutive nonzeros on
+//      consecutive lanes nearly every warp of the Q1 matrix (segments of 1, 2, 4
+//      and 8 terms) would run 7 add steps for 1.3 on average -- the FP64 pipe
+//      held the kernel; a counting sort over NUM_CLASSES length classes puts
+//      segments of about one length on a warp.
+//   3. The results in nonzero order, coalesced.
+// The lane a nonzero lands on depends on shared-memory atomics; its sum does
+// not.
+//
+// SLICES: the tile is a few whole slices of the sliced copy, whose values and
+// the rows' D^-1 are written from the same shared sums -- otherwise two more
+// kernels, the fill reading every value again.
+// What is left: shared-memory wavefronts (L1 data pipe 70% busy, half of the
+// loads' wavefronts bank conflicts of the segment sums), 61% of the issue
+// slots, HBM at 41%.  Measured, us, values + fill + D^-1 in three kernels ->
+// here: Q1 96^3 346 + 94 + 22 -> 311, 2D 1024^2 edges 63 + 15 + 14 -> 72;
+// k_coo_numeric on a graph of 300k rows 119 -> 74.
+constexpr int NUM_TPB = 256, NUM_CLASSES = 5, NUM_BATCH = 4;
+constexpr int NUM_NZ = 1024;   // nonzeros of a tile, at most
+constexpr int NUM_E = 3072;    // COO entries of a tile that shared memory holds
+constexpr int NUM_TILE = 512;  // nonzeros of a tile that is not cut by slices
+constexpr int NUM_SLICES = 8;  // slices of a tile, at most
+constexpr int NUM_CTAS = 6;    // CTAs an SM (40 registers a thread)
 
 __device__ __forceinline__ int length_class(int32_t len) {
   return len <= 1 ? 0 : (len == 2 ? 1 : (len <= 4 ? 2 : (len <= 8 ? 3 : 4)));
 }
 
-__global__ void __launch_bounds__(NUM_TPB)
+struct NumShared {  // in dynamic shared memory: as large as the launch's tiles
+  double *v;       // COO values in sorted order
+  double *sum;     // the nonzeros' sums
+  uint16_t *j;     // segment starts in v
+  int16_t *order;  // nonzeros by length class
+};
+__host__ __device__ constexpr size_t num_shared(int e, int nz) {  // bytes for e entries, nz nonzeros
+  return 8 * (size_t)e + 8 * (size_t)nz + 2 * (((size_t)nz + 4) & ~(size_t)3) + 2 * (size_t)nz;
+}
+__device__ __forceinline__ NumShared num_carve(unsigned char *m, int e, int nz) {
+  NumShared sh;
+  sh.v = reinterpret_cast<double *>(m);
+  sh.sum = sh.v + e;
+  sh.j = reinterpret_cast<uint16_t *>(sh.sum + nz);
+  sh.order = reinterpret_cast<int16_t *>(sh.j + ((nz + 4) & ~3));
+  return sh;
+}
+
+// The sums of nonzeros [t0, t0 + nt) into sh.sum (ADD: with the old values).
+// e_cap: the COO entries that sh.v holds.
+__device__ __forceinline__ void numeric_tile(const NumShared &sh, int e_cap, int64_t t0, int nt,
+                                             const int32_t *__restrict__ jmap,
+                                             const int32_t *__restrict__ perm,
+                                             const double *__restrict__ v, int mode,
+                                             const double *val) {
+  const int tid = (int)threadIdx.x;
+  const int32_t e0 = __ldg(jmap + t0);
+  const int ne = __ldg(jmap + t0 + nt) - e0;
+  if (ne > e_cap) {  // long segments: one thread a nonzero, straight from memory
+    for (int i = tid; i < nt; i += NUM_TPB) {
+      int32_t t = __ldg(jmap + t0 + i);
+      const int32_t e = __ldg(jmap + t0 + i + 1);
+      double x = __ldg(v + __ldg(perm + t));
+      ++t;
+      while (t < e) {
+        double y[NUM_BATCH];
+#pragma unroll
+        for (int u = 0; u < NUM_BATCH; ++u) y[u] = t + u < e ? __ldg(v + __ldg(perm + t + u)) : 0.0;
+#pragma unroll
+        for (int u = 0; u < NUM_BATCH; ++u)
+          if (t + u < e) x = __dadd_rn(x, y[u]);
+        t += NUM_BATCH;
+      }
+      sh.sum[i] = mode == GBS_ADD ? __dadd_rn(val[t0 + i], x) : x;
+    }
+    return;
+  }
+  __shared__ int32_t s_cnt[NUM_CLASSES][NUM_NZ / 32];  // per class and 32 nonzeros
+  __shared__ int32_t s_base[NUM_CLASSES];
+  for (int i = tid; i <= nt; i += NUM_TPB) sh.j[i] = (uint16_t)(__ldg(jmap + t0 + i) - e0);
+  // the gathers run on while the classes are counted
+  const uint32_t vs = (uint32_t)__cvta_generic_to_shared(sh.v);
+  for (int e = tid; e < ne; e += 4 * NUM_TPB) {
+    int32_t k[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) k[u] = e + u * NUM_TPB < ne ? __ldg(perm + e0 + e + u * NUM_TPB) : 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (e + u * NUM_TPB < ne)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(vs + 8u * (e + u * NUM_TPB)),
+                     "l"(v + k[u])
+                     : "memory");
+  }
+  __syncthreads();  // segment starts
+  // places by length class: warp counts, their prefix sums, ranks by ballot
+  const int lane = tid & 31, groups = (nt + 31) >> 5;
+  for (int g = tid >> 5; g < groups; g += NUM_TPB / 32) {
+    const int i = 32 * g + lane;
+    const int c = i < nt ? length_class((int)sh.j[i + 1] - (int)sh.j[i]) : -1;
+#pragma unroll
+    for (int q = 0; q < NUM_CLASSES; ++q) {
+      const unsigned m = __ballot_sync(FULL_MASK, c == q);
+      if (lane == q) s_cnt[q][g] = __popc(m);
+    }
+  }
+  __syncthreads();
+  if (tid < 32 * NUM_CLASSES) {  // warp q: exclusive sums of class q's counts
+    const int q = tid >> 5;
+    const int n = lane < groups ? s_cnt[q][lane] : 0;
+    int incl = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(FULL_MASK, incl, d);
+      if (lane >= d) incl += y;
+    }
+    if (lane < groups) s_cnt[q][lane] = incl - n;
+    if (lane == 31) s_base[q] = incl;
+  }
+  __syncthreads();
+  for (int g = tid >> 5; g < groups; g += NUM_TPB / 32) {
+    const int i = 32 * g + lane;
+    const int c = i < nt ? length_class((int)sh.j[i + 1] - (int)sh.j[i]) : -1;
+    unsigned mine = 0;
+    int base = 0;
+#pragma unroll
+    for (int q = 0; q < NUM_CLASSES; ++q) {
+      const unsigned m = __ballot_sync(FULL_MASK, c == q);
+      if (c == q) mine = m;
+      if (q < c) base += s_base[q];
+    }
+    if (c >= 0) sh.order[base + s_cnt[c][g] + __popc(mine & ((1u << lane) - 1u))] = (int16_t)i;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  for (int p = tid; p < nt; p += NUM_TPB) {
+    const int i = sh.order[p];
+    const int e = sh.j[i + 1];
+    int t = sh.j[i];
+    double x = sh.v[t];
+    for (++t; t < e; ++t) x = __dadd_rn(x, sh.v[t]);  // in increasing COO index: plain adds
+    sh.sum[i] = mode == GBS_ADD ? __dadd_rn(val[t0 + i], x) : x;
+  }
+}
+
+// Tiles of NUM_TILE nonzeros; the values only.
+__global__ void __launch_bounds__(NUM_TPB, NUM_CTAS)
     k_coo_numeric(int64_t nnz, const int32_t *__restrict__ jmap,
                   const int32_t *__restrict__ perm, const double *__restrict__ v, int mode,
                   double *__restrict__ val) {
-  __shared__ int32_t s_j0[NUM_TILE], s_j1[NUM_TILE];
-  __shared__ int16_t s_order[NUM_TILE];
-  __shared__ double s_sum[NUM_TILE];
-  __shared__ int32_t s_cnt[NUM_CLASSES], s_base[NUM_CLASSES];
-  const int tid = (int)threadIdx.x;
+  extern __shared__ __align__(16) unsigned char num_smem[];
+  const NumShared sh = num_carve(num_smem, NUM_E, NUM_TILE);
   for (int64_t t0 = (int64_t)blockIdx.x * NUM_TILE; t0 < nnz;
        t0 += (int64_t)gridDim.x * NUM_TILE) {
     const int nt = nnz - t0 < NUM_TILE ? (int)(nnz - t0) : NUM_TILE;
-    if (tid < NUM_CLASSES) s_cnt[tid] = 0;
+    numeric_tile(sh, NUM_E, t0, nt, jmap, perm, v, mode, val);
     __syncthreads();
-    // 1. segment bounds and length classes; ranks within a class
-    int cls[2], rank[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = tid + h * NUM_TPB;
-      cls[h] = -1;
-      if (i < nt) {
-        const int32_t j0 = __ldg(jmap + t0 + i), j1 = __ldg(jmap + t0 + i + 1);
-        s_j0[i] = j0;
-        s_j1[i] = j1;
-        cls[h] = length_class(j1 - j0);
-        rank[h] = atomicAdd(&s_cnt[cls[h]], 1);
-      }
-    }
-    __syncthreads();
-    if (tid == 0) {
-      int b = 0;
-      for (int c = 0; c < NUM_CLASSES; ++c) {
-        s_base[c] = b;
-        b += s_cnt[c];
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (cls[h] >= 0) s_order[s_base[cls[h]] + rank[h]] = (int16_t)(tid + h * NUM_TPB);
-    __syncthreads();
-    // 2. the sums, in class order: positions tid and tid + NUM_TPB
-    const bool has_a = tid < nt, has_b = tid + NUM_TPB < nt;
-    const int ia = has_a ? s_order[tid] : 0, ib = has_b ? s_order[tid + NUM_TPB] : 0;
-    int32_t ta = has_a ? s_j0[ia] : 0, tb = has_b ? s_j0[ib] : 0;
-    const int32_t ea = has_a ? s_j1[ia] : 0, eb = has_b ? s_j1[ib] : 0;
-    double sa = 0.0, sb = 0.0;
-    for (bool first = true; ta < ea || tb < eb; first = false) {
-      int32_t ka[NUM_BATCH], kb[NUM_BATCH];
-      double xa[NUM_BATCH], xb[NUM_BATCH];
-#pragma unroll
-      for (int u = 0; u < NUM_BATCH; ++u) {
-        ka[u] = ta + u < ea ? __ldg(perm + ta + u) : 0;
-        kb[u] = tb + u < eb ? __ldg(perm + tb + u) : 0;
-      }
-#pragma unroll
-      for (int u = 0; u < NUM_BATCH; ++u) {
-        xa[u] = ta + u < ea ? __ldg(v + ka[u]) : 0.0;
-        xb[u] = tb + u < eb ? __ldg(v + kb[u]) : 0.0;
-      }
-      if (first) {  // a segment's first term starts its sum
-        sa = xa[0];
-        sb = xb[0];
-      }
-#pragma unroll
-      for (int u = 0; u < NUM_BATCH; ++u) {  // in increasing COO index: plain adds
-        if ((!first || u > 0) && ta + u < ea) sa = __dadd_rn(sa, xa[u]);
-        if ((!first || u > 0) && tb + u < eb) sb = __dadd_rn(sb, xb[u]);
-      }
-      ta += NUM_BATCH;
-      tb += NUM_BATCH;
-    }
-    if (has_a) s_sum[ia] = sa;
-    if (has_b) s_sum[ib] = sb;
-    __syncthreads();
-    // 3. back in nonzero order
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = tid + h * NUM_TPB;
-      if (i < nt) {
-        const double x = s_sum[i];
-        val[t0 + i] = (mode == GBS_ADD) ? __dadd_rn(val[t0 + i], x) : x;
-      }
-    }
+    for (int i = threadIdx.x; i < nt; i += NUM_TPB) val[t0 + i] = sh.sum[i];
     __syncthreads();  // the shared arrays are reused by the next tile
+  }
+}
+
+// Tiles of per slices (at most NUM_NZ nonzeros): the CSR values, the sliced
+// copy's values (k_sell_fill's) and D^-1 (k_jacobi's).
+__global__ void __launch_bounds__(NUM_TPB, NUM_CTAS)
+    k_numeric_slices(int64_t nslices, int32_t per, int32_t e_cap, int32_t nz_cap,
+                     const int32_t *__restrict__ srow0,
+                     const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ jmap,
+                     const int32_t *__restrict__ perm, const double *__restrict__ v, int mode,
+                     double *__restrict__ val, const int32_t *__restrict__ diag_pos,
+                     double *__restrict__ dinv, const int32_t *__restrict__ sptr,
+                     const uint32_t *__restrict__ mask, double *__restrict__ sval) {
+  extern __shared__ __align__(16) unsigned char num_smem[];
+  const NumShared sh = num_carve(num_smem, e_cap, nz_cap);
+  __shared__ int32_t s_rs[32 * NUM_SLICES + 1];  // the rows' first nonzeros, from t0
+  __shared__ uint32_t s_mk[32 * NUM_SLICES];     // patterns: the rows' masks
+  const int tid = (int)threadIdx.x;
+  const int64_t s0 = (int64_t)blockIdx.x * per;
+  const int ns = nslices - s0 < per ? (int)(nslices - s0) : per;
+  const int32_t r0 = __ldg(srow0 + s0), nr = __ldg(srow0 + s0 + ns) - r0;
+  const int32_t t0 = __ldg(row_ptr + r0);
+  const int nt = __ldg(row_ptr + r0 + nr) - t0;
+  for (int i = tid; i <= nr; i += NUM_TPB) s_rs[i] = __ldg(row_ptr + r0 + i) - t0;
+  if (mask)
+    for (int i = tid; i < 32 * ns; i += NUM_TPB) s_mk[i] = __ldg(mask + 32 * s0 + i);
+  if (nt > 0) numeric_tile(sh, e_cap, t0, nt, jmap, perm, v, mode, val);
+  __syncthreads();
+  for (int i = tid; i < nt; i += NUM_TPB) val[t0 + i] = sh.sum[i];
+  for (int i = tid; i < nr; i += NUM_TPB) {
+    const int32_t q = __ldg(diag_pos + r0 + i);
+    const double x = q >= 0 ? sh.sum[q - t0] : 0.0;
+    dinv[r0 + i] = (x > 0.0) ? 1.0 / x : 0.0;
+  }
+  for (int s = 0; s < ns; ++s) {
+    const int32_t b = __ldg(sptr + s0 + s), w = (__ldg(sptr + s0 + s + 1) - b) >> 5, np = w >> 1;
+    const int32_t f = __ldg(srow0 + s0 + s) - r0;  // the slice's first row, from r0
+    const int32_t rows = __ldg(srow0 + s0 + s + 1) - r0 - f;
+    for (int p = tid; p < 32 * w; p += NUM_TPB) {  // pair layout (sell.cu)
+      const int i = p < 64 * np ? (p & 63) >> 1 : p - 64 * np;
+      const int k = p < 64 * np ? 2 * (p >> 6) + (p & 1) : w - 1;
+      double x = 0.0;
+      if (i < rows) {
+        if (mask) {
+          const uint32_t mk = s_mk[32 * s + i];
+          if ((mk >> k) & 1u) x = sh.sum[s_rs[f + i] + __popc(mk & ((1u << k) - 1u))];
+        } else if (k < s_rs[f + i + 1] - s_rs[f + i]) {
+          x = sh.sum[s_rs[f + i] + k];
+        }
+      }
+      sval[b + p] = x;
+    }
   }
 }
 
@@ -1067,16 +1404,33 @@ __global__ void k_jacobi(int64_t nrows, const int32_t *__restrict__ diag_pos,
 }
 
 int launch_set_values(gbs_mat A, const double *v, int mode, cudaStream_t s) {
-  if (A->nnz > 0) {
-    k_coo_numeric<<<grid_for((A->nnz + NUM_TILE - 1) / NUM_TILE, 1), NUM_TPB, 0, s>>>(
-        A->nnz, A->jmap, A->perm, v, mode, A->val);
+  // slices a tile holds, where every tile of so many fits (their largest
+  // counts are the shape's)
+  const int32_t per =
+      A->sell_val && A->slice_max_nnz > 0
+          ? (int32_t)std::min<int64_t>(NUM_SLICES, std::min<int64_t>(NUM_NZ / A->slice_max_nnz,
+                                                                     NUM_E / A->slice_max_coo))
+          : 0;
+  if (per >= 1) {
+    const int e_cap = per * A->slice_max_coo, nz_cap = per * A->slice_max_nnz;
+    k_numeric_slices<<<(unsigned)((A->nslices + per - 1) / per), NUM_TPB,
+                       num_shared(e_cap, nz_cap), s>>>(
+        A->nslices, per, e_cap, nz_cap, A->sell_row0, A->row_ptr, A->jmap, A->perm, v, mode, A->val,
+        A->diag_pos, A->dinv, A->sell_ptr, A->sell_npat ? A->sell_mask : nullptr, A->sell_val);
     GBS_LAUNCHED(1);
+  } else {
+    if (A->nnz > 0) {
+      k_coo_numeric<<<grid_for((A->nnz + NUM_TILE - 1) / NUM_TILE, 1), NUM_TPB,
+                      num_shared(NUM_E, NUM_TILE), s>>>(
+          A->nnz, A->jmap, A->perm, v, mode, A->val);
+      GBS_LAUNCHED(1);
+    }
+    if (A->nrows > 0) {
+      k_jacobi<<<grid_for(A->nrows, 256), 256, 0, s>>>(A->nrows, A->diag_pos, A->val, A->dinv);
+      GBS_LAUNCHED(1);
+    }
+    GBS_TRY(sell_values(A, s));
   }
-  if (A->nrows > 0) {
-    k_jacobi<<<grid_for(A->nrows, 256), 256, 0, s>>>(A->nrows, A->diag_pos, A->val, A->dinv);
-    GBS_LAUNCHED(1);
-  }
-  GBS_TRY(sell_values(A, s));
   A->values_set = true;
   A->val32_valid = false;
   A->values_version += 1;
@@ -1124,7 +1478,8 @@ __global__ void k_vec_scatter(int64_t n, const int32_t *__restrict__ row_ptr,
 // numeric kernel, INSERT into val), then the scatter into y.
 int launch_vec_set_values(gbs_mat A, const double *v, int mode, double *y, cudaStream_t s) {
   if (A->nnz > 0) {
-    k_coo_numeric<<<grid_for((A->nnz + NUM_TILE - 1) / NUM_TILE, 1), NUM_TPB, 0, s>>>(
+    k_coo_numeric<<<grid_for((A->nnz + NUM_TILE - 1) / NUM_TILE, 1), NUM_TPB,
+                      num_shared(NUM_E, NUM_TILE), s>>>(
         A->nnz, A->jmap, A->perm, v, GBS_INSERT, A->val);
     GBS_LAUNCHED(1);
   }

@@ -162,7 +162,6 @@ struct gbs_mat_s {
   int device = 0;
   int64_t nrows = 0, ncols = 0, ncoo = 0, nkept = 0, nnz = 0;
   int32_t nsys = 1;
-  int32_t max_row_nnz = 0;
   int32_t col_span = 0;         // largest |col - row| of the pattern (capped at 2^30)
   bool batched = false;
   bool values_set = false;
@@ -179,7 +178,6 @@ struct gbs_mat_s {
 
   // systems (host + device)
   std::vector<int64_t> row_off_h;  // nsys + 1
-  std::vector<int32_t> max_row_sys_h;
 
   // sliced-ELL copy used by the row products (sell.cu), built on demand
   int64_t nslices = 0, sell_nnz = 0;
@@ -193,6 +191,7 @@ struct gbs_mat_s {
   int32_t *sell_pat = nullptr;     // nslices: first offset of each slice's pattern in sell_pool
   int32_t *sell_pool = nullptr;    // the patterns' offsets col - row
   uint32_t *sell_mask = nullptr;   // 32 nslices: pattern entries each row holds
+  int32_t slice_max_nnz = 0, slice_max_coo = 0;  // largest nonzeros / COO entries of a slice
   int64_t sell_npat = 0;           // slices with a pattern (0 or nslices)
   int64_t sell_nnz_rows = 0;       // 32 x the slices' longest rows (the size without
                                    // patterns: the automatic plan's padding rule)
@@ -273,6 +272,11 @@ int launch_vec_set_values(gbs_mat A, const double *v, int mode, double *y, cudaS
 int launch_to_fp32(gbs_mat A, cudaStream_t s);
 int launch_adjoint_scatter(gbs_mat A, const double *lambda, const double *x,
                            double *dLda, double *dLdv, cudaStream_t s);
+// Exclusive scan of n uint32 on s (in may equal out; tmp: scan_tmp_words(n)
+// words; the total to *total on the device when non-null).
+int exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_t *tmp, uint32_t *total,
+                   cudaStream_t s);
+int64_t scan_tmp_words(int64_t n);
 int symbolic(gbs_mat A, const int32_t *i, const int32_t *j, const int64_t *coo_off_h,
              cudaStream_t s);
 int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,

@@ -26,7 +26,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <mutex>
+#include <utility>
 
 #include "device_util.cuh"
 #include "internal.cuh"
@@ -134,7 +136,20 @@ static PhaseKernels phase_kernels(bool refined, int lanes, bool wide = false) {
 // CTAs per SM that fit at once for the kernels walking the SpMV table (setup,
 // A, final) and the update table (B, C), FP64 and refined, for the plan's
 // row-product kernel.
+// The answers depend on the compiled kernels and the device alone: each is
+// asked for once (ten driver calls, 30 us of every plan).
 int phase_occupancy(int lanes, int *rows, int *upd) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, std::pair<int, int>> known;
+  int dev = 0;
+  GBS_TRY_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(mu);
+  const auto at = known.find({dev, lanes});
+  if (at != known.end()) {
+    *rows = at->second.first;
+    *upd = at->second.second;
+    return GBS_OK;
+  }
   const PhaseKernels K[2] = {phase_kernels(false, lanes), phase_kernels(true, lanes)};
   int r = 1 << 20, u = 1 << 20;
   for (const PhaseKernels &k : K) {
@@ -151,6 +166,7 @@ int phase_occupancy(int lanes, int *rows, int *upd) {
   }
   *rows = std::max(r, 1);
   *upd = std::max(u, 1);
+  known[{dev, lanes}] = {*rows, *upd};
   return GBS_OK;
 }
 

@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 #include <vector>
 
 #include "device_util.cuh"
@@ -67,24 +68,94 @@ __device__ int slice_union(const int32_t *__restrict__ col, int32_t r, int32_t j
   return n;
 }
 
-// One warp per slice: w[s] = its longest row; u[s] = the size of its rows'
-// offset union (33: more than 32, or patterns not built).
-__global__ void k_slice_shape(int64_t nslices, const int32_t *__restrict__ srow0,
-                              const int32_t *__restrict__ row_ptr,
-                              const int32_t *__restrict__ col, int32_t patterns,
-                              int32_t *__restrict__ w, int32_t *__restrict__ u) {
-  const int lane = threadIdx.x & 31;
+// Sums over all slices, read back once: they decide patterns and sizes.
+struct ShapeSums {
+  unsigned long long w, u;  // longest rows; offset unions (33 at most each)
+  int32_t over;             // a slice's union has more than 32 offsets
+  int32_t nnz, coo;         // largest nonzeros and COO entries of a slice
+  int32_t pad;
+};
+
+// One warp per slice: its first row (a batch's slices start at their system's
+// first row: sys holds nsys + 1 first rows, then nsys + 1 first slices), w[s] =
+// its longest row, u[s] = the size of its rows' offset union (33: more than
+// 32, or patterns not built); their sums over all slices.
+constexpr int SHAPE_TPB = 256;
+__global__ void __launch_bounds__(SHAPE_TPB)
+    k_slice_shape(int64_t nslices, int64_t nrows, int32_t nsys, const int32_t *__restrict__ sys,
+                  const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
+                  const int32_t *__restrict__ jmap, int32_t patterns,
+                  int32_t *__restrict__ srow0, uint32_t *__restrict__ w,
+                  uint32_t *__restrict__ u, ShapeSums *sums) {
+  __shared__ unsigned long long sw[SHAPE_TPB / 32], su[SHAPE_TPB / 32];
+  __shared__ int32_t sn[SHAPE_TPB / 32], se[SHAPE_TPB / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  unsigned long long tw = 0, tu = 0;
+  int32_t nz = 0, ne = 0;
+  bool over = false;
   for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices; s += nw) {
-    const int32_t r = srow0[s] + lane;
-    const bool live = r < srow0[s + 1];
+    int64_t r0 = 32 * s, r1 = nrows;
+    if (sys) {
+      int lo = 0, hi = nsys;  // the last system whose first slice is <= s
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(sys + nsys + 1 + mid) <= s) lo = mid;
+        else hi = mid;
+      }
+      r0 = __ldg(sys + lo) + 32 * (s - __ldg(sys + nsys + 1 + lo));
+      r1 = __ldg(sys + lo + 1);
+    }
+    const int64_t r = r0 + lane;
+    const bool live = r < r1;
     const int32_t rs = live ? row_ptr[r] : 0, re = live ? row_ptr[r + 1] : 0;
     const int32_t m = __reduce_max_sync(0xffffffffu, re - rs);
-    const int n = patterns ? slice_union(col, r, rs, re, lane, nullptr, nullptr) : 33;
+    const int n = patterns ? slice_union(col, (int32_t)r, rs, re, lane, nullptr, nullptr) : 33;
     if (lane == 0) {
-      w[s] = m;
-      u[s] = n;
+      srow0[s] = (int32_t)r0;
+      if (s == nslices - 1) srow0[nslices] = (int32_t)nrows;
+      w[s] = (uint32_t)m;
+      u[s] = (uint32_t)n;
     }
+    const int64_t rl = r0 + 32 < r1 ? r0 + 32 : r1;
+    const int32_t a = row_ptr[r0], b = row_ptr[rl];
+    nz = max(nz, b - a);
+    ne = max(ne, jmap[b] - jmap[a]);
+    tw += (unsigned long long)m;
+    tu += (unsigned long long)n;
+    over = over || n > 32;
+  }
+  if (lane == 0) {
+    sw[warp] = tw;
+    su[warp] = tu;
+    sn[warp] = nz;
+    se[warp] = ne;
+    if (over) sums->over = 1;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < SHAPE_TPB / 32; ++k) {
+      tw += sw[k];
+      tu += su[k];
+      nz = max(nz, sn[k]);
+      ne = max(ne, se[k]);
+    }
+    atomicAdd(&sums->w, tw);
+    atomicAdd(&sums->u, tu);
+    if (nz > *(volatile int32_t *)&sums->nnz) atomicMax(&sums->nnz, nz);
+    if (ne > *(volatile int32_t *)&sums->coo) atomicMax(&sums->coo, ne);
+  }
+}
+
+// Entries (size[s]) and, with patterns, pool words (even) of each slice, for
+// the scans that turn them into starts; one word beyond the last is 0.
+__global__ void k_slice_sizes(int64_t nslices, const uint32_t *__restrict__ width,
+                              uint32_t *__restrict__ size, uint32_t *__restrict__ pool) {
+  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s <= nslices;
+       s += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t k = s < nslices ? width[s] : 0u;
+    size[s] = 32u * k;
+    if (pool) pool[s] = (k + 1u) & ~1u;
   }
 }
 
@@ -170,75 +241,85 @@ void free_sell(gbs_mat A) {
 
 // Slice table, column patterns chosen and padded size (no entries yet); when
 // the padded size reaches 2^31 only the size is recorded.  Idempotent.
-// Synchronises s once (the slice widths decide the sizes).
+// Synchronises s once: the sums over the slices decide the sizes (the tables
+// themselves stay on the device).
 int sell_shape(gbs_mat A, cudaStream_t st) {
   if (A->sell_row0) return GBS_OK;
-  std::vector<int32_t> srow0;
-  for (int32_t q = 0; q < A->nsys; ++q)
-    for (int64_t r = A->row_off_h[q]; r < A->row_off_h[q + 1]; r += 32) srow0.push_back((int32_t)r);
-  const int64_t ns = (int64_t)srow0.size();
-  srow0.push_back((int32_t)A->nrows);
-  std::vector<int32_t> w(std::max<int64_t>(ns, 1), 0), u(std::max<int64_t>(ns, 1), 33);
-  GBS_TRY(dev_alloc(&A->sell_row0, ns + 1, st));
-  GBS_TRY_CUDA(cudaMemcpyAsync(A->sell_row0, srow0.data(), sizeof(int32_t) * (ns + 1),
-                               cudaMemcpyHostToDevice, st));
-  if (ns > 0) {
-    int32_t *dw = nullptr;
-    GBS_TRY(dev_alloc(&dw, 2 * ns, st));
-    k_slice_shape<<<grid_of(ns * 32, 256), 256, 0, st>>>(
-        ns, A->sell_row0, A->row_ptr, A->col, A->sell_patterns ? 1 : 0, dw, dw + ns);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(w.data(), dw, sizeof(int32_t) * ns, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(u.data(), dw + ns, sizeof(int32_t) * ns, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    dev_free(dw, st);
-    count_launches(1);
-    GBS_TRY_CUDA(e);
-  }
-  // patterns when every slice has at most 32 offsets and they add at most a
-  // quarter to the entries; pattern starts are even (pair loads)
-  int64_t sum_w = 0, sum_u = 0;
-  bool fit = A->sell_patterns && ns > 0;
-  for (int64_t s = 0; s < ns; ++s) {
-    sum_w += w[s];
-    sum_u += u[s];
-    fit = fit && u[s] <= 32;
-  }
-  fit = fit && 4 * sum_u <= 5 * sum_w;
-  std::vector<int32_t> pat(std::max<int64_t>(ns, 1), 0);
-  int64_t total = 0, pool_n = 0;
-  for (int64_t s = 0; s < ns; ++s) {
-    if (fit) {
-      pat[s] = (int32_t)pool_n;
-      pool_n += (u[s] + 1) & ~1;
-      w[s] = u[s];
-    }
-    total += 32 * (int64_t)w[s];
-  }
-  const int64_t npat = fit ? ns : 0;
-  A->sell_nnz_rows = 32 * sum_w;
-  A->nslices = ns;
-  A->sell_nnz = total;
-  if (total > 2147483647LL) return GBS_OK;  // too large for 32-bit offsets: no copy
-  std::vector<int32_t> sptr(ns + 1, 0);
-  for (int64_t s = 0; s < ns; ++s) sptr[s + 1] = sptr[s] + 32 * w[s];
-  GBS_TRY(dev_alloc(&A->sell_ptr, ns + 1, st));
-  GBS_TRY_CUDA(cudaMemcpyAsync(A->sell_ptr, sptr.data(), sizeof(int32_t) * (ns + 1),
-                               cudaMemcpyHostToDevice, st));
-  if (npat > 0) {
-    GBS_TRY(dev_alloc(&A->sell_pat, ns, st));
-    GBS_TRY(dev_alloc(&A->sell_pool, std::max<int64_t>(pool_n, 2), st));
-    GBS_TRY(dev_alloc(&A->sell_mask, 32 * ns, st));
-    GBS_TRY_CUDA(cudaMemcpyAsync(A->sell_pat, pat.data(), sizeof(int32_t) * ns,
-                                 cudaMemcpyHostToDevice, st));
-  }
-  A->sell_npat = npat;
   A->sell_slice0_h.assign(A->nsys + 1, 0);
   for (int32_t q = 0; q < A->nsys; ++q)
     A->sell_slice0_h[q + 1] =
         A->sell_slice0_h[q] + (int32_t)((A->row_off_h[q + 1] - A->row_off_h[q] + 31) / 32);
+  const int64_t ns = A->sell_slice0_h[A->nsys];
+  ShapeSums h;
+  memset(&h, 0, sizeof(h));
+  // w, u (ns + 1 words each, 16-byte aligned), the sums, a batch's first rows and slices
+  const int64_t pad = (ns + 4) & ~(int64_t)3, nsy = A->nsys > 1 ? 2 * (A->nsys + 1) : 0;
+  uint32_t *d = nullptr;
+  int32_t *row0 = nullptr;
+  GBS_TRY(dev_alloc(&row0, ns + 1, st));
+  if (ns == 0) {
+    const int32_t end = (int32_t)A->nrows;
+    GBS_TRY_CUDA(cudaMemcpyAsync(row0, &end, sizeof(end), cudaMemcpyHostToDevice, st));
+  }
+  struct Scratch {  // returned to the pool on every exit path
+    uint32_t *p = nullptr;
+    cudaStream_t s;
+    ~Scratch() { dev_free(p, s); }
+  } scratch{nullptr, st};
+  GBS_TRY(dev_alloc(&scratch.p, 2 * pad + (int64_t)sizeof(ShapeSums) / 4 + nsy, st));
+  d = scratch.p;
+  uint32_t *w = d, *u = d + pad;
+  ShapeSums *sums = reinterpret_cast<ShapeSums *>(d + 2 * pad);
+  int32_t *sys = nsy ? reinterpret_cast<int32_t *>(sums + 1) : nullptr;
+  A->sell_row0 = row0;
+  if (ns > 0) {
+    GBS_TRY_CUDA(cudaMemsetAsync(sums, 0, sizeof(ShapeSums), st));
+    if (sys) {
+      std::vector<int32_t> t(nsy);
+      for (int32_t q = 0; q <= A->nsys; ++q) {
+        t[q] = (int32_t)A->row_off_h[q];
+        t[A->nsys + 1 + q] = A->sell_slice0_h[q];
+      }
+      GBS_TRY_CUDA(cudaMemcpyAsync(sys, t.data(), sizeof(int32_t) * nsy, cudaMemcpyHostToDevice,
+                                   st));
+    }
+    k_slice_shape<<<grid_of(ns * 32, SHAPE_TPB), SHAPE_TPB, 0, st>>>(
+        ns, A->nrows, A->nsys, sys, A->row_ptr, A->col, A->jmap, A->sell_patterns ? 1 : 0,
+        row0, w, u, sums);
+    GBS_LAUNCHED(1);
+    GBS_TRY_CUDA(cudaMemcpyAsync(&h, sums, sizeof(h), cudaMemcpyDeviceToHost, st));
+    GBS_TRY_CUDA(cudaStreamSynchronize(st));
+  }
+  // patterns when every slice has at most 32 offsets and they add at most a
+  // quarter to the entries; pattern starts are even (pair loads)
+  const bool fit = A->sell_patterns && ns > 0 && !h.over && 4 * h.u <= 5 * h.w;
+  const int64_t total = 32 * (int64_t)(fit ? h.u : h.w);
+  A->sell_nnz_rows = 32 * (int64_t)h.w;
+  A->slice_max_nnz = h.nnz;
+  A->slice_max_coo = h.coo;
+  A->nslices = ns;
+  A->sell_nnz = total;
+  if (total > 2147483647LL) return GBS_OK;  // too large for 32-bit offsets: no copy
+  GBS_TRY(dev_alloc(&A->sell_ptr, ns + 1, st));
+  if (ns > 0) {
+    uint32_t *tmp = nullptr;
+    GBS_TRY(dev_alloc(&tmp, scan_tmp_words(ns + 1), st));
+    struct Scratch tmp_free {tmp, st};
+    if (fit) {
+      GBS_TRY(dev_alloc(&A->sell_pat, ns + 1, st));
+      GBS_TRY(dev_alloc(&A->sell_pool, h.u + ns + 2, st));  // (each start rounded up to even)
+      GBS_TRY(dev_alloc(&A->sell_mask, 32 * ns, st));
+    }
+    uint32_t *ptr = reinterpret_cast<uint32_t *>(A->sell_ptr);
+    uint32_t *pat = reinterpret_cast<uint32_t *>(A->sell_pat);
+    k_slice_sizes<<<grid_of(ns + 1, 256), 256, 0, st>>>(ns, fit ? u : w, ptr, pat);
+    GBS_LAUNCHED(1);
+    GBS_TRY(exclusive_scan(ptr, ptr, ns + 1, tmp, nullptr, st));
+    if (fit) GBS_TRY(exclusive_scan(pat, pat, ns + 1, tmp, nullptr, st));
+  } else {
+    GBS_TRY_CUDA(cudaMemsetAsync(A->sell_ptr, 0, sizeof(int32_t), st));
+  }
+  A->sell_npat = fit ? ns : 0;
   return GBS_OK;
 }
 

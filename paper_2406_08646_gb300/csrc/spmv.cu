@@ -266,6 +266,10 @@ static int build_cta_order(gbs_mat A, cudaStream_t st) {
     return A->row_off_h[u + 1] - A->row_off_h[u] > A->row_off_h[v + 1] - A->row_off_h[v];
   });
   if (!A->cta_order) GBS_TRY(dev_alloc(&A->cta_order, A->nsys, st));
+  if (A->nsys == 1) {
+    GBS_TRY_CUDA(cudaMemsetAsync(A->cta_order, 0, sizeof(int32_t), st));
+    return GBS_OK;
+  }
   GBS_TRY_CUDA(cudaMemcpyAsync(A->cta_order, ord.data(), sizeof(int32_t) * A->nsys,
                                cudaMemcpyHostToDevice, st));
   GBS_TRY_CUDA(cudaStreamSynchronize(st));  // ord is a local vector
