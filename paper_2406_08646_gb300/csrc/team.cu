@@ -227,8 +227,12 @@ struct Team {
 template <bool GRID, bool SM, bool WIN>
 __device__ __forceinline__ void team_pcg(const PcgArgs &a, Team<GRID> &tm, bool timers) {
   TeamShared &sh = tm.sh;
-  const TeamPart &g = sh.g;
+  // The element-wise passes copy the pointers they use: read through sh, every
+  // store of the pass might change them, and each row would load them again.
+  // (The streaming row products leave them there: their loads in flight take
+  // the registers.)
   const TeamVecs &V = sh.V;
+  const TeamPart &g = sh.g;
   const CallArgs &C = sh.call;
   const double *b = C.b;
   double *xg = C.x;
@@ -248,7 +252,8 @@ __device__ __forceinline__ void team_pcg(const PcgArgs &a, Team<GRID> &tm, bool 
   auto rows = [&](auto gather, const double *v, auto &f) {
     constexpr int NC = decltype(gather)::value;
     if constexpr (SM) {
-      sell_rows<double, false, NC, true, 2>(sh.sv, sh.sval, v, g.s0, g.s1, f);
+      const SellView sv = sh.sv;
+      sell_rows<double, false, NC, true, 2>(sv, sh.sval, v, g.s0, g.s1, f);
     } else {
       if (a.stream_matrix) sell_rows<double, true, NC, false, 4>(a.sv, a.sval, v, g.s0, g.s1, f);
       else sell_rows<double, false, NC, false, 4>(a.sv, a.sval, v, g.s0, g.s1, f);
@@ -256,60 +261,66 @@ __device__ __forceinline__ void team_pcg(const PcgArgs &a, Team<GRID> &tm, bool 
   };
   std::integral_constant<int, GATHER_CA> from_global;
   std::integral_constant<int, WIN ? GATHER_SM : GATHER_CA> from_p;
-  auto p_at = [&](int i) -> double {
-    if constexpr (WIN) return V.p[i];
-    else return __ldca(V.p + i);
+  auto p_at = [](const double *p, int i) -> double {
+    if constexpr (WIN) return p[i];
+    else return __ldca(p + i);
   };
-  // z of an own row: kept, and handed to the CTAs that hold the row in their halos
-  auto put_z = [&](int i, double z) {
-    V.z[i] = z;
+  // z of an own row, handed to the CTAs that hold the row in their halos
+  auto hand_z = [&](double *zown, double *zg, int i, double z) {
     if constexpr (WIN && GRID) {
-      if (V.z != V.zg) V.zg[i] = z;
+      if (zown != zg) zg[i] = z;
     } else if constexpr (WIN) {
-      for (int d = g.dlo; d <= g.dhi; ++d)
+      for (int d = g.dlo, e = g.dhi; d <= e; ++d)
         if (i >= sh.lo[d] && i < sh.hi[d]) st_remote(sh.to[d] + 8u * (uint32_t)i, z);
     }
   };
   // p = z (+ beta p), over the window or the own rows
   auto direction = [&](bool first, double be) {
     constexpr int U = 2;
+    double *const p = V.p;
+    const double *const z = V.z, *const zg = V.zg, *const zh = V.zh;
     double pv[U], zv[U];
     auto ld = [&](int i, int k) {
-      pv[k] = first ? 0.0 : p_at(i);
-      zv[k] = V.z[i];
+      pv[k] = first ? 0.0 : p_at(p, i);
+      zv[k] = z[i];
     };
-    auto use = [&](int i, int k) { V.p[i] = first ? zv[k] : fma(be, pv[k], zv[k]); };
-    cta_rows_by<U>(g.r0, g.r1, ld, use);
+    auto use = [&](int i, int k) { p[i] = first ? zv[k] : fma(be, pv[k], zv[k]); };
+    const int r0 = g.r0, r1 = g.r1;
+    cta_rows_by<U>(r0, r1, ld, use);
     if constexpr (WIN) {
-      const int nlo = g.r0 - g.w0, nh = nlo + g.w1 - g.r1;
+      const int w0 = g.w0, nlo = r0 - w0, nh = nlo + g.w1 - r1;
       for (int h = threadIdx.x; h < nh; h += blockDim.x) {
-        const int i = h < nlo ? g.w0 + h : g.r1 + (h - nlo);
-        const double z = GRID ? __ldcg(V.zg + i) : V.zh[h];
-        V.p[i] = first ? z : fma(be, V.p[i], z);
+        const int i = h < nlo ? w0 + h : r1 + (h - nlo);
+        const double zi = GRID ? __ldcg(zg + i) : zh[h];
+        p[i] = first ? zi : fma(be, p[i], zi);
       }
       __syncthreads();
     }
   };
   // setup: r = b - A x0, z = D^-1 r; r.z, r.r, then b.b, missing diagonals
   double u[2] = {0.0, 0.0}, w[2] = {0.0, 0.0};
-  auto start = [&](int i, double t) {
-    const double bv = b[i], rv = bv - t, d = a.dinv[i], z = d * rv;
-    if (V.dv != a.dinv) V.dv[i] = d;
-    V.r[i] = rv;
-    put_z(i, z);
-    u[0] = fma(rv, z, u[0]);
-    u[1] = fma(rv, rv, u[1]);
-    w[0] = fma(bv, bv, w[0]);
-    w[1] += (d == 0.0) ? 1.0 : 0.0;
-  };
-  if (C.nonzero_guess) {
-    if (V.x != xg)
-      for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) V.x[i] = xg[i];
-    rows(from_global, xg, start);
-  } else {
-    for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) {
-      V.x[i] = 0.0;
-      start(i, 0.0);
+  {
+    double *const r = V.r, *const z = V.z, *const zg = V.zg, *const dv = V.dv, *const x = V.x;
+    auto start = [&](int i, double t) {
+      const double bv = b[i], rv = bv - t, d = a.dinv[i], zv = d * rv;
+      if (dv != a.dinv) dv[i] = d;
+      r[i] = rv;
+      z[i] = zv;
+      hand_z(z, zg, i, zv);
+      u[0] = fma(rv, zv, u[0]);
+      u[1] = fma(rv, rv, u[1]);
+      w[0] = fma(bv, bv, w[0]);
+      w[1] += (d == 0.0) ? 1.0 : 0.0;
+    };
+    if (C.nonzero_guess) {
+      if (x != xg)
+        for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) x[i] = xg[i];
+      rows(from_global, xg, start);
+    } else {
+      for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) {
+        x[i] = 0.0;
+        start(i, 0.0);
+      }
     }
   }
   tm.template sum<2>(u);
@@ -344,11 +355,20 @@ __device__ __forceinline__ void team_pcg(const PcgArgs &a, Team<GRID> &tm, bool 
   while (go) {
     // q = A p, p.q -> alpha
     double pq[1] = {0.0};
-    auto fa = [&](int i, double y) {
-      V.q[i] = y;
-      pq[0] = fma(p_at(i), y, pq[0]);
-    };
-    rows(from_p, V.p, fa);
+    {
+      double *const ql = V.q;
+      const double *const pl = V.p;
+      auto fa = [&](int i, double y) {
+        if constexpr (SM) {
+          ql[i] = y;
+          pq[0] = fma(p_at(pl, i), y, pq[0]);
+        } else {
+          V.q[i] = y;
+          pq[0] = fma(p_at(V.p, i), y, pq[0]);
+        }
+      };
+      rows(from_p, pl, fa);
+    }
     tm.template sum<1>(pq);
     if (t0) {
       int status = -1;
@@ -363,27 +383,33 @@ __device__ __forceinline__ void team_pcg(const PcgArgs &a, Team<GRID> &tm, bool 
     if (sh.ipub[0] >= 0 || tm.aborted()) break;
     const double al = sh.pub[0];
     // x += alpha p, r -= alpha q, z = D^-1 r, r.z, r.r -> tests, beta
-    u[0] = u[1] = 0.0;
     {
       constexpr int U = 2;
+      const double *const q = V.q, *const p = V.p, *const dv = V.dv;
+      double *const r = V.r, *const z = V.z, *const zg = V.zg, *const x = V.x;
+      double rz = 0.0, rr = 0.0;
       double qv[U], rv0[U], d[U], pv[U], xv[U];
       auto ld = [&](int i, int k) {
-        qv[k] = V.q[i];
-        rv0[k] = V.r[i];
-        d[k] = V.dv[i];
-        pv[k] = p_at(i);
-        xv[k] = V.x[i];
+        qv[k] = q[i];
+        rv0[k] = r[i];
+        d[k] = dv[i];
+        pv[k] = p_at(p, i);
+        xv[k] = x[i];
       };
       auto use = [&](int i, int k) {
         const double rv = fma(-al, qv[k], rv0[k]);
-        const double z = d[k] * rv;
-        V.x[i] = fma(al, pv[k], xv[k]);
-        V.r[i] = rv;
-        put_z(i, z);
-        u[0] = fma(rv, z, u[0]);
-        u[1] = fma(rv, rv, u[1]);
+        const double zv = d[k] * rv;
+        x[i] = fma(al, pv[k], xv[k]);
+        r[i] = rv;
+        z[i] = zv;
+        hand_z(z, zg, i, zv);
+        rz = fma(rv, zv, rz);
+        rr = fma(rv, rv, rr);
       };
-      cta_rows_by<U>(g.r0, g.r1, ld, use);
+      const int r0 = g.r0, r1 = g.r1;
+      cta_rows_by<U>(r0, r1, ld, use);
+      u[0] = rz;
+      u[1] = rr;
     }
     // the time limit is the lead's clock: its verdict goes round with the sums
     double late[1] = {0.0};
@@ -418,8 +444,8 @@ __device__ __forceinline__ void team_pcg(const PcgArgs &a, Team<GRID> &tm, bool 
     mark(3);
   }
   // x out, then ||b - A x||^2 (x = 0 where b = 0)
-  if (zero_x || V.x != xg)
-    for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) xg[i] = zero_x ? 0.0 : V.x[i];
+  if (const double *const x = V.x; zero_x || x != xg)
+    for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) xg[i] = zero_x ? 0.0 : x[i];
   if (!tm.aborted()) tm.barrier();
   double tt[1] = {0.0};
   auto ft = [&](int i, double t) {
@@ -430,7 +456,7 @@ __device__ __forceinline__ void team_pcg(const PcgArgs &a, Team<GRID> &tm, bool 
   if (!tm.aborted()) tm.template sum<1>(tt);
   if (lead && t0) {
     const bool stopped = sh.timed || tm.aborted();
-    SysState &O = a.st[g.s];
+    SysState &O = a.st[sh.g.s];
     memset(&O, 0, sizeof(SysState));
     O.bb = S.bb;
     O.rnorm0 = S.rnorm0;
@@ -679,7 +705,7 @@ static TeamShape team_shape(gbs_mat A) {
     // the matrix streams past: every thread the registers allow, to have loads
     // in flight (2D 1024^2, us an iteration: 1024 threads 35.1, 512 40.3), and
     // p gathered through L1 rather than from windows (35.1 against 36.9)
-    T.tpb = 1024;
+    if (!T.cluster) T.tpb = 1024;
     c.nvec = (int32_t)std::min<int64_t>(4, TEAM_L1_SMEM / (8 * rows));
   }
   T.smem = (size_t)(16 * T.tpb + 8 * (c.win_cap + c.zh_cap) + c.nvec * 8 * rows + c.mat_cap);
@@ -697,8 +723,7 @@ int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, cudaStr
   T.cfg.slots = A->part;
   T.cfg.ctr = reinterpret_cast<unsigned *>(&A->ctl->queue);
   void (*const kernel)(PcgArgs, TeamCfg) =
-      T.tpb <= 512 ? (T.cluster ? k_team<false, 512> : k_team<true, 512>)
-                   : (T.cluster ? k_team<false, 1024> : k_team<true, 1024>);
+      T.cluster ? k_team<false, 512> : T.tpb <= 512 ? k_team<true, 512> : k_team<true, 1024>;
   GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)TEAM_SMEM));
   cudaLaunchConfig_t lc = {};
