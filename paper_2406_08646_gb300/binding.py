@@ -139,13 +139,24 @@ def _check(status: int):
         raise GbsError(status, last_error())
 
 
-def _stream(stream) -> ctypes.c_void_p:
+try:  # the current stream's handle without a Stream object around it
+    from torch._C import _cuda_getCurrentRawStream as _raw_stream, _cuda_getDevice as _device
+except ImportError:  # pragma: no cover - a torch without the raw calls
+    _raw_stream = None
+
+
+def _stream(stream) -> int:
+    """The cudaStream_t of a call as an integer (None: torch's current stream)."""
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(_device())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _dev(t: torch.Tensor | None, dtype, n: int | None = None, name: str = "tensor"):
+    """The device address of a tensor (an integer, which ctypes passes as a void
+    pointer), after the checks every entry point makes."""
     if t is None:
         return None
     if not t.is_cuda:
@@ -156,7 +167,7 @@ def _dev(t: torch.Tensor | None, dtype, n: int | None = None, name: str = "tenso
         raise ValueError(f"{name} must be contiguous")
     if n is not None and t.numel() != n:
         raise ValueError(f"{name} must have {n} elements, got {t.numel()}")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr() or None
 
 
 def make_opts(rtol=1e-8, maxit=-1, precision=FP64, inner_rtol=1e-4, max_outer=30,
@@ -203,8 +214,11 @@ def mat_set_values_coo(A, v: torch.Tensor, mode: int = INSERT, stream=None):
 
 
 def mat_mult(A, x: torch.Tensor, y: torch.Tensor, stream=None):
-    _check(lib().mat_mult(A, _dev(x, torch.float64, None, "x"), _dev(y, torch.float64, None, "y"),
-                          _stream(stream)))
+    # (the smallest products take less time than their call: the checks alone)
+    st = (_lib or lib()).mat_mult(A, _dev(x, torch.float64, None, "x"),
+                                  _dev(y, torch.float64, None, "y"), _stream(stream))
+    if st != OK:
+        _check(st)
 
 
 def ksp_solve_cg(A, b, x, opts: KspOpts | None = None, want_result=True, stream=None):
@@ -460,6 +474,7 @@ class Mat:
     def __init__(self, handle, batched_rows=None):
         self.h = handle
         self.info = mat_get_info(handle)
+        self._nrows = self.info["nrows"]
         self.batched_rows = batched_rows
 
     @classmethod
@@ -487,7 +502,7 @@ class Mat:
 
     def mult(self, x, y=None, stream=None):
         if y is None:
-            y = torch.empty(self.nrows, dtype=torch.float64, device=x.device)
+            y = x.new_empty(self._nrows, dtype=torch.float64)
         mat_mult(self.h, x, y, stream)
         return y
 
