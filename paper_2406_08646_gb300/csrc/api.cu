@@ -94,7 +94,7 @@ void free_handle(gbs_mat A) {
   void *dev[] = {A->row_ptr, A->col, A->val, A->val32, A->perm, A->jmap, A->diag_pos,
                  A->dinv, A->dinv32, A->r, A->p, A->q, A->r32, A->p32, A->q32, A->d32,
                  A->part, A->sys_cnt, A->st, A->ctl, A->call, A->cta_order,
-                 A->kv, A->sys_row0, A->halo_flags};  // sys_slice0 lies inside sys_row0's
+                 A->kv, A->sys_row0, A->halo_flags, A->order_s};  // sys_slice0 lies inside sys_row0's
   for (void *p : dev) dev_free(p, nullptr);
   free_table(A->ta);
   free_table(A->sa);

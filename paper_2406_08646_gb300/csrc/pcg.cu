@@ -286,6 +286,7 @@ PcgArgs make_args(gbs_mat A, bool per_system, bool refined) {
   a.grid_e = A->te.grid;
   a.row_ptr = A->row_ptr;
   a.col = A->col;
+  a.row_order = A->lanes == GBS_SPMV_SELL ? nullptr : A->order_a;
   a.val = A->val;
   a.val32 = A->val32;
   a.sv = sell_view(A);
@@ -616,6 +617,7 @@ int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_sys
       GBS_TRY(ensure_solver_workspace(A, refined, s));  // the split tables' slots
       PcgArgs a = make_args(A, per_system, refined);
       a.ta = view(A->sa);
+      a.row_order = nullptr;  // (table A's)
       a.te = view(A->se);
       a.part_e = A->sa.nslots;
       a.grid_a = A->sa.grid;

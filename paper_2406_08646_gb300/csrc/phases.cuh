@@ -73,6 +73,7 @@ struct PcgArgs {
   int64_t part_e;     // first reduction slot of table te
   int32_t grid_e;     // CTAs of the kernels that walk table te
   const int32_t *row_ptr, *col;
+  const int32_t *row_order;  // CSR-vector row products: table A's rows by length (or null)
   const double *val;
   const float *val32;
   SellView sv;           // sliced-ELL copy (kernels with L == 0)
@@ -447,11 +448,22 @@ __device__ __forceinline__ T transpose_reduce(T (&acc)[L], int li) {
 // lane), and transpose_reduce leaves row base+lane in lane `lane`, so f runs
 // on every lane with coalesced row indices.  L == 32: one row per warp, xor
 // butterfly, f on lane 0.  All lanes reach the shuffles.
-template <typename T, int L, class F>
+// order (may be null): the rows in the order they are dealt to lanes, a
+// permutation within [r0, r1) by length (k_row_order): a warp runs as many FP64
+// steps as the longest of its 32 rows, and on ragged matrices neighbours in
+// length, not in number, waste few of them (rows of 4 to 40 entries, 19 on
+// average: about 40 steps a warp in row order, 20 in length order).
+// AHEAD: the next step's columns and values are loaded before this step's
+// gathers are used, one round trip a step instead of two; it takes registers,
+// which the solves' one-wave phase kernels have to spare (graph of 300k rows,
+// product phase 26.8 us in row order, 24.0 in length order, 22.5 so) and
+// MatMult's many small CTAs do not (28.8, 26.7; 32.6 so).
+template <typename T, int L, bool AHEAD, class F>
 __device__ __forceinline__ void csr_rows(const int32_t *__restrict__ row_ptr,
                                          const int32_t *__restrict__ col,
                                          const T *__restrict__ val, const T *__restrict__ x,
-                                         int r0, int r1, F &f) {
+                                         int r0, int r1, const int32_t *__restrict__ order,
+                                         F &f) {
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   if constexpr (L == 32) {
@@ -467,9 +479,10 @@ __device__ __forceinline__ void csr_rows(const int32_t *__restrict__ row_ptr,
   } else {
     const int li = lane & (L - 1), g0 = lane - li;
     for (int base = r0 + warp * 32; base < r1; base += nw * 32) {
-      const int my = base + lane;
+      const int at = base + lane;
+      const int my = order && at < r1 ? __ldg(order + at) : at;  // (at >= r1: none)
       int s = 0, e = 0;
-      if (my < r1) {
+      if (at < r1) {
         s = __ldg(row_ptr + my);
         e = __ldg(row_ptr + my + 1);
       }
@@ -483,22 +496,51 @@ __device__ __forceinline__ void csr_rows(const int32_t *__restrict__ row_ptr,
       T acc[L];
 #pragma unroll
       for (int u = 0; u < L; ++u) acc[u] = T(0);
-      for (int t = 0; t < mxw; t += L) {
-        const int k = t + li;
+      if constexpr (!AHEAD) {
+        for (int t = 0; t < mxw; t += L) {
+          const int k = t + li;
+          int c[L];
+          T v[L];
+#pragma unroll
+          for (int u = 0; u < L; ++u) {
+            const bool ok = k < len[u];
+            c[u] = ok ? __ldg(col + rs[u] + k) : -1;
+            v[u] = ok ? __ldg(val + rs[u] + k) : T(0);
+          }
+#pragma unroll
+          for (int u = 0; u < L; ++u)
+            if (c[u] >= 0) acc[u] = fma_rn(v[u], __ldg(x + c[u]), acc[u]);
+        }
+      } else {
         int c[L];
         T v[L];
 #pragma unroll
         for (int u = 0; u < L; ++u) {
-          const bool ok = k < len[u];
-          c[u] = ok ? __ldg(col + rs[u] + k) : -1;
-          v[u] = ok ? __ldg(val + rs[u] + k) : T(0);
+          const bool ok = li < len[u];
+          c[u] = ok ? __ldg(col + rs[u] + li) : -1;
+          v[u] = ok ? __ldg(val + rs[u] + li) : T(0);
         }
+        for (int t = 0; t < mxw; t += L) {
+          const int k = t + L + li;
+          int cn[L];
+          T vn[L], g[L];
 #pragma unroll
-        for (int u = 0; u < L; ++u)
-          if (c[u] >= 0) acc[u] = fma_rn(v[u], __ldg(x + c[u]), acc[u]);
+          for (int u = 0; u < L; ++u) {
+            g[u] = c[u] >= 0 ? __ldg(x + c[u]) : T(0);
+            const bool ok = k < len[u];
+            cn[u] = ok ? __ldg(col + rs[u] + k) : -1;
+            vn[u] = ok ? __ldg(val + rs[u] + k) : T(0);
+          }
+#pragma unroll
+          for (int u = 0; u < L; ++u) {
+            if (c[u] >= 0) acc[u] = fma_rn(v[u], g[u], acc[u]);
+            c[u] = cn[u];
+            v[u] = vn[u];
+          }
+        }
       }
       const T sum = transpose_reduce<T, L>(acc, li);
-      if (my < r1) f(my, sum);
+      if (at < r1) f(my, sum);
     }
   }
 }
@@ -808,7 +850,7 @@ __device__ __forceinline__ void row_products(const PcgArgs &a, int b, int r0, in
     else
       sell_rows<T, false, GATHER_NC>(a.sv, sell_val, x, s0, s1, f);
   } else
-    csr_rows<T, L>(a.row_ptr, a.col, csr_val, x, r0, r1, f);
+    csr_rows<T, L, true>(a.row_ptr, a.col, csr_val, x, r0, r1, a.row_order, f);
 }
 
 // The convergence threshold thr = rtol ||b_s|| and two bounds of thr^2

@@ -19,16 +19,75 @@ __global__ void __launch_bounds__(PHASE_TPB) k_spmv(const int32_t *__restrict__ 
                                                     const int32_t *__restrict__ col,
                                                     const double *__restrict__ val,
                                                     const double *__restrict__ x,
-                                                    double *__restrict__ y, int32_t n) {
+                                                    double *__restrict__ y, int32_t n,
+                                                      const int32_t *__restrict__ order) {
   auto f = [&](int r, double s) { y[r] = s; };
   for (int64_t r0 = (int64_t)blockIdx.x * SPMV_ROWS; r0 < n;
        r0 += (int64_t)gridDim.x * SPMV_ROWS) {
     const int r1 = (int)(r0 + SPMV_ROWS < n ? r0 + SPMV_ROWS : n);
-    csr_rows<double, L>(row_ptr, col, val, x, (int)r0, r1, f);
+    csr_rows<double, L, false>(row_ptr, col, val, x, (int)r0, r1, order, f);
   }
 }
 
-// y = A x with the sliced-ELL row product (sell_rows), 8 slices per CTA pass.
+// order[r0 .. r1): the rows of [r0, r1) by decreasing length (ties by index),
+// in windows of at most W rows from r0 on -- one CTA a window, a bitonic sort in
+// shared memory.  Windows start at the blocks' first rows (row0, nblocks + 1)
+// or, without blocks, every W rows.
+constexpr int ORDER_W = 1024;
+__global__ void __launch_bounds__(ORDER_W)
+    k_row_order(int32_t nblocks, const int32_t *__restrict__ row0, int32_t n, int32_t W,
+                const int32_t *__restrict__ row_ptr, int32_t *__restrict__ order) {
+  __shared__ uint32_t key[ORDER_W];
+  const int t = (int)threadIdx.x;
+  for (int b = blockIdx.x; b < nblocks; b += gridDim.x) {
+    const int64_t f = row0 ? row0[b] : (int64_t)b * W;
+    const int64_t e = row0 ? row0[b + 1] : (f + W < n ? f + W : n);
+    for (int64_t w = f; w < e; w += W) {
+      const int m = e - w < W ? (int)(e - w) : W;
+      uint32_t k = ~0u;
+      if (t < m) {
+        const int len = row_ptr[w + t + 1] - row_ptr[w + t];
+        k = ((uint32_t)(0x1fffff - min(len, 0x1fffff)) << 10) | (uint32_t)t;
+      }
+      key[t] = k;
+      __syncthreads();
+      for (int s = 2; s <= ORDER_W; s <<= 1)
+        for (int j = s >> 1; j > 0; j >>= 1) {
+          const int q = t ^ j;
+          if (q > t) {
+            const uint32_t u = key[t], v = key[q];
+            if ((u > v) == ((t & s) == 0)) {
+              key[t] = v;
+              key[q] = u;
+            }
+          }
+          __syncthreads();
+        }
+      if (t < m) order[w + t] = (int32_t)(w + (int)(key[t] & 1023u));
+      __syncthreads();
+    }
+  }
+}
+
+// The row orders of a CSR-vector plan (after table A).
+static int build_row_orders(gbs_mat A, cudaStream_t st) {
+  const int64_t n = A->nrows;
+  if (n == 0) return GBS_OK;
+  if (!A->order_s) {
+    GBS_TRY(dev_alloc(&A->order_s, 2 * (size_t)n, st));
+    A->order_a = A->order_s + n;
+    const int32_t nb = (int32_t)((n + SPMV_ROWS - 1) / SPMV_ROWS);
+    k_row_order<<<(unsigned)std::min(nb, 1 << 16), ORDER_W, 0, st>>>(
+        nb, nullptr, (int32_t)n, SPMV_ROWS, A->row_ptr, A->order_s);
+    GBS_LAUNCHED(1);
+  }
+  k_row_order<<<(unsigned)std::min(std::max(A->ta.nblocks, 1), 1 << 16), ORDER_W, 0, st>>>(
+      A->ta.nblocks, A->ta.row0, (int32_t)n, ORDER_W, A->row_ptr, A->order_a);
+  GBS_LAUNCHED(1);
+  return GBS_OK;
+}
+
+// y = A x with the sliced-ELL row product (sell_rows), 16 slices per CTA pass.
 __global__ void __launch_bounds__(PHASE_TPB, SELL_MIN_CTAS)
     k_spmv_sell(const SellView S, const double *__restrict__ sval,
                 const double *__restrict__ x, double *__restrict__ y, int32_t nslices,
@@ -43,26 +102,54 @@ __global__ void __launch_bounds__(PHASE_TPB, SELL_MIN_CTAS)
   }
 }
 
+// The same with 64 registers a thread on a grid of two CTAs an SM, each with
+// its run of slices: sell_rows_deep, which has four pairs a thread and the next
+// slice's tables in flight.  The FP64 pipe bounds both (Q1 96^3: 40 us of FMAs);
+// this one keeps it busier while slices are wide, and costs a little where they
+// are not (their loads are few, and four CTAs an SM overlap more of them).
+// Measured, us a call: Q1 96^3 49.5 -> 47.6, 64^3 20.5 -> 18.5, 3D 7-point 150^3
+// 59.5 -> 56.1, 2D 5-point 1024^2 18.6 -> 19.5: mean widths from DEEP_WIDTH on.
+constexpr int DEEP_CTAS = 2;
+constexpr double DEEP_WIDTH = 6.0;
+__global__ void __launch_bounds__(PHASE_TPB, DEEP_CTAS)
+    k_spmv_sell_deep(const SellView S, const double *__restrict__ sval,
+                     const double *__restrict__ x, double *__restrict__ y, int32_t nslices,
+                     int32_t stream_matrix) {
+  auto f = [&](int r, double s) { y[r] = s; };
+  const int s0 = (int)((int64_t)nslices * blockIdx.x / gridDim.x);
+  const int s1 = (int)((int64_t)nslices * (blockIdx.x + 1) / gridDim.x);
+  if (stream_matrix)
+    sell_rows<double, true, GATHER_NC, false, 4>(S, sval, x, s0, s1, f);
+  else sell_rows<double, false, GATHER_NC, false, 4>(S, sval, x, s0, s1, f);
+}
+
 int launch_spmv(gbs_mat A, const double *x, double *y, cudaStream_t s) {
   if (A->nrows == 0) return GBS_OK;
   const int32_t n = (int32_t)A->nrows;
   if (A->lanes == GBS_SPMV_SELL) {
     GBS_TRY(sell_build(A, s));  // a no-op once built
     const int64_t ns = A->nslices, per = PHASE_TPB / 32;
-    const unsigned grid = (unsigned)std::min<int64_t>((ns + per - 1) / per, 1 << 20);
-    k_spmv_sell<<<grid, PHASE_TPB, 0, s>>>(sell_view(A), A->sell_val, x, y, (int32_t)ns,
-                                           stream_matrix(A, 12));
+    const int64_t ctas = (ns + per - 1) / per, wave = (int64_t)DEEP_CTAS * sm_count(A);
+    // (a full wave at least: fewer slices spread over more CTAs of the other)
+    const bool deep = A->sell_npat > 0 && ctas >= wave &&
+                      (double)A->sell_nnz >= 32.0 * DEEP_WIDTH * (double)ns;
+    if (deep)
+      k_spmv_sell_deep<<<(unsigned)wave, PHASE_TPB, 0, s>>>(
+          sell_view(A), A->sell_val, x, y, (int32_t)ns, stream_matrix(A, 12));
+    else
+      k_spmv_sell<<<(unsigned)std::min<int64_t>(ctas, 1 << 20), PHASE_TPB, 0, s>>>(
+          sell_view(A), A->sell_val, x, y, (int32_t)ns, stream_matrix(A, 12));
     GBS_LAUNCHED(1);
     return GBS_OK;
   }
   const int64_t chunks = (A->nrows + SPMV_ROWS - 1) / SPMV_ROWS;
   const unsigned grid = (unsigned)std::min<int64_t>(chunks, 1 << 20);
   switch (A->lanes) {
-    case 1: k_spmv<1><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n); break;
-    case 2: k_spmv<2><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n); break;
-    case 8: k_spmv<8><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n); break;
-    case 32: k_spmv<32><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n); break;
-    default: k_spmv<4><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n); break;
+    case 1: k_spmv<1><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
+    case 2: k_spmv<2><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
+    case 8: k_spmv<8><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
+    case 32: k_spmv<32><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
+    default: k_spmv<4><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
   }
   GBS_LAUNCHED(1);
   return GBS_OK;
@@ -323,6 +410,7 @@ int build_plan(gbs_mat A, int32_t Ra, int32_t Re, int32_t kernel, int32_t ctas_p
   if (Ra == 0) Ra = auto_rows(cap_a);
   if (Re == 0) Re = auto_rows(cap_e);
   GBS_TRY(build_table(A, Ra, cap_a, A->ta, st));
+  if (kernel != GBS_SPMV_SELL && kernel != 32) GBS_TRY(build_row_orders(A, st));
   halo_window(A, Ra, A->ta);
   GBS_TRY(build_table(A, Re, cap_e, A->te, st));
   GBS_TRY(build_cta_order(A, st));
