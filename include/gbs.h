@@ -420,7 +420,9 @@ int mat_get_plan(gbs_mat A, int32_t *spmv_rows, int32_t *update_rows, int32_t *k
  *     runs FP64 CG (textbook form, no host_loop) as one launch of a team of
  *     CTAs -- a thread-block cluster, or one CTA per SM launched
  *     cooperatively, whose bounded waits (about a second) end the solve with
- *     GBS_ERR_TIMEOUT -- with the same iteration up to reduction order;
+ *     GBS_ERR_TIMEOUT -- with the same iteration up to reduction order; a
+ *     batched solve of fewer than two systems per SM likewise gives each
+ *     system a cluster (systems of up to 163,840 rows), from a queue;
  *     ksp_result.solver names the solver it stands in for, and phase times
  *     are reported as for the phase kernels.
  * ksp_result.solver tells which one ran.  No synchronisation.

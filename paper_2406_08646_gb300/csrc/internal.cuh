@@ -286,7 +286,8 @@ int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_sys
           cudaStream_t s);
 void free_handle(gbs_mat A);
 bool use_team(gbs_mat A, bool per_system, const ksp_opts &o);
-int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, cudaStream_t s, bool *ran);
+int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,
+               cudaStream_t s, bool *ran);
 int solve_krylov(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,
                  cudaStream_t s);
 CallArgs call_args(const double *b, double *x, const ksp_opts &o);

@@ -45,7 +45,8 @@ namespace gbs {
 // to keep HBM busy.  MB = 2: the same kernels for plans that cap the grids at
 // one or two CTAs per SM anyway, with 64 registers a thread (no spills; C2
 // FP64 product phase at two CTAs per SM 62.9 -> 51.9 us per iteration with
-// column patterns).
+// column patterns, 50.7 with four pairs in flight; 2D 1024^2 19.4 against 23.2
+// at four CTAs per SM).
 #define GBS_ROWS_BOUNDS(L, MB) __launch_bounds__(PHASE_TPB, (L) == 0 ? (MB) : 1)
 
 template <bool REFINED, int L, int MB = SELL_MIN_CTAS>
@@ -65,7 +66,7 @@ __global__ void GBS_ROWS_BOUNDS(L, MB) k_pcg_spmv(PcgArgs a) {
   __shared__ double red[RED_SCRATCH1];
   if (!trip_live(a)) return;
   stamp_phase(a, 1);
-  phase_A<REFINED, L>(a, red);
+  phase_A<REFINED, L, MB == 2 ? 4 : 2>(a, red);
 }
 
 template <bool REFINED>
@@ -583,7 +584,7 @@ int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_sys
   }
   if (use_team(A, per_system, o)) {
     bool ran = false;
-    GBS_TRY(solve_team(A, b, x, o, s, &ran));
+    GBS_TRY(solve_team(A, b, x, o, per_system, s, &ran));
     if (ran) {
       A->last_solver = use_cta_solver(A, per_system) ? GBS_SOLVER_CTA : GBS_SOLVER_PHASES;
       return GBS_OK;

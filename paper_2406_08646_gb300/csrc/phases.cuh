@@ -839,16 +839,16 @@ __device__ __forceinline__ void sell_rows(const SellView &S, const T *__restrict
 
 // The row products of block b (rows [r0, r1) of table ta) with the plan's
 // kernel: L == 0 sliced ELL, else CSR-vector with L lanes per row.
-template <typename T, int L, class F>
+template <typename T, int L, int NP = 2, class F>
 __device__ __forceinline__ void row_products(const PcgArgs &a, int b, int r0, int r1,
                                              const T *csr_val, const T *sell_val, const T *x,
                                              F &f) {
   if constexpr (L == 0) {
     const int s0 = __ldg(a.ta.slice0 + b), s1 = blk_slice_end(a.ta, b);
     if (a.stream_matrix)
-      sell_rows<T, true, GATHER_NC>(a.sv, sell_val, x, s0, s1, f);
+      sell_rows<T, true, GATHER_NC, false, NP>(a.sv, sell_val, x, s0, s1, f);
     else
-      sell_rows<T, false, GATHER_NC>(a.sv, sell_val, x, s0, s1, f);
+      sell_rows<T, false, GATHER_NC, false, NP>(a.sv, sell_val, x, s0, s1, f);
   } else
     csr_rows<T, L, true>(a.row_ptr, a.col, csr_val, x, r0, r1, a.row_order, f);
 }
@@ -984,8 +984,9 @@ __device__ __forceinline__ void phase_setup(const PcgArgs &a, double *red) {
 // ------------------------------------------------------------------ phase A
 // FP64: q = A p, p.q -> alpha.  Refined: the FP32 inner product q32 = A32 p32
 // and p32.q32 (M_INNER), or the FP64 outer residual r = b - A x and ||r||
-// with the refinement tests (M_XUPD).
-template <bool REFINED, int L>
+// with the refinement tests (M_XUPD).  NP: pairs an FP64 product keeps in
+// flight (sell_rows; FP32 ones are faster with two at any register count).
+template <bool REFINED, int L, int NP = 2>
 __device__ __forceinline__ void phase_A(const PcgArgs &a, double *red) {
   const CallArgs &C = *a.call;
   auto fin = [&](int s, double(&tot)[1]) {
@@ -1041,7 +1042,7 @@ __device__ __forceinline__ void phase_A(const PcgArgs &a, double *red) {
         a.q[r] = qv;
         pq = fma(__ldg(a.p + r), qv, pq);
       };
-      row_products<double, L>(a, blk, r0, r1, a.val, a.sval, a.p, f);
+      row_products<double, L, NP>(a, blk, r0, r1, a.val, a.sval, a.p, f);
       acc[0] = pq;
     } else if (mode == M_INNER) {
       float pq = 0.0f;

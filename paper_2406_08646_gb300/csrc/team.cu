@@ -92,6 +92,8 @@ struct TeamShared {
   CallArgs call;                            // (global loads would wait on L2: L1 is dropped
                                             // at every meeting)
   unsigned long long ns[5], last;           // phase timers (one thread of rank 0)
+  TeamCfg cfg;                              // batches: this system's layout,
+  int next;                                 //   and the system the cluster solves
 };
 
 __device__ __forceinline__ void cluster_meet() {
@@ -530,37 +532,24 @@ __device__ bool team_cache(const SellView &S, const double *sval, const TeamPart
   return true;
 }
 
+// One system on the CTA's team: lays the CTA's part out in shared memory as c
+// says (the same in every CTA of a cluster, whose halo tables point into one
+// another) and solves.
 template <bool GRID>
-__device__ __forceinline__ void team_body(const PcgArgs &a, const TeamCfg &cfg) {
-  extern __shared__ __align__(16) unsigned char team_smem[];
-  __shared__ TeamShared sh;
-  uint32_t rank, size, cluster = 0, nclusters = 1;
-  if constexpr (GRID) {
-    rank = blockIdx.x;
-    size = gridDim.x;
-  } else {
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
-    asm("mov.u32 %0, %%clusterid.x;" : "=r"(cluster));
-    asm("mov.u32 %0, %%nclusterid.x;" : "=r"(nclusters));
-  }
-  double *red = reinterpret_cast<double *>(team_smem);
-  double *win = red + 2 * blockDim.x, *zh = win + cfg.win_cap, *vec = zh + cfg.zh_cap;
-  unsigned char *mat = reinterpret_cast<unsigned char *>(vec + (size_t)cfg.nvec * cfg.rows_cap);
-  if (threadIdx.x == 0) {
-    sh.abort = 0;
-    sh.call = *a.call;
-  }
-  Team<GRID> tm{(int)rank, (int)size, sh, red, cfg, a.ctl, 0u, 0};
-  const SysRange sys = cta_system(a, 0);
+__device__ __forceinline__ void team_system(const PcgArgs &a, const TeamCfg &c, TeamShared &sh,
+                                            double *red, const SysRange &sys, uint32_t rank,
+                                            uint32_t size, bool timers) {
+  double *win = red + 2 * blockDim.x, *zh = win + c.win_cap, *vec = zh + c.zh_cap;
+  unsigned char *mat = reinterpret_cast<unsigned char *>(vec + (size_t)c.nvec * c.rows_cap);
+  Team<GRID> tm{(int)rank, (int)size, sh, red, c, a.ctl, 0u, 0};
   const int64_t ns = sys.s1 - sys.s0;
   auto part = [&](int k, int &r0, int &r1) {  // rows of the team's CTA k
     r0 = min(sys.r1, sys.r0 + 32 * (int)(ns * k / size));
     r1 = min(sys.r1, sys.r0 + 32 * (int)(ns * (k + 1) / size));
   };
   auto window = [&](int r0, int r1, int &w0, int &w1) {  // (r1 - halo: no overflow)
-    w0 = r0 < r1 ? max(sys.r0, r0 - cfg.halo) : r0;
-    w1 = r0 < r1 ? (sys.r1 - r1 < cfg.halo ? sys.r1 : r1 + cfg.halo) : r1;
+    w0 = r0 < r1 ? max(sys.r0, r0 - c.halo) : r0;
+    w1 = r0 < r1 ? (sys.r1 - r1 < c.halo ? sys.r1 : r1 + c.halo) : r1;
   };
   TeamPart g;
   g.s = sys.s;
@@ -570,9 +559,8 @@ __device__ __forceinline__ void team_body(const PcgArgs &a, const TeamCfg &cfg) 
   window(g.r0, g.r1, g.w0, g.w1);
   g.dlo = 0;
   g.dhi = -1;
-  __syncthreads();  // sh.call
   if constexpr (!GRID) {
-    if (cfg.window) {
+    if (c.window && size > 1) {
       if (threadIdx.x < size) {
         const int d = threadIdx.x;
         int r0, r1, w0, w1;
@@ -592,12 +580,12 @@ __device__ __forceinline__ void team_body(const PcgArgs &a, const TeamCfg &cfg) 
     }
   }
   // q, r, [z,] D^-1, x: without windows z is kept over q
-  const bool w = cfg.window != 0;
+  const bool w = c.window != 0;
   if (threadIdx.x == 0) {
     int k = 0;
     auto home = [&](double *global) {
       const int at = k++;
-      return at < cfg.nvec ? vec + (int64_t)at * cfg.rows_cap - g.r0 : global;
+      return at < c.nvec ? vec + (int64_t)at * c.rows_cap - g.r0 : global;
     };
     TeamVecs &V = sh.V;
     V.q = home(w ? a.p : a.q);
@@ -612,25 +600,118 @@ __device__ __forceinline__ void team_body(const PcgArgs &a, const TeamCfg &cfg) 
   }
   SellView C;
   const double *vals = nullptr;
-  const bool cached = cfg.mat_cap > 0 && team_cache(a.sv, a.sval, g, mat, cfg.mat_cap, C, &vals);
+  const bool cached = c.mat_cap > 0 && team_cache(a.sv, a.sval, g, mat, c.mat_cap, C, &vals);
   if (threadIdx.x == 0 && cached) {
     sh.sv = C;
     sh.sval = vals;
   }
   __syncthreads();
   if (w) {
-    if (cached) team_pcg<GRID, true, true>(a, tm, true);
-    else team_pcg<GRID, false, true>(a, tm, true);
+    if (cached) team_pcg<GRID, true, true>(a, tm, timers);
+    else team_pcg<GRID, false, true>(a, tm, timers);
   } else {
-    if (cached) team_pcg<GRID, true, false>(a, tm, true);
-    else team_pcg<GRID, false, false>(a, tm, true);
+    if (cached) team_pcg<GRID, true, false>(a, tm, timers);
+    else team_pcg<GRID, false, false>(a, tm, timers);
   }
+}
+
+// One system (an ensemble solve).
+template <bool GRID, int TPB>
+__global__ void __launch_bounds__(TPB, 1) k_team(PcgArgs a, const __grid_constant__ TeamCfg cfg) {
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  __shared__ TeamShared sh;
+  uint32_t rank, size;
+  if constexpr (GRID) {
+    rank = blockIdx.x;
+    size = gridDim.x;
+  } else {
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
+  }
+  if (threadIdx.x == 0) {
+    sh.abort = 0;
+    sh.call = *a.call;
+  }
+  __syncthreads();
+  team_system<GRID>(a, cfg, sh, reinterpret_cast<double *>(team_smem), cta_system(a, 0), rank,
+                    size, true);
   if (!GRID && size > 1) cluster_meet();  // no CTA leaves while others may write to its boxes
 }
 
-template <bool GRID, int TPB>
-__global__ void __launch_bounds__(TPB, 1) k_team(PcgArgs a, const __grid_constant__ TeamCfg cfg) {
-  team_body<GRID>(a, cfg);
+// Shared memory of a batch's systems: windows where the halo's work stays
+// below the meeting they save, then as many vectors as fit, then the matrix.
+__device__ __forceinline__ TeamCfg team_layout(int n, int per_rows, int halo, int size,
+                                               int smem) {
+  TeamCfg c;
+  c.window = c.halo = c.win_cap = c.zh_cap = c.mat_cap = 0;
+  c.ctr = nullptr;
+  c.slots = nullptr;
+  c.rows_cap = max(per_rows, 32);
+  int room = smem / 8 - 2 * (int)blockDim.x;  // doubles
+  const int h = min(halo, n), win = (min(n, c.rows_cap + 2 * h) + 31) & ~31;
+  const int zh = (min(2 * h, n) + 31) & ~31;
+  if (2 * h <= max(c.rows_cap, 4096) && win + zh <= room / 2) {
+    c.window = 1;
+    c.halo = h;
+    c.win_cap = win;
+    c.zh_cap = zh;
+    room -= win + zh;
+  }
+  const int nv = c.window ? 5 : 4;
+  c.nvec = min(nv, room / c.rows_cap);
+  if (c.nvec == nv) c.mat_cap = 8 * (room - nv * c.rows_cap) & ~15;
+  return c;
+}
+
+// (Not inlined: what the systems share would be hoisted out of the loop over
+// them and spilled -- 2.6 KB a thread at 64 registers.)
+__device__ __noinline__ void batch_system(const PcgArgs &a, TeamShared &sh, double *red,
+                                          uint32_t rank, uint32_t size) {
+  team_system<false>(a, sh.cfg, sh, red, cta_system(a, sh.next), rank, size, false);
+}
+
+// A batch (FP64 CG, each system on its own): a persistent grid of clusters, each
+// taking system order[cluster], then the next unsolved one from a queue -- the
+// per-CTA solver's scheme with `size` SMs to a system: a batch of fewer systems
+// than SMs leaves none idle, and the largest systems end the batch sooner.
+template <int TPB>
+__global__ void __launch_bounds__(TPB, 1)
+    k_team_batch(const __grid_constant__ PcgArgs a, int32_t halo, int32_t smem) {
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  __shared__ TeamShared sh;
+  uint32_t rank, size, cluster;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(size));
+  asm("mov.u32 %0, %%clusterid.x;" : "=r"(cluster));
+  if (threadIdx.x == 0) {
+    sh.abort = 0;
+    sh.call = *a.call;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) sh.next = (int)cluster;
+  __syncthreads();
+  while (sh.next < a.cta_n) {
+    {
+      const SysRange sys = cta_system(a, sh.next);
+      if (threadIdx.x == 0)
+        sh.cfg = team_layout(sys.r1 - sys.r0, 32 * ((sys.s1 - sys.s0 + (int)size - 1) / (int)size),
+                             halo, (int)size, smem);
+      __syncthreads();
+      batch_system(a, sh, reinterpret_cast<double *>(team_smem), rank, size);
+    }
+    // the next system, from the lead's queue to every CTA of the cluster: after
+    // a meeting, so that no CTA still reads this one, its boxes or its halos
+    cluster_meet();
+    if (rank == 0 && threadIdx.x == 0) {
+      uint32_t nclusters;
+      asm("mov.u32 %0, %%nclusterid.x;" : "=r"(nclusters));
+      const int nx = (int)nclusters + atomicAdd(&a.ctl->queue, 1);
+      for (int d = 0; d < (int)size; ++d)
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(&sh.next, d)), "r"(nx)
+                     : "memory");
+    }
+    cluster_meet();
+  }
 }
 
 // ------------------------------------------------------------------ host side
@@ -649,11 +730,34 @@ constexpr int64_t TEAM_CLUSTER_WORK = 160000;
 // us an iteration on team / phases: 128^3 70.4 / 72.9, 160^3 141.6 / 134.0).
 constexpr int64_t TEAM_GRID_ROWS = 3 << 20;
 
+// CTAs a system of a batch gets: the smallest cluster that gives every SM work
+// and the largest system's CTAs at most TEAM_BATCH_ROWS rows each, so that most
+// of their vectors stay on the SM; 1: the solvers without a team.  (Automatic
+// solver and plan.)  Measured, ms, on edge-diffusion systems, half 2D, half 3D,
+// phase kernels -> clusters: 4 systems of 1k-8k rows 6.0 -> 2.6, 8 of 2k-20k
+// 13.2 -> 8.7, 40 of 500-3k 6.2 -> 3.3, 64 of 1k-20k 32.3 -> 27.7, 100 of 1k-3k
+// 9.5 -> 4.5, 150 of 1k-20k 67.7 -> 49.9, 200 of 5k-20k 96.6 -> 53.3.  From two
+// systems an SM on the per-CTA solver keeps every SM busy with no meetings (512
+// of 1k-20k: 82 ms against 105 on clusters of two).
+constexpr int64_t TEAM_BATCH_ROWS = 10240;
+static int team_batch_size(gbs_mat A, const ksp_opts &o) {
+  if (A->nsys < 2 || A->nsys >= 2 * sm_count(A) || o.method != GBS_KSP_CG ||
+      o.precision != GBS_FP64 || o.host_loop || A->lanes != GBS_SPMV_SELL || A->nrows == 0 ||
+      A->solver != GBS_SOLVER_AUTO || A->cg_form != GBS_CG_TEXTBOOK || !A->plan_auto)
+    return 1;
+  int size = 1;
+  while (size < TEAM_MAX_CLUSTER && ((int64_t)A->nsys * size < sm_count(A) ||
+                                     A->max_sys_rows > TEAM_BATCH_ROWS * size))
+    size *= 2;
+  return A->max_sys_rows <= TEAM_BATCH_ROWS * size ? size : 1;
+}
+
 // An automatic solver and plan take the team by size; the autotuner takes it
 // where it measured it fastest (team_tuned).  An explicit solver, plan or
 // single-reduction form is what the caller asked for.
 bool use_team(gbs_mat A, bool per_system, const ksp_opts &o) {
-  if (per_system || A->nsys != 1 || o.method != GBS_KSP_CG || o.precision != GBS_FP64 ||
+  if (per_system) return team_batch_size(A, o) > 1;
+  if (A->nsys != 1 || o.method != GBS_KSP_CG || o.precision != GBS_FP64 ||
       o.host_loop || A->lanes != GBS_SPMV_SELL || A->nrows == 0)
     return false;
   return A->team_tuned || (A->solver == GBS_SOLVER_AUTO && A->cg_form == GBS_CG_TEXTBOOK &&
@@ -712,11 +816,52 @@ static TeamShape team_shape(gbs_mat A) {
   return T;
 }
 
-// One FP64 CG solve on a team of CTAs; *ran stays false (and nothing has
-// started) where the device cannot hold the team at once.
-int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, cudaStream_t s,
-               bool *ran) {
+// FP64 CG on teams of CTAs; *ran stays false (and nothing has started) where
+// the device cannot hold a team at once.
+static int solve_team_batch(gbs_mat A, const double *b, double *x, const ksp_opts &o,
+                            cudaStream_t s, bool *ran) {
+  const int size = team_batch_size(A, o);
+  const int64_t per = (A->max_sys_rows / 32 + size) / size * 32;
+  const int tpb = per <= 1024 ? 512 : 1024;
+  void (*const kernel)(PcgArgs, int32_t, int32_t) =
+      tpb == 512 ? k_team_batch<512> : k_team_batch<1024>;
+  GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)TEAM_SMEM));
+  GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t lc = {};
+  cudaLaunchAttribute at[1];
+  memset(at, 0, sizeof(at));
+  lc.gridDim = dim3((unsigned)(sm_count(A) / size * size));
+  lc.blockDim = dim3((unsigned)tpb);
+  lc.dynamicSmemBytes = TEAM_SMEM;
+  lc.stream = s;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)size;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  int fit = 0;  // clusters resident at once
+  if (cudaOccupancyMaxActiveClusters(&fit, kernel, &lc) != cudaSuccess || fit < 1) {
+    cudaGetLastError();
+    return GBS_OK;
+  }
+  lc.gridDim = dim3((unsigned)(std::min<int64_t>(fit, A->nsys) * size));
+  PcgArgs a = make_args(A, true, false);
+  a.stream_matrix = 0;  // (a system's matrix is read again by the same SMs, from L2)
+  a.order = A->cta_order;
+  a.cta_n = A->nsys;
+  GBS_TRY_CUDA(cudaMemsetAsync(A->ctl, 0, sizeof(DevCtl), s));
+  GBS_TRY(put_call(A->call, call_args(b, x, o), s, A->ctl));
+  GBS_TRY_CUDA(cudaLaunchKernelEx(&lc, kernel, a, A->col_span, (int32_t)TEAM_SMEM));
+  count_launches(1);
+  *ran = true;
+  return GBS_OK;
+}
+
+int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,
+               cudaStream_t s, bool *ran) {
   *ran = false;
+  if (per_system) return solve_team_batch(A, b, x, o, s, ran);
   TeamShape T = team_shape(A);
   PcgArgs a = make_args(A, false, false);
   a.stream_matrix = stream_matrix(A, 8);

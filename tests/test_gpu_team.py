@@ -148,3 +148,83 @@ def test_two_streams_at_once():
         assert torch.equal(x, y)
     for A, _ in handles:
         A.close()
+
+
+def batch_of(shapes, seed):
+    rng = np.random.default_rng(seed)
+    I, J, V, rows, ncoo = [], [], [], [], []
+    for s in shapes:
+        n = int(np.prod(s))
+        if n:
+            ea, eb = W.grid_edges(s)
+            i, j, v = W.edge_coo(ea, eb, 10.0 ** rng.uniform(-1, 1, ea.shape[0]))
+        else:
+            i, j, v = np.zeros(0, np.int32), np.zeros(0, np.int32), np.zeros(0)
+        I.append(i), J.append(j), V.append(v), rows.append(n), ncoo.append(i.size)
+    b = rng.standard_normal(sum(rows))
+    A = B.Mat.from_coo_batched(rows, ncoo, t(np.concatenate(I)), t(np.concatenate(J)))
+    A.set_values(t(np.concatenate(V)))
+    off = np.concatenate([[0], np.cumsum(rows)])
+    gi = np.concatenate([np.where(i >= 0, i + o, -1) for i, o in zip(I, off)]).astype(np.int32)
+    gj = np.concatenate([np.where(j >= 0, j + o, -1) for j, o in zip(J, off)]).astype(np.int32)
+    O = oracle.coo_symbolic(int(off[-1]), int(off[-1]), gi, gj)
+    oracle.coo_numeric(O, np.concatenate(V))
+    return A, O, off, b
+
+
+BATCHES = {
+    # clusters of 16 (each other size below), systems of every kind of smallness
+    "2 systems": [(40, 40), (9, 10, 11)],
+    "9 systems, tiny and empty": [(32, 3), (8, 8), (0, 5), (33, 1), (64, 2), (12, 8), (20, 20),
+                                  (6, 6, 6), (31, 31)],
+    "12 systems": [(30 + k, 40) for k in range(12)],
+    "30 systems": [(20 + k, 23) for k in range(30)],
+    "60 systems": [(10 + k, 20) for k in range(60)],
+    "160 systems, one large": [(8 + k % 9, 16) for k in range(159)] + [(110, 100)],
+    "3 systems, the rows' limit": [(160, 1000), (40, 60, 60), (50, 50)],
+}
+
+
+@pytest.mark.parametrize("name", list(BATCHES))
+def test_batches(name):
+    A, O, off, b = batch_of(BATCHES[name], len(name))
+    c0 = B.launch_count()
+    x, rs = A.solve_batched(t(b), rtol=1e-10)
+    if A.plan()["kernel"] == B.SPMV_SELL:
+        assert B.launch_count() - c0 == 2
+    else:
+        assert "tiny" in name
+    xo, ros = oracle.pcg_batched(O, off, b, rtol=1e-10)
+    xg = x.cpu().numpy()
+    resid = b - oracle.spmv(O, xg)
+    for s, (r, ro) in enumerate(zip(rs, ros)):
+        sl = slice(off[s], off[s + 1])
+        assert r["status"] == B.OK and abs(r["iterations"] - ro["iterations"]) <= max(
+            2, 0.01 * ro["iterations"]), (s, r, ro)
+        assert np.linalg.norm(resid[sl]) <= 1.05e-10 * np.linalg.norm(b[sl])
+        assert np.linalg.norm(xg[sl] - xo[sl]) <= 1e-6 * np.linalg.norm(xo[sl])
+    x2, rs2 = A.solve_batched(t(b), rtol=1e-10)
+    assert torch.equal(x, x2) and rs == rs2
+    A.close()
+
+
+def test_batch_statuses():
+    A, O, off, b = batch_of([(30, 30), (20, 40), (25, 25), (10, 10, 10), (18, 30)], 3)
+    b[off[1]:off[2]] = 0.0
+    b[off[2] + 5] = np.nan
+    x, rs = A.solve_batched(t(b), x=torch.ones(b.size, dtype=torch.float64, device=DEV),
+                            rtol=1e-9, nonzero_guess=True)
+    assert [r["status"] for r in rs] == [B.OK, B.OK, B.ERR_NAN, B.OK, B.OK]
+    assert rs[1]["iterations"] == 0 and torch.count_nonzero(x[off[1]:off[2]]) == 0
+    xg = x.cpu().numpy()
+    for s in (0, 3, 4):
+        sl = slice(off[s], off[s + 1])
+        r = b[sl] - oracle.spmv(O, np.where(np.isfinite(xg), xg, 0.0))[sl]
+        assert np.linalg.norm(r) <= 1.05e-9 * np.linalg.norm(b[sl])
+    b[off[2] + 5] = 1.0
+    _, rs = A.solve_batched(t(b), maxit=3)
+    assert [r["status"] for r in rs] == [B.ERR_MAXIT, B.OK] + [B.ERR_MAXIT] * 3
+    _, rs = A.solve_batched(t(b), timeout_ns=1)
+    assert [r["status"] for r in rs] == [B.ERR_TIMEOUT, B.OK] + [B.ERR_TIMEOUT] * 3
+    assert all(r["iterations"] <= 1 for r in rs)
+    A.close()
