@@ -34,6 +34,10 @@ struct CtaShared {
   double lanes[BLOCK_SUMS_EXTRA];     // cta_sum0: lane partials
   double pub[4];                      // scalars published by thread 0
   int ipub[4];                        // [0]: < 0 keep going; [1], [2], [3]: flags
+  // thread 0's scalars (in every thread's registers they would leave the
+  // passes' loads in flight too few)
+  double sc[9];
+  int ic[5];
 };
 
 // Block sums of NV values, valid in warp 0 (thread 0): device_util.cuh's
@@ -91,13 +95,13 @@ __device__ __forceinline__ SysRange cta_system(const PcgArgs &a, int k) {
 }
 
 // Sliced-ELL row products of the system's slices, coherent x gathers.
-template <typename T, class F>
+template <typename T, int NP = 2, class F>
 __device__ __forceinline__ void cta_rows(const PcgArgs &a, const SysRange &g, const T *sval,
                                          const T *x, F &f) {
   if (a.stream_matrix)
-    sell_rows<T, true, GATHER_CA>(a.sv, sval, x, g.s0, g.s1, f);
+    sell_rows<T, true, GATHER_CA, false, NP>(a.sv, sval, x, g.s0, g.s1, f);
   else
-    sell_rows<T, false, GATHER_CA>(a.sv, sval, x, g.s0, g.s1, f);
+    sell_rows<T, false, GATHER_CA, false, NP>(a.sv, sval, x, g.s0, g.s1, f);
 }
 
 // Wall-clock limit (from the solve's start, DevCtl::t_start), for thread 0.
@@ -145,7 +149,7 @@ __device__ __forceinline__ void cta_true_residual(const PcgArgs &a, const SysRan
 }
 
 // FP64 PCG: the phases A, B, C of phases.cuh in one CTA, same tests.
-template <int U>
+template <int CPS>
 static __device__ __forceinline__ void cta_pcg_fp64(const PcgArgs &a, const SysRange &g, CtaShared &sh) {
   const CallArgs &C = *a.call;
   const double *b = C.b;
@@ -173,10 +177,11 @@ static __device__ __forceinline__ void cta_pcg_fp64(const PcgArgs &a, const SysR
   }
   cta_sum0<double, 4>(v, sh);
   // thread 0's scalars
-  double rho = 0.0, bb = 0.0, thr = 0.0, rn = 0.0, rnorm0 = 0.0;
-  int it = 0, status = -1;
-  bool zero = false, timed = false;
+  double &rho = sh.sc[0], &bb = sh.sc[1], &thr = sh.sc[2], &rn = sh.sc[3], &rnorm0 = sh.sc[4];
+  int &it = sh.ic[0], &status = sh.ic[1], &timed = sh.ic[2], &zero = sh.ic[3];
   if (t0) {
+    it = timed = zero = 0;
+    status = -1;
     rho = v[0];
     bb = v[2];
     thr = C.rtol * sqrt(bb);
@@ -185,7 +190,7 @@ static __device__ __forceinline__ void cta_pcg_fp64(const PcgArgs &a, const SysR
     else if (!isfinite(bb)) status = GBS_ERR_NAN;
     else if (bb == 0.0) {
       status = GBS_OK;
-      zero = true;
+      zero = 1;
       rn = rnorm0 = 0.0;
     } else if (!isfinite(v[1]) || !isfinite(rho)) status = GBS_ERR_NAN;
     else if (rn <= thr) status = GBS_OK;
@@ -199,11 +204,14 @@ static __device__ __forceinline__ void cta_pcg_fp64(const PcgArgs &a, const SysR
   while (go) {
     // A: q = A p, p.q -> alpha
     double pq[1] = {0.0};
+    double pr;
+    auto la = [&](int r) { pr = a.p[r]; };
     auto fa = [&](int r, double qv) {
       a.q[r] = qv;
-      pq[0] = fma(a.p[r], qv, pq[0]);
+      pq[0] = fma(pr, qv, pq[0]);
     };
-    cta_rows<double>(a, g, a.sval, a.p, fa);
+    RowFn<decltype(la) &, decltype(fa) &> f{la, fa};
+    cta_rows<double, CPS == 1 ? 4 : 2>(a, g, a.sval, a.p, f);
     cta_sum0<double, 1>(pq, sh);
     if (t0) {
       ++it;
@@ -217,25 +225,15 @@ static __device__ __forceinline__ void cta_pcg_fp64(const PcgArgs &a, const SysR
     const double al = sh.pub[0];
     // B: x += alpha p, r -= alpha q, z = D^-1 r (over q), r.z, r.r -> tests, beta
     double w[2] = {0.0, 0.0};
-    {
-      double qv[U], rv0[U], dv[U], pv[U], xv[U];
-      auto ld = [&](int r, int k) {
-        qv[k] = a.q[r];
-        rv0[k] = a.r[r];
-        dv[k] = a.dinv[r];
-        pv[k] = a.p[r];
-        xv[k] = x[r];
-      };
-      auto use = [&](int r, int k) {
-        const double rv = fma(-al, qv[k], rv0[k]);
-        const double z = dv[k] * rv;
-        x[r] = fma(al, pv[k], xv[k]);
-        a.r[r] = rv;
-        a.q[r] = z;
-        w[0] = fma(rv, z, w[0]);
-        w[1] = fma(rv, rv, w[1]);
-      };
-      cta_rows_by<U>(g.r0, g.r1, ld, use);
+    for (int r = g.r0 + threadIdx.x; r < g.r1; r += blockDim.x) {
+      const double qv = a.q[r], rv0 = a.r[r], dv = a.dinv[r], pv = a.p[r], xv = x[r];
+      const double rv = fma(-al, qv, rv0);
+      const double z = dv * rv;
+      x[r] = fma(al, pv, xv);
+      a.r[r] = rv;
+      a.q[r] = z;
+      w[0] = fma(rv, z, w[0]);
+      w[1] = fma(rv, rv, w[1]);
     }
     cta_sum0<double, 2>(w, sh);
     if (t0) {
@@ -243,7 +241,7 @@ static __device__ __forceinline__ void cta_pcg_fp64(const PcgArgs &a, const SysR
       if (!isfinite(rn) || !isfinite(w[0])) status = GBS_ERR_NAN;
       else if (rn <= thr) status = GBS_OK;
       else if (it >= C.maxit) status = GBS_ERR_MAXIT;
-      else if (cta_timed_out(a.ctl, C.timeout_ns)) timed = true;
+      else if (cta_timed_out(a.ctl, C.timeout_ns)) timed = 1;
       else {
         sh.pub[0] = w[0] / rho;
         rho = w[0];
@@ -254,14 +252,9 @@ static __device__ __forceinline__ void cta_pcg_fp64(const PcgArgs &a, const SysR
     if (sh.ipub[0] >= 0) break;
     const double be = sh.pub[0];
     // C: p = z + beta p (each thread its own rows: the rows B wrote)
-    {
-      double pv[U], zv[U];
-      auto ld = [&](int r, int k) {
-        pv[k] = a.p[r];
-        zv[k] = a.q[r];
-      };
-      auto use = [&](int r, int k) { a.p[r] = fma(be, pv[k], zv[k]); };
-      cta_rows_by<U>(g.r0, g.r1, ld, use);
+    for (int r = g.r0 + threadIdx.x; r < g.r1; r += blockDim.x) {
+      const double zv = a.q[r];
+      a.p[r] = fma(be, a.p[r], zv);
     }
     __syncthreads();  // p complete before the next product gathers it
   }
@@ -270,8 +263,9 @@ static __device__ __forceinline__ void cta_pcg_fp64(const PcgArgs &a, const SysR
 }
 
 // FP32 inner PCG under FP64 refinement, the oracle's order of steps.
-template <int U>
+template <int CPS>
 static __device__ __forceinline__ void cta_pcg_refined(const PcgArgs &a, const SysRange &g, CtaShared &sh) {
+  constexpr int U = CPS == 1 ? 2 : 1;  // FP32 rows in flight a thread
   const CallArgs &C = *a.call;
   const double *b = C.b;
   double *x = C.x;
@@ -286,10 +280,16 @@ static __device__ __forceinline__ void cta_pcg_refined(const PcgArgs &a, const S
   }
   cta_sum0<double, 2>(v, sh);  // (its barrier also orders the x writes before the first product)
   // thread 0's scalars
-  double bb = 0.0, bnorm = 0.0, rnorm0 = 0.0, rn = 0.0, prev_rn = INFINITY;
-  int status = -1, outer = 0, stall = 0, iters = 0;
-  bool zero = false, timed = false;
+  double &bb = sh.sc[0], &bnorm = sh.sc[1], &rnorm0 = sh.sc[2], &rn = sh.sc[3],
+         &prev_rn = sh.sc[4], &thr = sh.sc[5];
+  int &status = sh.ic[0], &outer = sh.ic[1], &stall = sh.ic[2], &iters = sh.ic[3],
+      &timed = sh.ic[4];
+  bool zero = false;
   if (t0) {
+    status = -1;
+    outer = stall = iters = timed = 0;
+    rnorm0 = rn = 0.0;
+    prev_rn = INFINITY;
     bb = v[0];
     bnorm = sqrt(bb);
     if (v[1] > 0.0) status = GBS_ERR_NOT_SPD;
@@ -322,7 +322,7 @@ static __device__ __forceinline__ void cta_pcg_refined(const PcgArgs &a, const S
       else if (outer >= C.max_outer) status = GBS_ERR_MAXIT;
       else if (outer > 0 && (stall = (rn > 0.5 * prev_rn) ? stall + 1 : 0) >= 2)
         status = GBS_ERR_STAGNATION;
-      else if (cta_timed_out(a.ctl, C.timeout_ns)) timed = true;
+      else if (cta_timed_out(a.ctl, C.timeout_ns)) timed = 1;
       else {
         prev_rn = rn;
         sh.pub[0] = rn;
@@ -346,7 +346,6 @@ static __device__ __forceinline__ void cta_pcg_refined(const PcgArgs &a, const S
     }
     cta_sum0<float, 2>(w, sh);
     float rho = 0.0f;
-    double thr = 0.0;
     int it = 0;
     if (t0) {
       rho = w[0];
@@ -358,11 +357,14 @@ static __device__ __forceinline__ void cta_pcg_refined(const PcgArgs &a, const S
     int inner = sh.ipub[1];
     while (inner) {
       float pq[1] = {0.0f};
+      float pr;
+      auto la = [&](int r) { pr = a.p32[r]; };
       auto fa = [&](int r, float qv) {
         a.q32[r] = qv;
-        pq[0] = fmaf(a.p32[r], qv, pq[0]);
+        pq[0] = fmaf(pr, qv, pq[0]);
       };
-      cta_rows<float>(a, g, a.sval32, a.p32, fa);
+      RowFn<decltype(la) &, decltype(fa) &> f{la, fa};
+      cta_rows<float, CPS == 1 ? 3 : 2>(a, g, a.sval32, a.p32, f);
       cta_sum0<float, 1>(pq, sh);
       if (t0) {
         const bool ok = pq[0] > 0.0f;
@@ -436,22 +438,31 @@ static __device__ __forceinline__ void cta_pcg_refined(const PcgArgs &a, const S
 // unsolved one (order[grid], order[grid + 1], ... by an atomic counter) until
 // none is left -- largest first, so the largest systems start at once and
 // the rest fill the SMs as they free up (greedy list scheduling).
-// CPS: CTAs per SM the grid runs.  The register budget follows (32 per
-// thread for two, 64 for one), and with it the rows a thread keeps in flight
-// in the element-wise loops (cta_rows_by): one for two CTAs per SM; for one,
-// two FP64 rows or four FP32 rows.  Measured on a batch of 512 systems of
-// 1k-200k rows: one CTA per SM, FP64 CG 2.14 s with one row in flight, 1.96
-// with two, 2.03 with four, 2.31 with eight; the refined solve 1.75, 1.43,
-// 1.39, 1.55 s; two CTAs per SM with two rows spill and slow down.
+// CPS: CTAs per SM the grid runs.  The register budget follows: 32 a thread for
+// two, 64 for one.  With one, the row products keep four (FP32: three) pairs
+// and the next slice's tables in flight (sell_rows_deep) and load the row of p
+// their dot product takes ahead of the sum, and the FP32 passes take two rows
+// at a time.  What bounds it: 152 systems' vectors and matrices do not stay in
+// L2, a pass waits on the latency of its loads, and a spilled register costs
+// more than a row in flight gains -- so thread 0's scalars live in shared
+// memory and the FP64 passes take one row at a time.  Measured, ms (a batch of
+// 512 systems of 1k-20k rows; 1024 of 500-4k; 310 of 20k-60k):
+//   FP64, scalars in registers, two pairs, two rows       83.1   22.0   428
+//     scalars in shared memory                             80.7   21.9
+//     ... and one row in flight                            76.4   20.6
+//     ... and four pairs, p ahead (this)                   71.0   20.6   382
+//     four pairs, two rows (spills)                        74.2   22.4   376
+//   refined, scalars in registers, two pairs, four rows    50.7   13.2   328
+//     this (three pairs, two rows)                         48.0   12.2   271
+//     four pairs, two rows; three pairs, one row           49.6, 50.5   12.8, 11.4   281, 305
 template <bool REFINED, int CPS>
 __global__ void __launch_bounds__(CTA_TPB, CPS) k_cta_pcg(PcgArgs a) {
-  constexpr int U = CPS == 1 ? (REFINED ? 4 : 2) : 1;
   __shared__ CtaShared sh;
   __shared__ int next;
   for (int k = blockIdx.x; k < a.cta_n;) {
     const SysRange g = cta_system(a, k);
-    if (REFINED) cta_pcg_refined<U>(a, g, sh);
-    else cta_pcg_fp64<U>(a, g, sh);
+    if (REFINED) cta_pcg_refined<CPS>(a, g, sh);
+    else cta_pcg_fp64<CPS>(a, g, sh);
     __syncthreads();  // every thread is done with sh and with the system
     if (threadIdx.x == 0) next = (int)gridDim.x + atomicAdd(&a.ctl->queue, 1);
     __syncthreads();

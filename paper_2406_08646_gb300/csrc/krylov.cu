@@ -93,6 +93,23 @@ __device__ __forceinline__ void kry_rows(const KrylovArgs &a, const KSys &g, con
   else sell_rows<double, false, GATHER_CA>(S, sval, x, g.s0, g.s1, f);
 }
 
+// ... with the consumer's own operands loaded ahead of each row's sum, or with it.
+template <bool AHEAD, int NP, class L, class F>
+__device__ __forceinline__ void kry_rows(const KrylovArgs &a, const KSys &g, const SellView &S,
+                                         const double *sval, const double *x, L load, F use) {
+  if constexpr (AHEAD) {
+    RowFn<L &, F &> f{load, use};
+    if (a.stream_matrix) sell_rows<double, true, GATHER_CA, false, NP>(S, sval, x, g.s0, g.s1, f);
+    else sell_rows<double, false, GATHER_CA, false, NP>(S, sval, x, g.s0, g.s1, f);
+  } else {
+    auto f = [&](int i, double y) {
+      load(i);
+      use(i, y);
+    };
+    kry_rows(a, g, S, sval, x, f);
+  }
+}
+
 // The system's closing state (thread 0), x = 0 where b = 0, then
 // ||b - A x||^2 into S.tt.
 __device__ void kry_close(const KrylovArgs &a, const KSys &g, CtaShared &sh, int status,
@@ -140,6 +157,7 @@ __device__ __forceinline__ int kry_start_status(double missing, double bb) {
 // (sh.ipub[0] < 0), and every thread reads them after one barrier.
 
 // ------------------------------------------------------------------ BiCG
+template <bool AHEAD>
 __device__ void kry_bicg(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
   const CallArgs &C = *a.call;
   const double *b = C.b;
@@ -168,21 +186,26 @@ __device__ void kry_bicg(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
   }
   cta_sum0<double, 4>(v, sh);
   // thread 0's scalars
-  double bb = 0.0, thr = 0.0, rn = 0.0, rnorm0 = 0.0, rho = 0.0, rho_prev = 0.0;
-  int status = -1, it = 0;
-  bool timed = false;
+  double loc[6];
+  double *const sc = AHEAD ? sh.sc : loc;
+  double &bb = sc[0], &thr = sc[1], &rn = sc[2], &rnorm0 = sc[3], &rho = sc[4], &rho_prev = sc[5];
+  int iloc[3];
+  int *const ic = AHEAD ? sh.ic : iloc;
+  int &status = ic[0], &it = ic[1], &timed = ic[2];
   // the tests before an iteration; publishes beta (ipub[1]: first iteration)
   auto top = [&]() {
     if (!isfinite(rn)) status = GBS_ERR_NAN;
     else if (rn <= thr) status = GBS_OK;
     else if (it >= C.maxit) status = GBS_ERR_MAXIT;
     else if (rho == 0.0) status = GBS_ERR_BREAKDOWN;
-    else if (it > 0 && cta_timed_out(a.ctl, C.timeout_ns)) timed = true;
+    else if (it > 0 && cta_timed_out(a.ctl, C.timeout_ns)) timed = 1;
     else sh.pub[0] = it == 0 ? 0.0 : rho / rho_prev;
     sh.ipub[0] = (status < 0 && !timed) ? -1 : 0;
     sh.ipub[1] = it == 0;
   };
   if (t0) {
+    it = timed = 0;
+    rho_prev = 0.0;
     bb = v[1];
     thr = C.rtol * sqrt(bb);
     rn = rnorm0 = sqrt(v[0]);
@@ -200,20 +223,29 @@ __device__ void kry_bicg(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
     const double beta = sh.pub[0];
     const bool first = sh.ipub[1] != 0;
     for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) {
-      const double dv = dinv[i], z = dv * r[i], zt = dv * rt[i];
-      p[i] = first ? z : fma(beta, p[i], z);
-      pt[i] = first ? zt : fma(beta, pt[i], zt);
+      const double dv = dinv[i], z = dv * r[i], pv = first ? 0.0 : p[i];
+      double zt, ptv;
+      auto rest = [&] {
+        zt = dv * rt[i];
+        ptv = first ? 0.0 : pt[i];  // (not set before the first iteration)
+      };
+      if constexpr (AHEAD) rest();
+      p[i] = first ? z : fma(beta, pv, z);
+      if constexpr (!AHEAD) rest();
+      pt[i] = first ? zt : fma(beta, ptv, zt);
     }
     __syncthreads();
     // q = A p with pt.q, qt = A^T pt
     double sg[1] = {0.0};
-    auto fq = [&](int i, double y) {
-      q[i] = y;
-      sg[0] = fma(pt[i], y, sg[0]);
-    };
-    kry_rows(a, g, a.sv, a.sval, p, fq);
+    double pti;
+    kry_rows<AHEAD, 4>(
+        a, g, a.sv, a.sval, p, [&](int i) { pti = pt[i]; },
+        [&](int i, double y) {
+          q[i] = y;
+          sg[0] = fma(pti, y, sg[0]);
+        });
     auto fqt = [&](int i, double y) { qt[i] = y; };
-    kry_rows(a, g, a.tv, a.tval, pt, fqt);
+    kry_rows<AHEAD, 4>(a, g, a.tv, a.tval, pt, [](int) {}, fqt);
     cta_sum0<double, 1>(sg, sh);
     if (t0) {
       ++it;
@@ -228,13 +260,24 @@ __device__ void kry_bicg(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
     // x += alpha p, r -= alpha q, rt -= alpha qt; ||r||^2, (D^-1 r).rt
     double u[2] = {0.0, 0.0};
     for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) {
-      x[i] = fma(alpha, p[i], x[i]);
-      const double rv = fma(-alpha, q[i], r[i]);
-      const double rtv = fma(-alpha, qt[i], rt[i]);
+      const double pv = p[i], xv = x[i];
+      double qv, r0, qtv, rt0, dv;
+      auto rest = [&] {
+        qv = q[i];
+        r0 = r[i];
+        qtv = qt[i];
+        rt0 = rt[i];
+        dv = dinv[i];
+      };
+      if constexpr (AHEAD) rest();
+      x[i] = fma(alpha, pv, xv);
+      if constexpr (!AHEAD) rest();
+      const double rv = fma(-alpha, qv, r0);
+      const double rtv = fma(-alpha, qtv, rt0);
       r[i] = rv;
       rt[i] = rtv;
       u[0] = fma(rv, rv, u[0]);
-      u[1] = fma(dinv[i] * rv, rtv, u[1]);
+      u[1] = fma(dv * rv, rtv, u[1]);
     }
     cta_sum0<double, 2>(u, sh);
     if (t0) {
@@ -249,6 +292,7 @@ __device__ void kry_bicg(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
 }
 
 // ------------------------------------------------------------------ TFQMR
+template <bool AHEAD>
 __device__ void kry_tfqmr(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
   const CallArgs &C = *a.call;
   const double *b = C.b;
@@ -281,11 +325,13 @@ __device__ void kry_tfqmr(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
   }
   cta_sum0<double, 3>(v, sh);
   // thread 0's scalars
-  double bb = 0.0, thr = 0.0, rnorm0 = 0.0, rn = 0.0;
-  double rho = 0.0, tau = 0.0, theta = 0.0, eta = 0.0, alpha = 0.0;
-  int status = -1, it = 0, m = 0;
-  bool timed = false;
+  double &bb = sh.sc[0], &thr = sh.sc[1], &rnorm0 = sh.sc[2], &rn = sh.sc[3], &rho = sh.sc[4],
+         &tau = sh.sc[5], &theta = sh.sc[6], &eta = sh.sc[7], &alpha = sh.sc[8];
+  int &status = sh.ic[0], &it = sh.ic[1], &timed = sh.ic[2];
+  int m = 0;
   if (t0) {
+    it = timed = 0;
+    theta = eta = alpha = 0.0;
     bb = v[1];
     thr = C.rtol * sqrt(bb);
     rn = rnorm0 = sqrt(v[0]);
@@ -346,13 +392,14 @@ __device__ void kry_tfqmr(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
       // half step 1 with (y1, B y1); y2 = y1 - alpha v, t = D^-1 y2
       double s1[1] = {0.0};
       for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) {
-        const double y1i = y1[i];
-        const double y2i = y1i - al * vv[i];
+        const double y1i = y1[i], v0 = vv[i], dv = dinv[i];
+        const double w0 = w[i], by = by1[i], d0 = d[i];
+        const double y2i = y1i - al * v0;
         y2[i] = y2i;
-        t[i] = dinv[i] * y2i;
-        const double wn = w[i] - al * by1[i];
+        t[i] = dv * y2i;
+        const double wn = w0 - al * by;
         w[i] = wn;
-        d[i] = y1i + coef1 * d[i];
+        d[i] = y1i + coef1 * d0;
         s1[0] = fma(wn, wn, s1[0]);
       }
       cta_sum0<double, 1>(s1, sh);
@@ -368,17 +415,28 @@ __device__ void kry_tfqmr(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
       // B y2 (= A t) fused with half step 1's x update and half step 2
       const double e1 = sh.pub[2], coef2 = sh.pub[3];
       double s2[2] = {0.0, 0.0};
-      auto f1 = [&](int i, double y) {
-        by2[i] = y;
-        const double di = d[i];
-        x[i] = fma(e1, dinv[i] * di, x[i]);
-        d[i] = y2[i] + coef2 * di;
-        const double wn = w[i] - al * y;
-        w[i] = wn;
-        s2[0] = fma(wn, wn, s2[0]);
-        s2[1] = fma(rt[i], wn, s2[1]);
-      };
-      kry_rows(a, g, a.sv, a.sval, t, f1);
+      {
+        double di, dv, xv, yv, w0, rv;
+        kry_rows<AHEAD, 2>(
+            a, g, a.sv, a.sval, t,
+            [&](int i) {
+              di = d[i];
+              dv = dinv[i];
+              xv = x[i];
+              yv = y2[i];
+              w0 = w[i];
+              rv = rt[i];
+            },
+            [&](int i, double y) {
+              by2[i] = y;
+              x[i] = fma(e1, dv * di, xv);
+              d[i] = yv + coef2 * di;
+              const double wn = w0 - al * y;
+              w[i] = wn;
+              s2[0] = fma(wn, wn, s2[0]);
+              s2[1] = fma(rv, wn, s2[1]);
+            });
+      }
       cta_sum0<double, 2>(s2, sh);
       if (t0) {
         bool stop = half(s2[0]);
@@ -387,7 +445,7 @@ __device__ void kry_tfqmr(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
           stop = true;
         }
         if (!stop && cta_timed_out(a.ctl, C.timeout_ns)) {
-          timed = true;
+          timed = 1;
           stop = true;
         }
         sh.pub[2] = eta;
@@ -402,23 +460,32 @@ __device__ void kry_tfqmr(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
       // y1 = w + beta y2, t = D^-1 y1, half step 2's x update
       const double e2 = sh.pub[2], beta = sh.pub[3];
       for (int i = g.r0 + threadIdx.x; i < g.r1; i += blockDim.x) {
-        const double dv = dinv[i];
-        const double y = w[i] + beta * y2[i];
+        const double dv = dinv[i], w0 = w[i], y0 = y2[i], d0 = d[i], xv = x[i];
+        const double y = w0 + beta * y0;
         y1[i] = y;
         t[i] = dv * y;
-        x[i] = fma(e2, dv * d[i], x[i]);
+        x[i] = fma(e2, dv * d0, xv);
       }
       pend = false;
       __syncthreads();
       // B y1 (= A t), v = B y1 + beta (B y2 + beta v), rt.v
       double s3[1] = {0.0};
-      auto f2 = [&](int i, double y) {
-        by1[i] = y;
-        const double vn = y + beta * (by2[i] + beta * vv[i]);
-        vv[i] = vn;
-        s3[0] = fma(rt[i], vn, s3[0]);
-      };
-      kry_rows(a, g, a.sv, a.sval, t, f2);
+      {
+        double b2, v0, rv;
+        kry_rows<AHEAD, 2>(
+            a, g, a.sv, a.sval, t,
+            [&](int i) {
+              b2 = by2[i];
+              v0 = vv[i];
+              rv = rt[i];
+            },
+            [&](int i, double y) {
+              by1[i] = y;
+              const double vn = y + beta * (b2 + beta * v0);
+              vv[i] = vn;
+              s3[0] = fma(rv, vn, s3[0]);
+            });
+      }
       cta_sum0<double, 1>(s3, sh);
       if (t0) {
         ++it;  // B y1
@@ -439,12 +506,31 @@ __device__ void kry_tfqmr(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
 // registers, a few hundred bytes of spills) keeps two systems in flight per
 // SM, which a batch of at least two systems per SM repays (about 1.4x the
 // solves per second on 1024 convection-diffusion systems).
+//
+// What bounds it: 152 systems' matrices and twelve vectors do not stay in L2,
+// so every pass waits on its loads' latency.  A pass that stores a row's
+// values between its loads keeps the compiler from moving the loads together
+// (the pointers may alias), so a row's operands are loaded before its first
+// store, in the products before the row's sum (AHEAD; BiCG's products with
+// four pairs in flight), and thread 0's scalars live in shared memory to free
+// registers for them.  At two CTAs per SM the registers do not allow it: BiCG
+// keeps its scalars local and its passes' loads spread out.  Every thread adds
+// the same rows in the same order either way.  Measured, ms (systems x rows):
+//                              before   this
+//   TFQMR 256 x 1k-20k           97.8   76.5
+//   BiCG  256 x 1k-20k           99.5   78.1
+//   BiCG  152 x 15k-20k         105.5   81.2
+//   TFQMR 1024 x 500-4k (two)    23.1   21.7
+//   BiCG  512 x 1k-8k (two)      34.9   34.2
+// Two rows in flight spill (TFQMR 85.2, BiCG 96.9); clusters of two or four
+// CTAs a system with the same 1024 threads give 100 and 90.
 template <int METHOD, int MINB>
 __global__ void __launch_bounds__(CTA_TPB, MINB) k_cta_krylov(KrylovArgs a) {
   __shared__ CtaShared sh;
   const KSys g = kry_system(a);
-  if (METHOD == GBS_KSP_BICG) kry_bicg(a, g, sh);
-  else kry_tfqmr(a, g, sh);
+  constexpr bool AHEAD = MINB == 1;
+  if (METHOD == GBS_KSP_BICG) kry_bicg<AHEAD>(a, g, sh);
+  else kry_tfqmr<AHEAD>(a, g, sh);
 }
 
 // ------------------------------------------------------------------ phases

@@ -648,6 +648,22 @@ __device__ __forceinline__ int2 sell_pair_cols(const int2 *__restrict__ c2,
   return ld_entry<STREAM, SM>(c2 + pi);
 }
 
+// A row's consumer with operands of its own: load(r) issues their loads before
+// the row's products are summed, use(r, sum) finishes the row.
+template <class L, class U>
+struct RowFn {
+  L load;
+  U use;
+  template <typename T>
+  __device__ __forceinline__ void operator()(int r, T v) { use(r, v); }
+};
+template <class F>
+__device__ __forceinline__ void row_loads(F &, int, int) {}
+template <class L, class U>
+__device__ __forceinline__ void row_loads(RowFn<L, U> &f, int r, int re) {
+  if (r < re) f.load(r);
+}
+
 // Slices with column patterns (S.pat set: every slice has one).  SM: the view
 // and the values are copies in shared memory (team.cu), read by plain loads.
 template <typename T, bool STREAM, int NC, bool SM = false, class F>
@@ -661,6 +677,7 @@ __device__ __forceinline__ void sell_rows_pat(const SellView &S, const T *__rest
     const int r = ld_meta<SM>(S.row0 + sl) + lane, re = ld_meta<SM>(S.row0 + sl + 1);
     const int2 *__restrict__ pat2 = reinterpret_cast<const int2 *>(S.pool + ld_meta<SM>(S.pat + sl));
     uint32_t mk = ld_meta<SM>(S.mask + 32 * (int64_t)sl + lane);
+    row_loads(f, r, re);
     if constexpr (STREAM && !SM && sizeof(T) == 4) {  // the slice's whole run in flight at once
       if (lane == 0) prefetch_rows(sval, b0, b1);
     }
@@ -746,6 +763,7 @@ __device__ __forceinline__ void sell_rows_deep(const SellView &S, const T *__res
       np0 = ld_meta<SM>(S.pat + nx);
       nmk = ld_meta<SM>(S.mask + 32 * (int64_t)nx + lane);
     }
+    row_loads(f, r + lane, re);
     const int w = (b1 - b0) >> 5;
     const T *xr = x + r + lane;
     const P *v2 = reinterpret_cast<const P *>(sval) + (b0 >> 1) + lane;
@@ -796,6 +814,7 @@ __device__ __forceinline__ void sell_rows(const SellView &S, const T *__restrict
   for (int sl = s0 + (int)(threadIdx.x >> 5); sl < s1; sl += (int)(blockDim.x >> 5)) {
     const int b0 = ld_meta<SM>(S.ptr + sl), b1 = ld_meta<SM>(S.ptr + sl + 1);
     const int r = ld_meta<SM>(S.row0 + sl) + lane, re = ld_meta<SM>(S.row0 + sl + 1);
+    row_loads(f, r, re);
     if constexpr (STREAM && !SM && sizeof(T) == 4) {  // the slice's whole run in flight at once
       if (lane == 0) prefetch_rows(sval, b0, b1);
       else if (lane == 1) {
