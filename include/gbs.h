@@ -481,9 +481,9 @@ int mat_get_tuning(gbs_mat A, int32_t *solver, int32_t *cg_form, int64_t *split_
  *
  * mat_autotune_file: the same, persisted.  path names a text file (created if
  * missing) of one line per tuned key: "<key> | Ra Re kernel ctas_per_sm
- * solver cg_form split_rows patterns | <time>" (patterns: 0 or 1, plus 2 where one
- * system's CG runs on the team of CTAs; lines without the last one
- * or two fields leave those settings as they are).  The key holds the handle's sizes, a hash of its
+ * solver cg_form split_rows patterns | <time>" (patterns: 0 or 1, plus 2 where FP64 CG
+ * runs on teams of CTAs; lines without the last one or two fields leave those
+ * settings as they are).  The key holds the handle's sizes, a hash of its
  * systems' sizes and of 257 sampled entries each of row_ptr and col, the
  * device name and SM count, and "fp64".  A matching line is applied without
  * timing (*from_cache = 1); otherwise the handle is tuned and the line

@@ -523,7 +523,7 @@ struct Tuning {
   int32_t Ra, Re, kernel, cpsm, solver, cg_form;
   int64_t split_rows;
   int32_t patterns;  // column patterns of the sliced copy (1 / 0; -1: as they are)
-  int32_t team;      // one system: the team of CTAs instead of the phase kernels
+  int32_t team;      // teams of CTAs (team.cu) instead of the phase kernels
 };
 
 // Makes t the handle's plan (rebuilt only when it differs from the current
@@ -537,7 +537,7 @@ int apply_tuning(gbs_mat A, const Tuning &t, cudaStream_t s) {
   A->solver_batched_only = A->nsys > 1;  // tuned on the batched solve
   A->cg_form = t.cg_form;
   A->split_rows = t.split_rows;
-  A->team_tuned = t.team != 0 && A->nsys == 1;
+  A->team_tuned = t.team != 0;
   return GBS_OK;
 }
 
@@ -634,6 +634,9 @@ static int autotune(gbs_mat A, cudaStream_t s, Tuning *out, float *out_ms) {
     if (per_system) {
       t.cg_form = GBS_CG_SINGLE_REDUCTION;
       timed(t);
+      t.cg_form = GBS_CG_TEXTBOOK;
+      t.team = 1;
+      if (st == GBS_OK && batch_teams(A)) timed(t);
     } else {  // the one-kernel form (where it fits, else two)
       t.cg_form = GBS_CG_SINGLE_KERNEL;
       timed(t);
@@ -674,7 +677,7 @@ static int autotune(gbs_mat A, cudaStream_t s, Tuning *out, float *out_ms) {
   // the copy takes none either way
   if (st == GBS_OK && per_system && best.kernel == GBS_SPMV_SELL &&
       apply_tuning(A, best, s) == GBS_OK && (best.patterns == 0 || A->sell_npat > 0)) {
-    Tuning t = best;
+    Tuning t = best;  // (a team's row products read either alike)
     t.patterns = best.patterns ? 0 : 1;
     timed(t);
   }

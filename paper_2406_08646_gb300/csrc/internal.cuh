@@ -208,7 +208,7 @@ struct gbs_mat_s {
   int32_t Ra = 256, Re = 512;   // rows per SpMV block / per update block
   int32_t lanes = 0;
   bool plan_auto = false;       // every part of the plan was left automatic
-  bool team_tuned = false;      // the autotuner chose the team of CTAs (team.cu) for one system
+  bool team_tuned = false;      // the autotuner chose teams of CTAs (team.cu) for FP64 CG
   int32_t ctas_per_sm = 0;      // grid cap per SM, 0 = as many as fit (one wave)
   int32_t solver = 0;           // GBS_SOLVER_AUTO / PHASES / CTA / SPLIT
   int64_t split_rows = 1;       // GBS_SOLVER_SPLIT: systems of at least this many rows on
@@ -285,6 +285,7 @@ int symbolic(gbs_mat A, const int32_t *i, const int32_t *j, const int64_t *coo_o
 int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,
           cudaStream_t s);
 void free_handle(gbs_mat A);
+bool batch_teams(gbs_mat A);  // a batch whose systems would get a cluster each
 bool use_team(gbs_mat A, bool per_system, const ksp_opts &o);
 int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,
                cudaStream_t s, bool *ran);

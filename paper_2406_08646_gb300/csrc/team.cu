@@ -472,7 +472,7 @@ __device__ __forceinline__ void team_pcg(const PcgArgs &a, Team<GRID> &tm, bool 
   }
   mark(4);
   if (clk)
-    for (int k = 0; k < 5; ++k) a.ctl->phase_ns[k] = (int64_t)sh.ns[k];
+    for (int k = 0; k < 5; ++k) a.ctl->phase_ns[k] += (int64_t)sh.ns[k];
 }
 
 __device__ __forceinline__ size_t up16(size_t n) { return (n + 15) & ~(size_t)15; }
@@ -667,7 +667,8 @@ __device__ __forceinline__ TeamCfg team_layout(int n, int per_rows, int halo, in
 // them and spilled -- 2.6 KB a thread at 64 registers.)
 __device__ __noinline__ void batch_system(const PcgArgs &a, TeamShared &sh, double *red,
                                           uint32_t rank, uint32_t size) {
-  team_system<false>(a, sh.cfg, sh, red, cta_system(a, sh.next), rank, size, false);
+  team_system<false>(a, sh.cfg, sh, red, cta_system(a, sh.next), rank, size,
+                     blockIdx.x == 0);  // (the first cluster's phase times)
 }
 
 // A batch (FP64 CG, each system on its own): a persistent grid of clusters, each
@@ -740,16 +741,23 @@ constexpr int64_t TEAM_GRID_ROWS = 3 << 20;
 // systems an SM on the per-CTA solver keeps every SM busy with no meetings (512
 // of 1k-20k: 82 ms against 105 on clusters of two).
 constexpr int64_t TEAM_BATCH_ROWS = 10240;
-static int team_batch_size(gbs_mat A, const ksp_opts &o) {
-  if (A->nsys < 2 || A->nsys >= 2 * sm_count(A) || o.method != GBS_KSP_CG ||
-      o.precision != GBS_FP64 || o.host_loop || A->lanes != GBS_SPMV_SELL || A->nrows == 0 ||
-      A->solver != GBS_SOLVER_AUTO || A->cg_form != GBS_CG_TEXTBOOK || !A->plan_auto)
-    return 1;
+static int team_clusters(gbs_mat A) {
+  if (A->nsys < 2 || A->nsys >= 2 * sm_count(A) || A->nrows == 0) return 1;
   int size = 1;
   while (size < TEAM_MAX_CLUSTER && ((int64_t)A->nsys * size < sm_count(A) ||
                                      A->max_sys_rows > TEAM_BATCH_ROWS * size))
     size *= 2;
   return A->max_sys_rows <= TEAM_BATCH_ROWS * size ? size : 1;
+}
+bool batch_teams(gbs_mat A) { return team_clusters(A) > 1; }
+
+static int team_batch_size(gbs_mat A, const ksp_opts &o) {
+  if (o.method != GBS_KSP_CG || o.precision != GBS_FP64 || o.host_loop ||
+      A->lanes != GBS_SPMV_SELL ||
+      !(A->team_tuned || (A->solver == GBS_SOLVER_AUTO && A->cg_form == GBS_CG_TEXTBOOK &&
+                          A->plan_auto)))
+    return 1;
+  return team_clusters(A);
 }
 
 // An automatic solver and plan take the team by size; the autotuner takes it
