@@ -415,14 +415,18 @@ int mat_get_plan(gbs_mat A, int32_t *spmv_rows, int32_t *update_rows, int32_t *k
  *   GBS_SOLVER_AUTO (default): CTA when the largest system solved has at
  *     most 40000 nonzeros plus eight per row (the FP64 work of one iteration
  *     that one SM does faster than the phase kernels' fixed cost per
- *     iteration), or a batched solve has at least 2 systems per SM; else
- *     PHASES.  One system of at most 3,145,728 rows whose plan is automatic
+ *     iteration), or a batched solve has at least 2 systems per SM; with an
+ *     automatic plan (textbook form, no host_loop) also for refined solves of
+ *     systems of at most 120000 such operations, and for batches of systems of
+ *     at most 80,000 rows whose rows fill half the SMs with systems of the
+ *     largest one's size; else PHASES.  One system of at most 3,145,728 rows whose plan is automatic
  *     runs FP64 CG (textbook form, no host_loop) as one launch of a team of
  *     CTAs -- a thread-block cluster, or one CTA per SM launched
  *     cooperatively, whose bounded waits (about a second) end the solve with
  *     GBS_ERR_TIMEOUT -- with the same iteration up to reduction order; a
- *     batched solve of fewer than two systems per SM likewise gives each
- *     system a cluster (systems of up to 163,840 rows), from a queue;
+ *     batched solve of fewer than two systems per SM, and of fewer rows than
+ *     would fill every SM with systems of the largest one's size, likewise
+ *     gives each system a cluster (systems of up to 163,840 rows), from a queue;
  *     ksp_result.solver names the solver it stands in for, and phase times
  *     are reported as for the phase kernels.
  * ksp_result.solver tells which one ran.  No synchronisation.

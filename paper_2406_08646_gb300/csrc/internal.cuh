@@ -30,6 +30,8 @@ constexpr uint64_t POOL_KEEP_BYTES = 32ull << 30;
 // The per-CTA solver's automatic size rule: systems of at most this many
 // FP64 operations per iteration (nonzeros plus eight per row; pcg.cu).
 constexpr int64_t CTA_AUTO_WORK = 40000;
+constexpr int64_t CTA_AUTO_WORK32 = 120000;  // ... of a refined solve's
+constexpr int64_t CTA_BATCH_ROWS = 80000;    // ... and a full batch's largest system
 int dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s);
 void dev_free(void *p, cudaStream_t s);
 template <typename T>

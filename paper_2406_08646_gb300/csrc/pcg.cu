@@ -546,12 +546,40 @@ int sm_count(gbs_mat A) {
   return nsm;
 }
 
-bool use_cta_solver(gbs_mat A, bool per_system) {
+// With an automatic plan (and no host loop, no single-reduction form) the
+// per-CTA solver also takes
+//   refined solves of systems of up to CTA_AUTO_WORK32 operations: an FP32
+//     iteration costs an SM about a third of an FP64 one, the phase kernels no
+//     less time.  Measured, ms, phases / this: 2D 64^2 (53k operations) 5.12 /
+//     2.50, 80^2 (83k) 6.66 / 4.93, 3D 20^3 (118k) 2.14 / 1.95, 2D 100^2 (130k)
+//     8.37 / 8.53, Q1 16^3 (157k) 1.33 / 1.39, 3D 24^3 (205k) 2.37 / 3.73;
+//   batches whose rows would fill half the SMs with systems of the largest
+//     one's size, if that has at most CTA_BATCH_ROWS (the largest measured): a
+//     phase's time grows with the batch, this one's is the largest system's.
+//     Measured, ms, phases / this, at n systems (rows over the largest's rows
+//     in brackets): refined 100 of 10k-20k (75) 53 / 41, of 20k-40k (75) 117 /
+//     116, 160 of 3k-10k 33 / 15, 160 of 30k-80k (110) 462 / 352, 220 of 10k-30k
+//     140 / 81; FP64 160 of 500-3k (93) 10.4 / 5.6, 300 13.7 / 5.8, of 8k-12k
+//     (250) 94 / 46, 160 of 30k-80k 586 / 520; below the line refined 40 of
+//     10k-20k (30) 33 / 38, 20 of 20k-40k 39 / 100.
+static bool cta_auto_rule(gbs_mat A, bool per_system, const ksp_opts &o) {
+  const bool refined = o.precision == GBS_FP32_REFINED;
+  if (o.method != GBS_KSP_CG || o.host_loop || !A->plan_auto ||
+      (!refined && A->cg_form != GBS_CG_TEXTBOOK))
+    return false;
+  const int64_t nz = per_system ? A->max_sys_nnz : A->nnz;
+  const int64_t rows = per_system ? A->max_sys_rows : A->nrows;
+  if (refined && nz + 8 * rows <= CTA_AUTO_WORK32) return true;
+  return per_system && rows <= CTA_BATCH_ROWS && 2 * A->nrows >= rows * sm_count(A);
+}
+
+bool use_cta_solver(gbs_mat A, bool per_system, const ksp_opts &o) {
   const int32_t sv = solver_for(A, per_system);
   if (sv == GBS_SOLVER_CTA) return true;
   if (sv == GBS_SOLVER_PHASES || A->lanes != GBS_SPMV_SELL) return false;
   if (sv == GBS_SOLVER_SPLIT && per_system) return false;  // solve() splits the batch
-  return cta_size_rule(A, per_system, 2);  // two 1024-thread PCG CTAs fit an SM
+  return cta_size_rule(A, per_system, 2) ||  // two 1024-thread PCG CTAs fit an SM
+         (sv == GBS_SOLVER_AUTO && cta_auto_rule(A, per_system, o));
 }
 
 int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,
@@ -566,7 +594,7 @@ int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_sys
   const bool split =
       per_system && solver_for(A, per_system) == GBS_SOLVER_SPLIT && A->lanes == GBS_SPMV_SELL;
   if (!refined && A->cg_form != GBS_CG_TEXTBOOK && A->lanes == GBS_SPMV_SELL && !split &&
-      !use_cta_solver(A, per_system)) {
+      !use_cta_solver(A, per_system, o)) {
     ksp_opts sr = o;
     sr.method = GBS_KSP_CGSR;
     return solve_krylov(A, b, x, sr, per_system, s);
@@ -586,11 +614,14 @@ int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_sys
     bool ran = false;
     GBS_TRY(solve_team(A, b, x, o, per_system, s, &ran));
     if (ran) {
-      A->last_solver = use_cta_solver(A, per_system) ? GBS_SOLVER_CTA : GBS_SOLVER_PHASES;
+      A->last_solver = solver_for(A, per_system) == GBS_SOLVER_AUTO &&
+                               cta_size_rule(A, per_system, 2)
+                           ? GBS_SOLVER_CTA
+                           : GBS_SOLVER_PHASES;
       return GBS_OK;
     }
   }
-  if (use_cta_solver(A, per_system)) {
+  if (use_cta_solver(A, per_system, o)) {
     if (A->lanes != GBS_SPMV_SELL) {
       set_error("the per-CTA solver needs the sliced-ELL row products (plan kernel)");
       return GBS_ERR_ARG;

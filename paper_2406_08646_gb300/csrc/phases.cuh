@@ -123,7 +123,7 @@ int run_loop_stepped(const LoopPlan &P, PcgArgs a, int grid_a, int grid_e, int64
                      DevCtl *ctl, cudaStream_t s);
 int run_loop(gbs_mat A, const LoopPlan &P, int kind, const PcgArgs &a, const double *b,
              double *x, const ksp_opts &o, bool per_system, cudaStream_t s);
-bool use_cta_solver(gbs_mat A, bool per_system);
+bool use_cta_solver(gbs_mat A, bool per_system, const ksp_opts &o);
 int32_t split_count(gbs_mat A);
 // The per-CTA solver's automatic choice: the largest system solved has at
 // most CTA_AUTO_WORK nonzeros plus eight per row, or a batch gives every SM

@@ -737,12 +737,17 @@ constexpr int64_t TEAM_GRID_ROWS = 3 << 20;
 // solver and plan.)  Measured, ms, on edge-diffusion systems, half 2D, half 3D,
 // phase kernels -> clusters: 4 systems of 1k-8k rows 6.0 -> 2.6, 8 of 2k-20k
 // 13.2 -> 8.7, 40 of 500-3k 6.2 -> 3.3, 64 of 1k-20k 32.3 -> 27.7, 100 of 1k-3k
-// 9.5 -> 4.5, 150 of 1k-20k 67.7 -> 49.9, 200 of 5k-20k 96.6 -> 53.3.  From two
-// systems an SM on the per-CTA solver keeps every SM busy with no meetings (512
-// of 1k-20k: 82 ms against 105 on clusters of two).
+// 9.5 -> 4.5, 150 of 1k-20k 67.7 -> 49.9, 200 of 5k-20k 96.6 -> 53.3.  A batch
+// whose rows fill every SM with systems of the largest one's size keeps the
+// SMs busy on the per-CTA solver, with no meetings (ms on clusters / there, rows
+// over the largest's rows in brackets: 200 of 5k-20k (125) 54 / 67, 250 (156) 67 /
+// 68, 300 of 10k-30k (200) 164 / 130, of 8k-12k (250) 59 / 46), as does one of two
+// systems an SM (512 of 1k-20k: 105 / 71).
 constexpr int64_t TEAM_BATCH_ROWS = 10240;
 static int team_clusters(gbs_mat A) {
-  if (A->nsys < 2 || A->nsys >= 2 * sm_count(A) || A->nrows == 0) return 1;
+  if (A->nsys < 2 || A->nsys >= 2 * sm_count(A) || A->nrows == 0 ||
+      A->nrows >= A->max_sys_rows * sm_count(A))
+    return 1;
   int size = 1;
   while (size < TEAM_MAX_CLUSTER && ((int64_t)A->nsys * size < sm_count(A) ||
                                      A->max_sys_rows > TEAM_BATCH_ROWS * size))

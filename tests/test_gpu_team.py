@@ -228,3 +228,41 @@ def test_batch_statuses():
     assert [r["status"] for r in rs] == [B.ERR_TIMEOUT, B.OK] + [B.ERR_TIMEOUT] * 3
     assert all(r["iterations"] <= 1 for r in rs)
     A.close()
+
+
+FULL = [(60, 60)] * 100 + [(59, 61)] * 54 + [(1023, 1), (1025, 1), (31, 33), (33, 1), (1, 1), (0, 5)]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "refined"])
+@pytest.mark.parametrize("name, shapes, solver", [
+    ("full", FULL, "CTA"),              # rows for more than half the SMs of the largest's size
+    ("one large", [(10, 10)] * 159 + [(110, 100)], "PHASES"),
+])
+def test_batch_choice(name, shapes, solver, precision):
+    """Automatic choice for batches of one to two systems an SM (the large one of the
+    second batch: FP64 takes a cluster, reported as the phase kernels' choice)."""
+    A, O, off, b = batch_of(shapes, 7)
+    kw = dict(rtol=1e-10, precision=B.FP32_REFINED if precision == "refined" else B.FP64)
+    x, rs = A.solve_batched(t(b), **kw)
+    resid = b - oracle.spmv(O, x.cpu().numpy())
+    for s, r in enumerate(rs):
+        sl = slice(off[s], off[s + 1])
+        assert r["status"] == B.OK and r["solver"] == getattr(B, "SOLVER_" + solver), (s, r)
+        assert np.linalg.norm(resid[sl]) <= 1.05e-10 * np.linalg.norm(b[sl])
+    x2, rs2 = A.solve_batched(t(b), **kw)
+    assert torch.equal(x, x2) and rs == rs2
+    A.set_solver(B.SOLVER_PHASES)
+    _, rs = A.solve_batched(t(b), **kw)
+    assert all(r["status"] == B.OK and r["solver"] == B.SOLVER_PHASES for r in rs)
+    A.close()
+
+
+@pytest.mark.parametrize("n, solver", [(64, "CTA"), (86, "CTA"), (110, "PHASES")])
+def test_refined_choice(n, solver):
+    g = grid((n, n), n)
+    A, O = make(*g)
+    b = np.random.default_rng(n).standard_normal(n * n)
+    x, r = A.solve(t(b), rtol=1e-10, precision=B.FP32_REFINED)
+    assert r["status"] == B.OK and r["solver"] == getattr(B, "SOLVER_" + solver)
+    assert np.linalg.norm(b - oracle.spmv(O, x.cpu().numpy())) <= 1.05e-10 * np.linalg.norm(b)
+    A.close()
