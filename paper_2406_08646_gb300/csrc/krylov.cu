@@ -94,12 +94,20 @@ __device__ __forceinline__ void kry_rows(const KrylovArgs &a, const KSys &g, con
 }
 
 // ... with the consumer's own operands loaded ahead of each row's sum, or with it.
+// NP > 2 pairs in flight (sell_rows_deep) pay from a few slices a warp on: BiCG,
+// ms with two / three / four pairs: 78 systems of 767-2,866 rows 5.17 / 5.23 /
+// 5.31, 200 of 1k-5k 10.78 / 10.44 / 10.50, 256 of 1k-20k 86.8 / 77.4 / 78.2.
+// (TFQMR, whose consumers hold more operands: 5.28 / 5.53 / 5.57, 10.5 / 11.0 /
+// 11.1, 76.5 / 74.8 / 76.0: two.)
+constexpr int KRY_DEEP_SLICES = 96;
 template <bool AHEAD, int NP, class L, class F>
 __device__ __forceinline__ void kry_rows(const KrylovArgs &a, const KSys &g, const SellView &S,
                                          const double *sval, const double *x, L load, F use) {
   if constexpr (AHEAD) {
     RowFn<L &, F &> f{load, use};
-    if (a.stream_matrix) sell_rows<double, true, GATHER_CA, false, NP>(S, sval, x, g.s0, g.s1, f);
+    if (NP == 2 || g.s1 - g.s0 <= KRY_DEEP_SLICES) kry_rows(a, g, S, sval, x, f);
+    else if (a.stream_matrix)
+      sell_rows<double, true, GATHER_CA, false, NP>(S, sval, x, g.s0, g.s1, f);
     else sell_rows<double, false, GATHER_CA, false, NP>(S, sval, x, g.s0, g.s1, f);
   } else {
     auto f = [&](int i, double y) {
@@ -238,14 +246,14 @@ __device__ void kry_bicg(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
     // q = A p with pt.q, qt = A^T pt
     double sg[1] = {0.0};
     double pti;
-    kry_rows<AHEAD, 4>(
+    kry_rows<AHEAD, 3>(
         a, g, a.sv, a.sval, p, [&](int i) { pti = pt[i]; },
         [&](int i, double y) {
           q[i] = y;
           sg[0] = fma(pti, y, sg[0]);
         });
     auto fqt = [&](int i, double y) { qt[i] = y; };
-    kry_rows<AHEAD, 4>(a, g, a.tv, a.tval, pt, [](int) {}, fqt);
+    kry_rows<AHEAD, 3>(a, g, a.tv, a.tval, pt, [](int) {}, fqt);
     cta_sum0<double, 1>(sg, sh);
     if (t0) {
       ++it;
@@ -511,14 +519,14 @@ __device__ void kry_tfqmr(const KrylovArgs &a, const KSys &g, CtaShared &sh) {
 // so every pass waits on its loads' latency.  A pass that stores a row's
 // values between its loads keeps the compiler from moving the loads together
 // (the pointers may alias), so a row's operands are loaded before its first
-// store, in the products before the row's sum (AHEAD; BiCG's products with
-// four pairs in flight), and thread 0's scalars live in shared memory to free
+// store, in the products before the row's sum (AHEAD; BiCG's products of larger
+// systems with three pairs in flight), and thread 0's scalars live in shared memory to free
 // registers for them.  At two CTAs per SM the registers do not allow it: BiCG
 // keeps its scalars local and its passes' loads spread out.  Every thread adds
 // the same rows in the same order either way.  Measured, ms (systems x rows):
 //                              before   this
 //   TFQMR 256 x 1k-20k           97.8   76.5
-//   BiCG  256 x 1k-20k           99.5   78.1
+//   BiCG  256 x 1k-20k           99.5   77.5
 //   BiCG  152 x 15k-20k         105.5   81.2
 //   TFQMR 1024 x 500-4k (two)    23.1   21.7
 //   BiCG  512 x 1k-8k (two)      34.9   34.2

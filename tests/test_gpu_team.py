@@ -266,3 +266,22 @@ def test_refined_choice(n, solver):
     assert r["status"] == B.OK and r["solver"] == getattr(B, "SOLVER_" + solver)
     assert np.linalg.norm(b - oracle.spmv(O, x.cpu().numpy())) <= 1.05e-10 * np.linalg.norm(b)
     A.close()
+
+
+@pytest.mark.parametrize("method", ["BICG", "TFQMR"])
+def test_nonsymmetric_batch_sizes(method):
+    """Per-CTA BiCG and TFQMR on systems around the size (96 slices) from which BiCG's
+    products keep more pairs in flight, and on far smaller ones; the bar of the
+    nonsymmetric solvers' tests (twice rtol)."""
+    A, O, off, b = batch_of([(37, 83), (48, 64), (7, 439), (32, 97), (64, 70), (5, 8), (1, 1)], 5)
+    A.set_solver(B.SOLVER_CTA)
+    kw = dict(rtol=1e-9, method=getattr(B, "KSP_" + method))
+    x, rs = A.solve_batched(t(b), **kw)
+    resid = b - oracle.spmv(O, x.cpu().numpy())
+    for s, r in enumerate(rs):
+        sl = slice(off[s], off[s + 1])
+        assert r["status"] == B.OK and r["solver"] == B.SOLVER_CTA, (s, r)
+        assert np.linalg.norm(resid[sl]) <= 2e-9 * np.linalg.norm(b[sl]), s
+    x2, rs2 = A.solve_batched(t(b), **kw)
+    assert torch.equal(x, x2) and rs == rs2
+    A.close()
