@@ -712,11 +712,13 @@ __device__ __forceinline__ void sell_rows_pat(const SellView &S, const T *__rest
 // thread: the next slice's bounds, pattern and masks are loaded while the
 // current slice is summed, a step issues the loads of NP pairs (offsets,
 // values, gathers) before its first FMA, and the odd last entry's loads go
-// out before the first step.  An absent entry gathers the slice's first row,
-// whose value its FMA then does not use, so no load waits on a branch.
+// out before the first step.  An absent entry gathers x at the slice's first
+// row, or at `last` (x's last index) where the matrix has more rows than x has
+// elements; its FMA does not use the value, so no load waits on a branch.
+// none: that element's place from the lane's own row.
 template <int N, typename T, bool STREAM, int NC, bool SM>
 __device__ __forceinline__ void sell_step(const typename Pair<T>::type *v2,
-                                          const int2 *pat2, const T *xr, uint32_t mk, int lane,
+                                          const int2 *pat2, const T *xr, uint32_t mk, int none,
                                           T &acc) {
   typename Pair<T>::type v[N];
   int2 o[N];
@@ -728,8 +730,8 @@ __device__ __forceinline__ void sell_step(const typename Pair<T>::type *v2,
   }
 #pragma unroll
   for (int j = 0; j < N; ++j) {
-    g[2 * j] = ld_x<NC>(xr + ((mk >> (2 * j)) & 1u ? o[j].x : -lane));
-    g[2 * j + 1] = ld_x<NC>(xr + ((mk >> (2 * j + 1)) & 1u ? o[j].y : -lane));
+    g[2 * j] = ld_x<NC>(xr + ((mk >> (2 * j)) & 1u ? o[j].x : none));
+    g[2 * j + 1] = ld_x<NC>(xr + ((mk >> (2 * j + 1)) & 1u ? o[j].y : none));
   }
 #pragma unroll
   for (int j = 0; j < N; ++j) {
@@ -742,7 +744,7 @@ __device__ __forceinline__ void sell_step(const typename Pair<T>::type *v2,
 
 template <typename T, bool STREAM, int NC, bool SM, int NP, class F>
 __device__ __forceinline__ void sell_rows_deep(const SellView &S, const T *__restrict__ sval,
-                                               const T *x, int s0, int s1, F &f) {
+                                               const T *x, int s0, int s1, F &f, int last) {
   typedef typename Pair<T>::type P;
   const int lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
   int sl = s0 + (int)(threadIdx.x >> 5);
@@ -765,6 +767,7 @@ __device__ __forceinline__ void sell_rows_deep(const SellView &S, const T *__res
     }
     row_loads(f, r + lane, re);
     const int w = (b1 - b0) >> 5;
+    const int none = min(r, last) - (r + lane);
     const T *xr = x + r + lane;
     const P *v2 = reinterpret_cast<const P *>(sval) + (b0 >> 1) + lane;
     const int2 *pat2 = reinterpret_cast<const int2 *>(S.pool + p0);
@@ -773,17 +776,17 @@ __device__ __forceinline__ void sell_rows_deep(const SellView &S, const T *__res
     if (w & 1) {
       const int o = ld_meta<SM>(S.pool + p0 + w - 1);
       vo = ld_entry<STREAM, SM>(sval + (b1 - 32 + lane));
-      xo = ld_x<NC>(xr + (odd ? o : -lane));
+      xo = ld_x<NC>(xr + (odd ? o : none));
     }
     T acc = T(0);
     int m = w >> 1;
     for (; m >= NP; m -= NP, v2 += 32 * NP, pat2 += NP, mk >>= 2 * NP)
-      sell_step<NP, T, STREAM, NC, SM>(v2, pat2, xr, mk, lane, acc);
+      sell_step<NP, T, STREAM, NC, SM>(v2, pat2, xr, mk, none, acc);
     if (NP > 2 && m >= 2) {
-      sell_step<2, T, STREAM, NC, SM>(v2, pat2, xr, mk, lane, acc);
+      sell_step<2, T, STREAM, NC, SM>(v2, pat2, xr, mk, none, acc);
       m -= 2, v2 += 64, pat2 += 2, mk >>= 4;
     }
-    if (m > 0) sell_step<1, T, STREAM, NC, SM>(v2, pat2, xr, mk, lane, acc);
+    if (m > 0) sell_step<1, T, STREAM, NC, SM>(v2, pat2, xr, mk, none, acc);
     const T t = fma_rn(vo, xo, acc);
     acc = odd ? t : acc;
     if (r + lane < re) f(r + lane, acc);
@@ -798,11 +801,13 @@ __device__ __forceinline__ void sell_rows_deep(const SellView &S, const T *__res
   }
 }
 
+// last: x's last index, for matrices that may have more rows than columns.
 template <typename T, bool STREAM, int NC, bool SM = false, int NP = 2, class F>
 __device__ __forceinline__ void sell_rows(const SellView &S, const T *__restrict__ sval,
-                                          const T *x, int s0, int s1, F &f) {
+                                          const T *x, int s0, int s1, F &f,
+                                          int last = INT32_MAX) {
   if (S.pat) {
-    if constexpr (NP > 2) sell_rows_deep<T, STREAM, NC, SM, NP>(S, sval, x, s0, s1, f);
+    if constexpr (NP > 2) sell_rows_deep<T, STREAM, NC, SM, NP>(S, sval, x, s0, s1, f, last);
     else sell_rows_pat<T, STREAM, NC, SM>(S, sval, x, s0, s1, f);
     return;
   }

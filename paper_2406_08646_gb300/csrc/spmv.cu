@@ -114,13 +114,13 @@ constexpr double DEEP_WIDTH = 6.0;
 __global__ void __launch_bounds__(PHASE_TPB, DEEP_CTAS)
     k_spmv_sell_deep(const SellView S, const double *__restrict__ sval,
                      const double *__restrict__ x, double *__restrict__ y, int32_t nslices,
-                     int32_t stream_matrix) {
+                     int32_t ncols, int32_t stream_matrix) {
   auto f = [&](int r, double s) { y[r] = s; };
   const int s0 = (int)((int64_t)nslices * blockIdx.x / gridDim.x);
   const int s1 = (int)((int64_t)nslices * (blockIdx.x + 1) / gridDim.x);
   if (stream_matrix)
-    sell_rows<double, true, GATHER_NC, false, 4>(S, sval, x, s0, s1, f);
-  else sell_rows<double, false, GATHER_NC, false, 4>(S, sval, x, s0, s1, f);
+    sell_rows<double, true, GATHER_NC, false, 4>(S, sval, x, s0, s1, f, ncols - 1);
+  else sell_rows<double, false, GATHER_NC, false, 4>(S, sval, x, s0, s1, f, ncols - 1);
 }
 
 int launch_spmv(gbs_mat A, const double *x, double *y, cudaStream_t s) {
@@ -135,7 +135,7 @@ int launch_spmv(gbs_mat A, const double *x, double *y, cudaStream_t s) {
                       (double)A->sell_nnz >= 32.0 * DEEP_WIDTH * (double)ns;
     if (deep)
       k_spmv_sell_deep<<<(unsigned)wave, PHASE_TPB, 0, s>>>(
-          sell_view(A), A->sell_val, x, y, (int32_t)ns, stream_matrix(A, 12));
+          sell_view(A), A->sell_val, x, y, (int32_t)ns, (int32_t)A->ncols, stream_matrix(A, 12));
     else
       k_spmv_sell<<<(unsigned)std::min<int64_t>(ctas, 1 << 20), PHASE_TPB, 0, s>>>(
           sell_view(A), A->sell_val, x, y, (int32_t)ns, stream_matrix(A, 12));
