@@ -633,6 +633,7 @@ __global__ void __launch_bounds__(TPB, 1) k_team(PcgArgs a, const __grid_constan
     sh.call = *a.call;
   }
   __syncthreads();
+  if (!GRID && size > 1) cluster_meet();  // every CTA runs before its shared memory is written
   team_system<GRID>(a, cfg, sh, reinterpret_cast<double *>(team_smem), cta_system(a, 0), rank,
                     size, true);
   if (!GRID && size > 1) cluster_meet();  // no CTA leaves while others may write to its boxes
@@ -691,6 +692,7 @@ __global__ void __launch_bounds__(TPB, 1)
   __syncthreads();
   if (threadIdx.x == 0) sh.next = (int)cluster;
   __syncthreads();
+  cluster_meet();  // every CTA runs before its shared memory is written
   while (sh.next < a.cta_n) {
     {
       const SysRange sys = cta_system(a, sh.next);
