@@ -96,7 +96,10 @@ struct TeamShared {
   int next;                                 //   and the system the cluster solves
 };
 
+// (The aligned forms want the whole warp at once: callers come from code that some of
+// its lanes skip.)
 __device__ __forceinline__ void cluster_meet() {
+  __syncwarp();
   asm volatile(
       "barrier.cluster.arrive.release.aligned;\n\t"
       "barrier.cluster.wait.acquire.aligned;" ::
