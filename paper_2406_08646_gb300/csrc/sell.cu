@@ -239,12 +239,14 @@ void free_sell(gbs_mat A) {
   A->nslices = A->sell_nnz = 0;
 }
 
-// Slice table, column patterns chosen and padded size (no entries yet); when
-// the padded size reaches 2^31 only the size is recorded.  Idempotent.
-// Synchronises s once: the sums over the slices decide the sizes (the tables
-// themselves stay on the device).
-int sell_shape(gbs_mat A, cudaStream_t st) {
-  if (A->sell_row0) return GBS_OK;
+// ... after a failed step, once the steps before it are done with the arrays.
+static void drop_copy(gbs_mat A, cudaStream_t s) {
+  cudaStreamSynchronize(s);
+  free_sell(A);
+}
+
+// The slice table, the column patterns chosen and the padded size.
+static int shape_copy(gbs_mat A, cudaStream_t st) {
   A->sell_slice0_h.assign(A->nsys + 1, 0);
   for (int32_t q = 0; q < A->nsys; ++q)
     A->sell_slice0_h[q + 1] =
@@ -255,8 +257,8 @@ int sell_shape(gbs_mat A, cudaStream_t st) {
   // w, u (ns + 1 words each, 16-byte aligned), the sums, a batch's first rows and slices
   const int64_t pad = (ns + 4) & ~(int64_t)3, nsy = A->nsys > 1 ? 2 * (A->nsys + 1) : 0;
   uint32_t *d = nullptr;
-  int32_t *row0 = nullptr;
-  GBS_TRY(dev_alloc(&row0, ns + 1, st));
+  GBS_TRY(dev_alloc(&A->sell_row0, ns + 1, st));
+  int32_t *const row0 = A->sell_row0;
   if (ns == 0) {
     const int32_t end = (int32_t)A->nrows;
     GBS_TRY_CUDA(cudaMemcpyAsync(row0, &end, sizeof(end), cudaMemcpyHostToDevice, st));
@@ -271,7 +273,6 @@ int sell_shape(gbs_mat A, cudaStream_t st) {
   uint32_t *w = d, *u = d + pad;
   ShapeSums *sums = reinterpret_cast<ShapeSums *>(d + 2 * pad);
   int32_t *sys = nsy ? reinterpret_cast<int32_t *>(sums + 1) : nullptr;
-  A->sell_row0 = row0;
   if (ns > 0) {
     GBS_TRY_CUDA(cudaMemsetAsync(sums, 0, sizeof(ShapeSums), st));
     if (sys) {
@@ -323,6 +324,38 @@ int sell_shape(gbs_mat A, cudaStream_t st) {
   return GBS_OK;
 }
 
+// Slice table, column patterns chosen and padded size (no entries yet); when
+// the padded size reaches 2^31 only the size is recorded.  Idempotent.
+// Synchronises s once: the sums over the slices decide the sizes (the tables
+// themselves stay on the device).  sell_row0 and sell_val say that the shape
+// and the copy exist: where a step fails, what the others made goes back, so
+// that the next call starts over instead of using half a copy.
+int sell_shape(gbs_mat A, cudaStream_t st) {
+  if (A->sell_row0) return GBS_OK;
+  const int status = shape_copy(A, st);
+  if (status != GBS_OK) drop_copy(A, st);
+  return status;
+}
+
+// The copy's arrays beyond its shape: column patterns' masks and offsets or
+// column indices, and the values if they are set.
+static int fill_copy(gbs_mat A, cudaStream_t s) {
+  const size_t m = (size_t)std::max<int64_t>(A->sell_nnz, 1);
+  GBS_TRY(dev_alloc(&A->sell_val, m, s));
+  if (A->sell_npat == 0) {
+    if (A->col_span <= 32767) GBS_TRY(dev_alloc(&A->sell_off16, m, s));
+    else GBS_TRY(dev_alloc(&A->sell_col, m, s));
+  }
+  if (A->nslices > 0) {
+    k_sell_fill<double, true><<<grid_of(A->nslices * 32, 256), 256, 0, s>>>(
+        A->nslices, A->sell_ptr, A->sell_row0, A->row_ptr, A->col, (const double *)nullptr,
+        A->sell_npat ? A->sell_pat : nullptr, A->sell_pool, A->sell_mask, A->sell_col,
+        A->sell_off16, (double *)nullptr);
+    GBS_LAUNCHED(1);
+  }
+  return A->values_set ? sell_values(A, s) : GBS_OK;
+}
+
 // Column patterns or column indices and, if the values are set, FP64 values
 // of the sliced copy.  Column indices are stored as 16-bit offsets col - row
 // when every column lies within 2^15 - 1 of its row (the symbolic stage
@@ -334,23 +367,10 @@ int sell_build(gbs_mat A, cudaStream_t s) {
               (long long)A->sell_nnz);
     return GBS_ERR_ARG;
   }
-  if (!A->sell_val) {
-    const size_t m = (size_t)std::max<int64_t>(A->sell_nnz, 1);
-    GBS_TRY(dev_alloc(&A->sell_val, m, s));
-    if (A->sell_npat == 0) {
-      if (A->col_span <= 32767) GBS_TRY(dev_alloc(&A->sell_off16, m, s));
-      else GBS_TRY(dev_alloc(&A->sell_col, m, s));
-    }
-    if (A->nslices > 0) {
-      k_sell_fill<double, true><<<grid_of(A->nslices * 32, 256), 256, 0, s>>>(
-          A->nslices, A->sell_ptr, A->sell_row0, A->row_ptr, A->col, (const double *)nullptr,
-          A->sell_npat ? A->sell_pat : nullptr, A->sell_pool, A->sell_mask, A->sell_col,
-          A->sell_off16, (double *)nullptr);
-      GBS_LAUNCHED(1);
-    }
-    if (A->values_set) GBS_TRY(sell_values(A, s));
-  }
-  return GBS_OK;
+  if (A->sell_val) return GBS_OK;
+  const int status = fill_copy(A, s);
+  if (status != GBS_OK) drop_copy(A, s);
+  return status;
 }
 
 // FP64 values of the sliced copy from the CSR values (after every numeric
