@@ -600,7 +600,9 @@ int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_sys
     return solve_krylov(A, b, x, sr, per_system, s);
   }
   GBS_TRY(ensure_solver_workspace(A, refined, s));
-  if (refined && !A->val32_valid) GBS_TRY(launch_to_fp32(A, s));
+  // (a plan set after the last refined solve may have made the sliced copy since)
+  if (refined && (!A->val32_valid || (A->lanes == GBS_SPMV_SELL && !A->sell_val32)))
+    GBS_TRY(launch_to_fp32(A, s));
   A->last_count = per_system ? A->nsys : 1;
   A->last_ensemble = !per_system;
   A->trips_counted = true;
