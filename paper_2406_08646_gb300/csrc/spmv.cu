@@ -74,16 +74,21 @@ static int build_row_orders(gbs_mat A, cudaStream_t st) {
   const int64_t n = A->nrows;
   if (n == 0) return GBS_OK;
   if (!A->order_s) {
-    GBS_TRY(dev_alloc(&A->order_s, 2 * (size_t)n, st));
-    A->order_a = A->order_s + n;
+    int32_t *order = nullptr;
+    GBS_TRY(dev_alloc(&order, 2 * (size_t)n, st));
     const int32_t nb = (int32_t)((n + SPMV_ROWS - 1) / SPMV_ROWS);
     k_row_order<<<(unsigned)std::min(nb, 1 << 16), ORDER_W, 0, st>>>(
-        nb, nullptr, (int32_t)n, SPMV_ROWS, A->row_ptr, A->order_s);
-    GBS_LAUNCHED(1);
+        nb, nullptr, (int32_t)n, SPMV_ROWS, A->row_ptr, order);
+    count_launches(1);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) dev_free(order, st);
+    GBS_TRY_CUDA(e);
+    A->order_s = order;
   }
   k_row_order<<<(unsigned)std::min(std::max(A->ta.nblocks, 1), 1 << 16), ORDER_W, 0, st>>>(
-      A->ta.nblocks, A->ta.row0, (int32_t)n, ORDER_W, A->row_ptr, A->order_a);
+      A->ta.nblocks, A->ta.row0, (int32_t)n, ORDER_W, A->row_ptr, A->order_s + n);
   GBS_LAUNCHED(1);
+  A->order_a = A->order_s + n;
   return GBS_OK;
 }
 
@@ -388,6 +393,7 @@ int build_plan(gbs_mat A, int32_t Ra, int32_t Re, int32_t kernel, int32_t ctas_p
   free_table(A->sa);  // the size split's tables follow the plan
   free_table(A->se);
   A->split_built = 0;
+  A->order_a = nullptr;  // (it orders the rows of table A's blocks, which change below)
   if (kernel == GBS_SPMV_AUTO) {
     GBS_TRY(sell_shape(A, st));
     kernel = (A->sell_ptr && (double)A->sell_nnz_rows <= 1.2 * (double)A->nnz)
