@@ -107,15 +107,27 @@ __global__ void __launch_bounds__(PHASE_TPB, SELL_MIN_CTAS)
   }
 }
 
-// The same with 64 registers a thread on a grid of two CTAs an SM, each with
-// its run of slices: sell_rows_deep, which has four pairs a thread and the next
-// slice's tables in flight.  The FP64 pipe bounds both (Q1 96^3: 40 us of FMAs);
-// this one keeps it busier while slices are wide, and costs a little where they
-// are not (their loads are few, and four CTAs an SM overlap more of them).
-// Measured, us a call: Q1 96^3 49.5 -> 47.6, 64^3 20.5 -> 18.5, 3D 7-point 150^3
-// 59.5 -> 56.1, 2D 5-point 1024^2 18.6 -> 19.5: mean widths from DEEP_WIDTH on.
+// The same with 64 registers a thread on a grid of two CTAs an SM, one wave,
+// each with its run of slices: sell_rows_deep, which has four pairs a thread and
+// the next slice's tables in flight.  The FP64 pipe bounds wide slices in both
+// (Q1 96^3: 40 us of FMAs), HBM and the gathers' latency narrow ones.
+// k_spmv_sell's many small CTAs balance themselves and, four of them an SM, hide
+// more latency where slices are narrow, so this form is taken where it was
+// measured to be the faster one (deep_form).  Measured, us a product,
+// k_spmv_sell / this (waves of slices in brackets):
+//   27-point 60^3 (1.4) 14.5 / 15.9   64^3 (1.8) 19.1 / 16.6   72^3 (2.5) 25.0 / 23.3
+//            80^3 (3.4) 29.3 / 30.5   96^3 (5.9) 48.0 / 45.9   90^3 (4.8) 38.9 / 37.5
+//            102^3 (7.0) 52.1 / 55.3  120^3 (11.4) 85.7 / 87.2
+//            (mean of 18 sizes between 1.5 and 7 waves: 3% faster; 0.95 to 1.15)
+//   19-point 60^3 9.7 / 10.1   120^3 59.7 / 62.2   13-point 700^2 15.5 / 17.9   9-point 1000^2 20.1 / 24.1
+//   7-point  70^3 6.7 / 7.3    140^3 (208 MB) 40.2 / 41.2
+//            150^3 (256 MB) 52.8 / 50.3   170^3 83.3 / 76.4   192^3 118.5 / 112.5
+//   9-point 2000^2 (368 MB, near neighbours) 78.8 / 84.4
+//   27-point 65^3 followed by three times as many diagonal rows 19.1 / 44.3, by
+//            7-point 90^3 25.4 / 41.5
+// (The slices dealt to the CTAs in turns: the same mean, 0.97 to 1.12, 96^3 1% slower,
+// 7-point 150^3 54.0; the uneven ones 21.9 and 26.8, slower than k_spmv_sell still.)
 constexpr int DEEP_CTAS = 2;
-constexpr double DEEP_WIDTH = 6.0;
 __global__ void __launch_bounds__(PHASE_TPB, DEEP_CTAS)
     k_spmv_sell_deep(const SellView S, const double *__restrict__ sval,
                      const double *__restrict__ x, double *__restrict__ y, int32_t nslices,
@@ -128,18 +140,36 @@ __global__ void __launch_bounds__(PHASE_TPB, DEEP_CTAS)
   else sell_rows<double, false, GATHER_NC, false, 4>(S, sval, x, s0, s1, f, ncols - 1);
 }
 
+// Whether MatMult takes k_spmv_sell_deep.  Slices have to be alike (the largest
+// at most an eighth over the mean), or the CTAs' runs are not; then wide ones (24
+// entries a row and more) from 1.5 up to 7 waves, and narrow ones (6 to 12) of matrices
+// that stream from HBM (from 7/4 of the L2's size on) and gather from afar (8192
+// rows and more away).
+constexpr double DEEP_WIDTH = 6.0, DEEP_NARROW = 12.0, DEEP_WIDE = 24.0;
+constexpr int32_t DEEP_SPAN = 8192;
+static bool deep_form(gbs_mat A) {
+  const int64_t ns = A->nslices;
+  const double width = (double)A->sell_nnz / (32.0 * (double)ns);
+  if (A->sell_npat == 0 || width < DEEP_WIDTH ||
+      8.0 * (double)A->slice_max_nnz * (double)ns > 9.0 * (double)A->nnz)
+    return false;
+  const int64_t wave = (int64_t)DEEP_CTAS * sm_count(A) * (PHASE_TPB / 32);  // slices of a wave
+  if (width >= DEEP_WIDE) return 2 * ns >= 3 * wave && ns < 7 * wave;
+  if (width > DEEP_NARROW || A->col_span < DEEP_SPAN) return false;
+  int l2 = 0;
+  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, A->device);
+  return 4 * (8 * A->sell_nnz + 20 * A->nrows) >= 7 * (int64_t)l2;
+}
+
 int launch_spmv(gbs_mat A, const double *x, double *y, cudaStream_t s) {
   if (A->nrows == 0) return GBS_OK;
   const int32_t n = (int32_t)A->nrows;
   if (A->lanes == GBS_SPMV_SELL) {
     GBS_TRY(sell_build(A, s));  // a no-op once built
     const int64_t ns = A->nslices, per = PHASE_TPB / 32;
-    const int64_t ctas = (ns + per - 1) / per, wave = (int64_t)DEEP_CTAS * sm_count(A);
-    // (a full wave at least: fewer slices spread over more CTAs of the other)
-    const bool deep = A->sell_npat > 0 && ctas >= wave &&
-                      (double)A->sell_nnz >= 32.0 * DEEP_WIDTH * (double)ns;
-    if (deep)
-      k_spmv_sell_deep<<<(unsigned)wave, PHASE_TPB, 0, s>>>(
+    const int64_t ctas = (ns + per - 1) / per;
+    if (deep_form(A))
+      k_spmv_sell_deep<<<(unsigned)(DEEP_CTAS * sm_count(A)), PHASE_TPB, 0, s>>>(
           sell_view(A), A->sell_val, x, y, (int32_t)ns, (int32_t)A->ncols, stream_matrix(A, 12));
     else
       k_spmv_sell<<<(unsigned)std::min<int64_t>(ctas, 1 << 20), PHASE_TPB, 0, s>>>(
