@@ -194,6 +194,7 @@ struct gbs_mat_s {
   int32_t *sell_pool = nullptr;    // the patterns' offsets col - row
   uint32_t *sell_mask = nullptr;   // 32 nslices: pattern entries each row holds
   int32_t slice_max_nnz = 0, slice_max_coo = 0;  // largest nonzeros / COO entries of a slice
+  int32_t run_max_nnz = 0;         // one system: largest nonzeros of its slices' equal runs, one an SM
   int64_t sell_npat = 0;           // slices with a pattern (0 or nslices)
   int64_t sell_nnz_rows = 0;       // 32 x the slices' longest rows (the size without
                                    // patterns: the automatic plan's padding rule)
@@ -287,6 +288,7 @@ int symbolic(gbs_mat A, const int32_t *i, const int32_t *j, const int64_t *coo_o
 int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,
           cudaStream_t s);
 void free_handle(gbs_mat A);
+int sm_count(gbs_mat A);
 bool batch_teams(gbs_mat A);  // a batch whose systems would get a cluster each
 bool use_team(gbs_mat A, bool per_system, const ksp_opts &o);
 int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,

@@ -73,18 +73,19 @@ struct ShapeSums {
   unsigned long long w, u;  // longest rows; offset unions (33 at most each)
   int32_t over;             // a slice's union has more than 32 offsets
   int32_t nnz, coo;         // largest nonzeros and COO entries of a slice
-  int32_t pad;
+  int32_t run;              // largest nonzeros of a run of slices (one system, cut into nruns)
 };
 
 // One warp per slice: its first row (a batch's slices start at their system's
 // first row: sys holds nsys + 1 first rows, then nsys + 1 first slices), w[s] =
 // its longest row, u[s] = the size of its rows' offset union (33: more than
-// 32, or patterns not built); their sums over all slices.
+// 32, or patterns not built); their sums over all slices.  Block 0 also cuts one
+// system's slices into nruns equal runs, as team.cu does.
 constexpr int SHAPE_TPB = 256;
 __global__ void __launch_bounds__(SHAPE_TPB)
     k_slice_shape(int64_t nslices, int64_t nrows, int32_t nsys, const int32_t *__restrict__ sys,
                   const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                  const int32_t *__restrict__ jmap, int32_t patterns,
+                  const int32_t *__restrict__ jmap, int32_t patterns, int32_t nruns,
                   int32_t *__restrict__ srow0, uint32_t *__restrict__ w,
                   uint32_t *__restrict__ u, ShapeSums *sums) {
   __shared__ unsigned long long sw[SHAPE_TPB / 32], su[SHAPE_TPB / 32];
@@ -94,6 +95,15 @@ __global__ void __launch_bounds__(SHAPE_TPB)
   unsigned long long tw = 0, tu = 0;
   int32_t nz = 0, ne = 0;
   bool over = false;
+  if (!sys && blockIdx.x == 0) {
+    int32_t run = 0;
+    for (int k = threadIdx.x; k < nruns; k += SHAPE_TPB) {
+      const int64_t f = 32 * (nslices * k / nruns), e = 32 * (nslices * (k + 1) / nruns);
+      run = max(run, row_ptr[e < nrows ? e : nrows] - row_ptr[f < nrows ? f : nrows]);
+    }
+    run = __reduce_max_sync(0xffffffffu, run);
+    if (lane == 0) atomicMax(&sums->run, run);
+  }
   for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices; s += nw) {
     int64_t r0 = 32 * s, r1 = nrows;
     if (sys) {
@@ -286,7 +296,7 @@ static int shape_copy(gbs_mat A, cudaStream_t st) {
     }
     k_slice_shape<<<grid_of(ns * 32, SHAPE_TPB), SHAPE_TPB, 0, st>>>(
         ns, A->nrows, A->nsys, sys, A->row_ptr, A->col, A->jmap, A->sell_patterns ? 1 : 0,
-        row0, w, u, sums);
+        sm_count(A), row0, w, u, sums);
     GBS_LAUNCHED(1);
     GBS_TRY_CUDA(cudaMemcpyAsync(&h, sums, sizeof(h), cudaMemcpyDeviceToHost, st));
     GBS_TRY_CUDA(cudaStreamSynchronize(st));
@@ -298,6 +308,7 @@ static int shape_copy(gbs_mat A, cudaStream_t st) {
   A->sell_nnz_rows = 32 * (int64_t)h.w;
   A->slice_max_nnz = h.nnz;
   A->slice_max_coo = h.coo;
+  A->run_max_nnz = h.run;
   A->nslices = ns;
   A->sell_nnz = total;
   if (total > 2147483647LL) return GBS_OK;  // too large for 32-bit offsets: no copy

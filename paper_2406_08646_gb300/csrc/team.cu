@@ -735,6 +735,34 @@ constexpr int64_t TEAM_CLUSTER_WORK = 160000;
 // hide HBM's latency better than the saved meetings are worth (3D 7-point,
 // us an iteration on team / phases: 128^3 70.4 / 72.9, 160^3 141.6 / 134.0).
 constexpr int64_t TEAM_GRID_ROWS = 3 << 20;
+// A team's CTA owns one run of slices, alone on its SM, where the phase kernels'
+// four CTAs an SM take blocks from four places of the matrix: where the rows'
+// lengths differ from place to place the team waits for its longest run.  That
+// pays while the longest has at most a quarter over the mean's nonzeros, or its
+// excess takes less of the FP64 pipe than the phase kernels' boundaries (28,000
+// FMAs: 7 us) on a system of up to 2^20 rows.  Measured, us an iteration on team /
+// phases (27-point rows followed by diagonal or 7-point ones; the longest run over
+// the mean, its excess): 200k rows 1.36 (10k) 24.9 / 29.3, 2.0 (18k) 24.8 / 26.8,
+// 7.7 (30k) 22.3 / 24.0; 600k 1.25 50.7 / 55.0, 1.34 (27k) 50.5 / 54.6, 1.62 (41k)
+// 50.0 / 48.2, 2.29 (59k) 47.8 / 46.2, 7.7 (90k) 46.7 / 35.1; 1.5M 1.24 104.7 / 105.9,
+// 1.60 105.2 / 93.6; 7-point rows followed by 5-point ones 600k 1.34 (8k) 27.1 / 31.2,
+// 1.5M 1.17 53.1 / 54.2, 1.34 (18k) 58.0 / 53.4.
+constexpr int64_t TEAM_EXCESS = 28000, TEAM_EXCESS_ROWS = 1 << 20;
+// Without column patterns (gathers from anywhere, columns to read) only while
+// matrix and vectors keep to half of L2: random columns, 9 a row, 400k rows
+// (59 MB) 30.8 / 34.1, 550k (81) 42.6 / 42.2, 850k 63.1 / 56.1; 25 a row 150k 26.1 /
+// 30.2, 450k 69.3 / 65.9; 3D edges 300k 20.0 / 25.0, 1M (110) 51.8 / 47.0, 3M 131 / 106.
+static bool team_suits(gbs_mat A) {
+  const int64_t n = A->nrows, run = A->run_max_nnz, sms = sm_count(A);
+  if (n > TEAM_GRID_ROWS) return false;
+  if (4 * run * sms > 5 * A->nnz &&
+      (n > TEAM_EXCESS_ROWS || run - A->nnz / sms > TEAM_EXCESS))
+    return false;
+  if (A->sell_npat > 0) return true;
+  int l2 = 0;
+  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, A->device);
+  return 2 * (A->sell_nnz * (A->col_span <= 32767 ? 10 : 12) + 40 * n) <= (int64_t)l2;
+}
 
 // CTAs a system of a batch gets: the smallest cluster that gives every SM work
 // and the largest system's CTAs at most TEAM_BATCH_ROWS rows each, so that most
@@ -779,7 +807,7 @@ bool use_team(gbs_mat A, bool per_system, const ksp_opts &o) {
       o.host_loop || A->lanes != GBS_SPMV_SELL || A->nrows == 0)
     return false;
   return A->team_tuned || (A->solver == GBS_SOLVER_AUTO && A->cg_form == GBS_CG_TEXTBOOK &&
-                           A->plan_auto && A->nrows <= TEAM_GRID_ROWS);
+                           A->plan_auto && team_suits(A));
 }
 
 // The team of a solve on A: its CTAs, their threads and their shared memory.
