@@ -415,21 +415,31 @@ int mat_get_plan(gbs_mat A, int32_t *spmv_rows, int32_t *update_rows, int32_t *k
  *   GBS_SOLVER_AUTO (default): CTA when the largest system solved has at
  *     most 40000 nonzeros plus eight per row (the FP64 work of one iteration
  *     that one SM does faster than the phase kernels' fixed cost per
- *     iteration), or a batched solve has at least 2 systems per SM; with an
- *     automatic plan (textbook form, no host_loop) also for refined solves of
- *     systems of at most 120000 such operations, and for batches of systems of
- *     at most 80,000 rows whose rows fill half the SMs with systems of the
- *     largest one's size; else PHASES.  One system of at most 3,145,728 rows whose plan is automatic
- *     runs FP64 CG (textbook form, no host_loop) as one launch of a team of
- *     CTAs -- a thread-block cluster, or one CTA per SM launched
- *     cooperatively, whose bounded waits (about a second) end the solve with
- *     GBS_ERR_TIMEOUT -- with the same iteration up to reduction order; a
- *     batched solve of fewer than two systems per SM, and of fewer rows than
- *     would fill every SM with systems of the largest one's size, likewise
- *     gives each system a cluster (systems of up to 163,840 rows), from a queue;
- *     ksp_result.solver names the solver it stands in for, and phase times
- *     are reported as for the phase kernels.
- * ksp_result.solver tells which one ran.  No synchronisation.
+ *     iteration), or a batched solve has at least 2 systems per SM; else
+ *     PHASES.  With an automatic plan, the textbook form and no host_loop it
+ *     also chooses among
+ *       - CTA for refined solves of systems of at most 120000 such operations;
+ *       - teams of CTAs for FP64 CG on one system of at most 3,145,728 rows:
+ *         every iteration in one launch, on a thread-block cluster (up to
+ *         160000 operations) or on one CTA per SM.  Systems whose rows' lengths
+ *         differ much from place to place, or whose columns are scattered
+ *         beyond half of L2, stay on PHASES;
+ *       - for a batch of fewer than 2 systems per SM, by an estimate of each
+ *         one's time from the systems' rows and nonzeros: PHASES, CTA and, for
+ *         FP64 CG, a cluster per system from a queue or a share of one grid's
+ *         CTAs per system.
+ * Teams run the same iteration up to reduction order.  A team of one CTA per SM
+ * (one system's, or a batch's shared grid) is launched cooperatively and takes
+ * every SM until the solve ends: solves on several streams then run one after
+ * another, where PHASES lets them overlap -- set it for handles that are solved
+ * at the same time on streams of their own (four systems of 40,000 rows at once:
+ * 4.0 ms on PHASES, 7.3 on teams, which take 1.8 for one alone against 3.4).  Its
+ * waits are bounded; should one last over a second the solve ends with
+ * GBS_ERR_TIMEOUT, whatever timeout_ns, and x is undefined.
+ * ksp_result.solver is the solver that ran; for a team, the one that AUTO would
+ * take without teams (PHASES, or CTA by the first rule).  ksp_get_phase_ns gives a
+ * team's times as for the phase kernels, of a batch those of its first team.
+ * No synchronisation.
  */
 int mat_set_solver(gbs_mat A, int32_t solver);
 /* The row count from which a system of a batched solve runs on the phase

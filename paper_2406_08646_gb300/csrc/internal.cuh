@@ -31,7 +31,10 @@ constexpr uint64_t POOL_KEEP_BYTES = 32ull << 30;
 // FP64 operations per iteration (nonzeros plus eight per row; pcg.cu).
 constexpr int64_t CTA_AUTO_WORK = 40000;
 constexpr int64_t CTA_AUTO_WORK32 = 120000;  // ... of a refined solve's
-constexpr int64_t CTA_BATCH_ROWS = 80000;    // ... and a full batch's largest system
+constexpr int32_t RUN_EVEN = 1024, RUN_SYSTEMS = 1024;
+// Reduction slots (32 bytes) kept for the counters of a batch's grid teams (team.cu): 64
+// counters, each in a line of its own.
+constexpr int64_t TEAM_CTR_SLOTS = 64 * 4;
 int dev_alloc_bytes(void **p, size_t bytes, cudaStream_t s);
 void dev_free(void *p, cudaStream_t s);
 template <typename T>
@@ -195,6 +198,8 @@ struct gbs_mat_s {
   uint32_t *sell_mask = nullptr;   // 32 nslices: pattern entries each row holds
   int32_t slice_max_nnz = 0, slice_max_coo = 0;  // largest nonzeros / COO entries of a slice
   int32_t run_max_nnz = 0;         // one system: largest nonzeros of its slices' equal runs, one an SM
+  int32_t run_uneven = 0;          // a batch (of up to RUN_SYSTEMS): largest nonzeros of a sixteenth of
+                                   // a system's slices over their mean, in units of 1 / RUN_EVEN
   int64_t sell_npat = 0;           // slices with a pattern (0 or nslices)
   int64_t sell_nnz_rows = 0;       // 32 x the slices' longest rows (the size without
                                    // patterns: the automatic plan's padding rule)
@@ -224,7 +229,13 @@ struct gbs_mat_s {
   // products, for CTAs c - halo_lo .. c - halo_lo + halo_n - 1 (mod grid) to
   // have updated their rows of u (set by build_plan from col_span)
   int32_t halo_lo = 0, halo_n = 0;
-  int32_t *cta_order = nullptr; // nsys: systems by decreasing rows (per-CTA solver)
+  int32_t *cta_order = nullptr; // nsys: systems by decreasing rows (per-CTA solver, teams)
+  std::vector<int32_t> cta_order_h;  // the same
+  std::vector<int64_t> sys_nnz_h;    // nonzeros, in that order
+  // the automatic choice for batches (batch_choice in team.cu; -1: not made yet), FP64
+  // and refined; the better kind of team, its cluster size and its systems' first CTAs
+  int32_t batch_engine[2] = {-1, -1}, batch_team = 0, batch_cluster = 0;
+  std::vector<int16_t> batch_parts;
   int64_t max_sys_rows = 0, max_sys_nnz = 0;
 
   // solver workspace (device, allocated on first solve)
@@ -289,7 +300,10 @@ int solve(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_sys
           cudaStream_t s);
 void free_handle(gbs_mat A);
 int sm_count(gbs_mat A);
-bool batch_teams(gbs_mat A);  // a batch whose systems would get a cluster each
+// The engines of a batched solve.
+enum { BATCH_PHASES = 0, BATCH_CTA = 1, BATCH_CLUSTER = 2, BATCH_PARTS = 3 };
+int batch_choice(gbs_mat A);
+bool batch_teams(gbs_mat A);  // a batch that can run on teams
 bool use_team(gbs_mat A, bool per_system, const ksp_opts &o);
 int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,
                cudaStream_t s, bool *ran);

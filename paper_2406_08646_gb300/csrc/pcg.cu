@@ -214,7 +214,8 @@ int ensure_solver_workspace(gbs_mat A, bool refined, cudaStream_t s) {
   // reduction slots: table A's, table E's, and a third region the size of
   // table E's for partial sums of E's slots
   const int64_t need = std::max({A->ta.nslots + 2 * A->te.nslots,
-                                 A->sa.nslots + 2 * A->se.nslots, (int64_t)sm_count(A)}) + 1;
+                                 A->sa.nslots + 2 * A->se.nslots,
+                                 (int64_t)sm_count(A) + TEAM_CTR_SLOTS}) + 1;
   if (A->part_cap < need) {
     if (A->part) {
       GBS_TRY_CUDA(cudaStreamSynchronize(s));
@@ -553,15 +554,7 @@ int sm_count(gbs_mat A) {
 //     less time.  Measured, ms, phases / this: 2D 64^2 (53k operations) 5.12 /
 //     2.50, 80^2 (83k) 6.66 / 4.93, 3D 20^3 (118k) 2.14 / 1.95, 2D 100^2 (130k)
 //     8.37 / 8.53, Q1 16^3 (157k) 1.33 / 1.39, 3D 24^3 (205k) 2.37 / 3.73;
-//   batches whose rows would fill half the SMs with systems of the largest
-//     one's size, if that has at most CTA_BATCH_ROWS (the largest measured): a
-//     phase's time grows with the batch, this one's is the largest system's.
-//     Measured, ms, phases / this, at n systems (rows over the largest's rows
-//     in brackets): refined 100 of 10k-20k (75) 53 / 41, of 20k-40k (75) 117 /
-//     116, 160 of 3k-10k 33 / 15, 160 of 30k-80k (110) 462 / 352, 220 of 10k-30k
-//     140 / 81; FP64 160 of 500-3k (93) 10.4 / 5.6, 300 13.7 / 5.8, of 8k-12k
-//     (250) 94 / 46, 160 of 30k-80k 586 / 520; below the line refined 40 of
-//     10k-20k (30) 33 / 38, 20 of 20k-40k 39 / 100.
+//   batches where batch_choice (team.cu) expects it to be the fastest.
 static bool cta_auto_rule(gbs_mat A, bool per_system, const ksp_opts &o) {
   const bool refined = o.precision == GBS_FP32_REFINED;
   if (o.method != GBS_KSP_CG || o.host_loop || !A->plan_auto ||
@@ -570,7 +563,8 @@ static bool cta_auto_rule(gbs_mat A, bool per_system, const ksp_opts &o) {
   const int64_t nz = per_system ? A->max_sys_nnz : A->nnz;
   const int64_t rows = per_system ? A->max_sys_rows : A->nrows;
   if (refined && nz + 8 * rows <= CTA_AUTO_WORK32) return true;
-  return per_system && rows <= CTA_BATCH_ROWS && 2 * A->nrows >= rows * sm_count(A);
+  return per_system && A->nsys >= 2 && batch_choice(A) == GBS_OK &&
+         A->batch_engine[refined ? 1 : 0] == BATCH_CTA;
 }
 
 bool use_cta_solver(gbs_mat A, bool per_system, const ksp_opts &o) {

@@ -74,13 +74,15 @@ struct ShapeSums {
   int32_t over;             // a slice's union has more than 32 offsets
   int32_t nnz, coo;         // largest nonzeros and COO entries of a slice
   int32_t run;              // largest nonzeros of a run of slices (one system, cut into nruns)
+  int32_t uneven, pad;      // run_uneven (a batch)
 };
 
 // One warp per slice: its first row (a batch's slices start at their system's
 // first row: sys holds nsys + 1 first rows, then nsys + 1 first slices), w[s] =
 // its longest row, u[s] = the size of its rows' offset union (33: more than
 // 32, or patterns not built); their sums over all slices.  Block 0 also cuts one
-// system's slices into nruns equal runs, as team.cu does.
+// system's slices into nruns equal runs, as team.cu does; a batch's systems of 16
+// slices and more are cut into 16.
 constexpr int SHAPE_TPB = 256;
 __global__ void __launch_bounds__(SHAPE_TPB)
     k_slice_shape(int64_t nslices, int64_t nrows, int32_t nsys, const int32_t *__restrict__ sys,
@@ -103,6 +105,18 @@ __global__ void __launch_bounds__(SHAPE_TPB)
     }
     run = __reduce_max_sync(0xffffffffu, run);
     if (lane == 0) atomicMax(&sums->run, run);
+  }
+  if (sys && nsys <= RUN_SYSTEMS) {
+    const int k = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 4, c = threadIdx.x & 15;
+    if (k < nsys) {
+      const int64_t f = sys[k], e = sys[k + 1], n = sys[nsys + 2 + k] - sys[nsys + 1 + k];
+      const int64_t a = f + 32 * (n * c / 16), b = f + 32 * (n * (c + 1) / 16);
+      const int64_t nn = row_ptr[e] - row_ptr[f];
+      if (n >= 16 && nn > 0) {
+        const int64_t x = 16 * RUN_EVEN * (int64_t)(row_ptr[b < e ? b : e] - row_ptr[a]) / nn;
+        if (4 * x > 5 * RUN_EVEN) atomicMax(&sums->uneven, (int32_t)x);
+      }
+    }
   }
   for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices; s += nw) {
     int64_t r0 = 32 * s, r1 = nrows;
@@ -309,6 +323,7 @@ static int shape_copy(gbs_mat A, cudaStream_t st) {
   A->slice_max_nnz = h.nnz;
   A->slice_max_coo = h.coo;
   A->run_max_nnz = h.run;
+  A->run_uneven = h.uneven;
   A->nslices = ns;
   A->sell_nnz = total;
   if (total > 2147483647LL) return GBS_OK;  // too large for 32-bit offsets: no copy

@@ -387,6 +387,10 @@ static int build_cta_order(gbs_mat A, cudaStream_t st) {
   std::stable_sort(ord.begin(), ord.end(), [&](int32_t u, int32_t v) {
     return A->row_off_h[u + 1] - A->row_off_h[u] > A->row_off_h[v + 1] - A->row_off_h[v];
   });
+  A->cta_order_h = ord;
+  A->sys_nnz_h.resize(A->nsys);
+  for (int32_t k = 0; k < A->nsys; ++k) A->sys_nnz_h[k] = noff[ord[k] + 1] - noff[ord[k]];
+  A->batch_engine[0] = A->batch_engine[1] = -1;
   if (!A->cta_order) GBS_TRY(dev_alloc(&A->cta_order, A->nsys, st));
   if (A->nsys == 1) {
     GBS_TRY_CUDA(cudaMemsetAsync(A->cta_order, 0, sizeof(int32_t), st));

@@ -35,7 +35,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
+#include <functional>
+#include <map>
+#include <mutex>
+#include <tuple>
+#include <vector>
 
 #include "cta.cuh"
 #include "device_util.cuh"
@@ -720,6 +726,43 @@ __global__ void __launch_bounds__(TPB, 1)
   }
 }
 
+// A batch of few systems, larger than a cluster should hold: the CTAs of one
+// cooperative grid shared out among them, system order[k] on CTAs [first[k],
+// first[k + 1]), a grid team of its own with its own counter and slots.
+constexpr int TEAM_PARTS_MAX = 64;
+constexpr int TEAM_CTR_STRIDE = 32;  // words from one team's counter to the next: a line each
+struct TeamParts {
+  int16_t first[TEAM_PARTS_MAX + 1];
+};
+
+template <int TPB>
+__global__ void __launch_bounds__(TPB, 1)
+    k_team_parts(const __grid_constant__ PcgArgs a, const __grid_constant__ TeamParts parts,
+                 int32_t halo, int32_t smem, int32_t streams, unsigned *ctr, double *slots) {
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  __shared__ TeamShared sh;
+  int k = 0;
+  while (k + 1 < a.cta_n && (int)blockIdx.x >= parts.first[k + 1]) ++k;
+  const int first = parts.first[k], size = parts.first[k + 1] - first;
+  const SysRange sys = cta_system(a, k);
+  if (threadIdx.x == 0) {
+    sh.abort = 0;
+    sh.call = *a.call;
+    TeamCfg c = team_layout(sys.r1 - sys.r0, 32 * ((sys.s1 - sys.s0 + size - 1) / size), halo,
+                            size, smem);
+    if (streams) {  // (as one system's: p through L1, and room left for it)
+      c.window = c.halo = c.win_cap = c.zh_cap = c.mat_cap = 0;
+      c.nvec = min(4, (smem / 8 - 2 * (int)blockDim.x) / c.rows_cap);
+    }
+    c.ctr = ctr + k * TEAM_CTR_STRIDE;
+    c.slots = slots + 4 * first;
+    sh.cfg = c;
+  }
+  __syncthreads();
+  team_system<true>(a, sh.cfg, sh, reinterpret_cast<double *>(team_smem), sys,
+                    blockIdx.x - first, size, blockIdx.x == 0);  // (the first team's phase times)
+}
+
 // ------------------------------------------------------------------ host side
 
 constexpr int64_t TEAM_SMEM = 219 * 1024;  // dynamic shared memory a CTA may take (of 227 KB)
@@ -764,50 +807,238 @@ static bool team_suits(gbs_mat A) {
   return 2 * (A->sell_nnz * (A->col_span <= 32767 ? 10 : 12) + 40 * n) <= (int64_t)l2;
 }
 
-// CTAs a system of a batch gets: the smallest cluster that gives every SM work
-// and the largest system's CTAs at most TEAM_BATCH_ROWS rows each, so that most
-// of their vectors stay on the SM; 1: the solvers without a team.  (Automatic
-// solver and plan.)  Measured, ms, on edge-diffusion systems, half 2D, half 3D,
-// phase kernels -> clusters: 4 systems of 1k-8k rows 6.0 -> 2.6, 8 of 2k-20k
-// 13.2 -> 8.7, 40 of 500-3k 6.2 -> 3.3, 64 of 1k-20k 32.3 -> 27.7, 100 of 1k-3k
-// 9.5 -> 4.5, 150 of 1k-20k 67.7 -> 49.9, 200 of 5k-20k 96.6 -> 53.3.  A batch
-// whose rows fill every SM with systems of the largest one's size keeps the
-// SMs busy on the per-CTA solver, with no meetings (ms on clusters / there, rows
-// over the largest's rows in brackets: 200 of 5k-20k (125) 54 / 67, 250 (156) 67 /
-// 68, 300 of 10k-30k (200) 164 / 130, of 8k-12k (250) 59 / 46), as does one of two
-// systems an SM (512 of 1k-20k: 105 / 71).
-constexpr int64_t TEAM_BATCH_ROWS = 10240;
-static int team_clusters(gbs_mat A) {
-  if (A->nsys < 2 || A->nsys >= 2 * sm_count(A) || A->nrows == 0 ||
-      A->nrows >= A->max_sys_rows * sm_count(A))
-    return 1;
-  int size = 1;
-  while (size < TEAM_MAX_CLUSTER && ((int64_t)A->nsys * size < sm_count(A) ||
-                                     A->max_sys_rows > TEAM_BATCH_ROWS * size))
-    size *= 2;
-  return A->max_sys_rows <= TEAM_BATCH_ROWS * size ? size : 1;
-}
-bool batch_teams(gbs_mat A) { return team_clusters(A) > 1; }
+// How a batch runs under the automatic choice: an estimate of each engine's time
+// for one iteration of every system (us; fitted to 536 measured batches: equal
+// systems, 2 to 300 of 1,500 to 500,000 rows, 5- to 27-point, and mixed ones), the
+// least wins.  A system's iterations count as its rows to the 0.385th power: the
+// larger ones go on when the smaller have converged.  Systems of unlike size are
+// unlike in iterations too: every second one then counts UNLIKE of them where a
+// queue hands on the SMs that it leaves early, and the shared grid, whose SMs would
+// idle, UNLIKE_SHARE of its time; and clusters take the size that gives every SM work,
+// larger ones where their estimate is less than UNLIKE_SIZE of it.
+//   phase kernels   PHASES_US, and the operations at the whole chip's rate, dearer
+//                   where the systems' blocks do not fit one wave; refined, the bytes
+//   per-CTA solver  one SM a system, from a queue
+//   clusters        the same with `size` SMs, as many clusters as are resident
+//   shared grid     every system its own share of the SMs (k_team_parts)
+// Measured, ms per 100 iterations, phase kernels / per-CTA / clusters of 2, 4, 8, 16 /
+// shared grid:
+//   2D   2 x 1.5k      1.0 / 1.0 / 0.95 0.81 0.75 0.71 / 0.92
+//        2 x 150k      2.5 / 49 / 32 17 8.7 5.3 / 1.9
+//        8 x 40k       2.4 / 13 / 8.9 5.3 3.1 4.1 / 2.0
+//        64 x 60k     17.5 / 22 / 18 17 22 25 / 12.8
+//        140 x 20k    12.9 / 8.0 / 12 12 20 25
+//        160 x 40k    28.7 / 30 / 29 29 34 47
+//   Q1   4 x 20k       2.4 / 18 / 9.8 5.5 3.3 2.3 / 1.5
+//        16 x 60k      8.8 / 52 / 33 18 18 15 / 7.6
+//        16 x 150k    17.2 / 130 / 82 44 40 34 / 17.7
+//        100 x 30k    30.9 / 27 / 35 29 36 40
+//   mixed, to 1e-10: 9 Q1 5k-47k 3.1 / 40 / 21 11 6.6 3.7 / 2.6;  135 of 600-3.6k
+//        8.8 / 6.1 / 4.7 4.6 8.6 17;  211 of 3k-12k 43 / 29 / 23 24 38 62
+//   refined, phase kernels / per-CTA: 76 x 8k Q1 3.1 / 3.2, 2D 78 x 40k 118 / 99, Q1 78 x
+//        40k 20.8 / 24.3, 140 x 40k 35.7 / 27.4, 160 x 40k 41 / 47, 2D 160 x 40k 260 / 206
+// On the 536 the engine chosen takes 3% more than the fastest in the geometric mean
+// and is 1.34 times faster than the choice between phase kernels and per-CTA solver
+// by size alone; on eleven it is 3 to 13% slower than that.  On 70 others, drawn after
+// the fit, 1.40 times and at worst 2% slower.
+// (Clusters of a size that gave every SM work, whatever the systems' size, took 2.1
+// times the phase kernels' time on 2D 2 x 150k, 2.0 on Q1 16 x 150k.)
+// An SM's time goes with a system's nonzeros and, at the vectors' passes, its rows.
+constexpr double PHASES_US = 15.5, PHASES_US_PER_OP = 2.1e-6, PHASES_US_PER_OP_TAIL = 3.05e-6,
+                 PHASES_BYTES_PER_US32 = 2.8e6;
+constexpr double CTA_US = 5.9, CTA_US_PER_NZ = 2.05e-4, CTA_US_PER_OP32 = 1.3e-4;
+constexpr double CLUSTER_US = 6.0, CLUSTER_US_PER_NZ = 2.35e-4;
+constexpr double PARTS_US = 8.4, PARTS_US_PER_NZ = 2.6e-4;
+constexpr int64_t CTA_ROW_NZ = 11, CLUSTER_ROW_NZ = 16, PARTS_ROW_NZ = 11;  // nonzeros a row counts as
+constexpr double UNLIKE = 0.57, UNLIKE_SHARE = 1.3, UNLIKE_SIZE = 0.8;
+constexpr int64_t TEAM_BATCH_ROWS = 10240;  // rows a CTA of an unlike batch's clusters,
+constexpr int64_t UNLIKE_ROWS = 40000;      // ... which take systems of up to so many
 
-static int team_batch_size(gbs_mat A, const ksp_opts &o) {
-  if (o.method != GBS_KSP_CG || o.precision != GBS_FP64 || o.host_loop ||
-      A->lanes != GBS_SPMV_SELL ||
-      !(A->team_tuned || (A->solver == GBS_SOLVER_AUTO && A->cg_form == GBS_CG_TEXTBOOK &&
-                          A->plan_auto)))
-    return 1;
-  return team_clusters(A);
+// The makespan of the systems on k machines that take them in the solvers' order
+// as they fall free; us(q): system q's time on one.
+template <class F>
+static double makespan(int64_t n, int64_t k, F us) {
+  std::vector<double> busy((size_t)std::min(std::max<int64_t>(k, 1), n), 0.0);
+  double end = 0.0;  // (a heap: the machine that falls free first in front)
+  for (int64_t q = 0; q < n; ++q) {
+    std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+    busy.back() += us(q);
+    end = std::max(end, busy.back());
+    std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+  }
+  return end;
 }
 
-// An automatic solver and plan take the team by size; the autotuner takes it
-// where it measured it fastest (team_tuned).  An explicit solver, plan or
-// single-reduction form is what the caller asked for.
+typedef void (*BatchKernel)(PcgArgs, int32_t, int32_t);
+
+// The launch of clusters of `size` CTAs for A's batch, and how many of them are
+// resident at once (0: none) -- a matter of the kernel and the device alone, asked
+// for once.
+struct ClusterLaunch {
+  cudaLaunchConfig_t lc;
+  cudaLaunchAttribute at[1];
+  BatchKernel kernel;
+  int fit;
+};
+static int cluster_launch(gbs_mat A, int size, ClusterLaunch &L) {
+  const int64_t per = (A->max_sys_rows / 32 + size) / size * 32;
+  L.kernel = per <= 1024 ? k_team_batch<512> : k_team_batch<1024>;
+  memset(&L.lc, 0, sizeof(L.lc));
+  memset(L.at, 0, sizeof(L.at));
+  L.lc.gridDim = dim3((unsigned)(sm_count(A) / size * size));
+  L.lc.blockDim = dim3(per <= 1024 ? 512u : 1024u);
+  L.lc.dynamicSmemBytes = TEAM_SMEM;
+  L.lc.attrs = L.at;
+  L.lc.numAttrs = 1;
+  L.at[0].id = cudaLaunchAttributeClusterDimension;
+  L.at[0].val.clusterDim.x = (unsigned)size;
+  L.at[0].val.clusterDim.y = L.at[0].val.clusterDim.z = 1;
+  GBS_TRY_CUDA(cudaFuncSetAttribute(L.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)TEAM_SMEM));
+  GBS_TRY_CUDA(cudaFuncSetAttribute(L.kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, unsigned>, int> known;
+  std::lock_guard<std::mutex> lk(mu);
+  const auto key = std::make_tuple(A->device, size, L.lc.blockDim.x);
+  const auto at = known.find(key);
+  if (at != known.end()) {
+    L.fit = at->second;
+    return GBS_OK;
+  }
+  if (cudaOccupancyMaxActiveClusters(&L.fit, L.kernel, &L.lc) != cudaSuccess) {
+    cudaGetLastError();
+    L.fit = 0;
+  }
+  known[key] = L.fit;
+  return GBS_OK;
+}
+
+// Nonzeros plus per_row a row of the q-th system in the solvers' order.
+static int64_t system_cost(gbs_mat A, int64_t q, int64_t per_row) {
+  const int32_t sy = A->cta_order_h[q];
+  return A->sys_nnz_h[q] + per_row * (A->row_off_h[sy + 1] - A->row_off_h[sy]);
+}
+
+// The first CTAs of the systems on the shared grid: one CTA each, then every
+// further one to the system whose CTAs have the most to do.
+static std::vector<int16_t> share_out(gbs_mat A) {
+  const size_t n = A->cta_order_h.size();
+  std::vector<int64_t> ops(n);
+  for (size_t q = 0; q < n; ++q) ops[q] = system_cost(A, (int64_t)q, PARTS_ROW_NZ);
+  std::vector<int16_t> size(n, 1), first(n + 1, 0);
+  for (int64_t k = (int64_t)n; k < sm_count(A); ++k) {
+    size_t most = 0;
+    for (size_t q = 1; q < n; ++q)
+      if (ops[q] * size[most] > ops[most] * size[q]) most = q;
+    size[most] += 1;
+  }
+  for (size_t q = 0; q < n; ++q) first[q + 1] = (int16_t)(first[q] + size[q]);
+  return first;
+}
+
+// Makes the choice for A's plan (kept until the plan changes).
+int batch_choice(gbs_mat A) {
+  if (A->batch_engine[0] >= 0) return GBS_OK;
+  const int64_t n = A->nsys;
+  A->batch_team = BATCH_PHASES;
+  A->batch_cluster = 0;
+  A->batch_parts.clear();
+  if (A->nsys >= 2 * sm_count(A)) {  // (two per-CTA solvers an SM: cta_size_rule)
+    A->batch_engine[0] = A->batch_engine[1] = BATCH_CTA;
+    return GBS_OK;
+  }
+  // iterations: its for the engines that advance every system at once, queued for
+  // those that take them from a queue
+  std::vector<double> its(n), queued(n);
+  std::vector<int64_t> ops(n);
+  for (int64_t q = 0; q < n; ++q) ops[q] = system_cost(A, q, 8);
+  const auto ends = std::minmax_element(ops.begin(), ops.end());
+  const bool unlike = 4 * *ends.second > 5 * *ends.first;
+  double most_its = 1e-9, work = 0.0;
+  for (int64_t q = 0; q < n; ++q) {
+    const int32_t sy = A->cta_order_h[q];
+    its[q] = pow((double)(A->row_off_h[sy + 1] - A->row_off_h[sy]), 0.385);
+    queued[q] = unlike && (q & 1) ? UNLIKE * its[q] : its[q];
+    most_its = std::max(most_its, its[q]);
+    work += its[q] * (double)ops[q];
+  }
+  double team_us = 1e300;
+  if (A->nsys >= 2 && A->nslices > 0 && A->nnz > 0) {
+    // rows of uneven lengths: the CTA with the longest keeps its team waiting
+    const double uneven = std::max(1.0, (double)A->run_uneven / (1.25 * RUN_EVEN));
+    int small = 2;
+    if (unlike)
+      while (small < TEAM_MAX_CLUSTER && ((int64_t)A->nsys * small < sm_count(A) ||
+                                          A->max_sys_rows > TEAM_BATCH_ROWS * small))
+        small *= 2;
+    for (int size = small; size <= TEAM_MAX_CLUSTER; size *= 2) {
+      if (unlike && A->max_sys_rows > UNLIKE_ROWS) break;
+      ClusterLaunch L;
+      GBS_TRY(cluster_launch(A, size, L));
+      if (L.fit < 1) continue;
+      const double us = makespan(n, L.fit, [&](int64_t q) {
+        return queued[q] * (CLUSTER_US + uneven * CLUSTER_US_PER_NZ *
+                                             (double)system_cost(A, q, CLUSTER_ROW_NZ) / size);
+      });
+      if (us >= (unlike && size > small ? UNLIKE_SIZE : 1.0) * team_us) continue;
+      team_us = us;
+      A->batch_team = BATCH_CLUSTER;
+      A->batch_cluster = size;
+    }
+    if (A->nsys <= TEAM_PARTS_MAX && A->nsys <= sm_count(A)) {
+      A->batch_parts = share_out(A);
+      double us = 0.0;
+      for (int64_t q = 0; q < n; ++q)
+        us = std::max(us, its[q] * (PARTS_US + uneven * PARTS_US_PER_NZ *
+                                                   (double)system_cost(A, q, PARTS_ROW_NZ) /
+                                                   (A->batch_parts[q + 1] - A->batch_parts[q])));
+      if (unlike) us *= UNLIKE_SHARE;
+      if (us < team_us) {
+        team_us = us;
+        A->batch_team = BATCH_PARTS;
+      }
+    }
+  }
+  const double op = A->ta.nblocks <= A->ta.grid ? PHASES_US_PER_OP : PHASES_US_PER_OP_TAIL;
+  const double phases[2] = {
+      PHASES_US * most_its + op * work,
+      most_its * (PHASES_US + (4.0 * (double)A->nnz + 44.0 * (double)A->nrows) / PHASES_BYTES_PER_US32)};
+  for (int refined = 0; refined < 2; ++refined) {
+    const double cta = makespan(n, sm_count(A), [&](int64_t q) {
+      return queued[q] * (CTA_US + (refined ? CTA_US_PER_OP32 * (double)ops[q]
+                                            : CTA_US_PER_NZ * (double)system_cost(A, q, CTA_ROW_NZ)));
+    });
+    int32_t e = cta < phases[refined] ? BATCH_CTA : BATCH_PHASES;
+    if (!refined && team_us < std::min(cta, phases[0])) e = A->batch_team;
+    A->batch_engine[refined] = e;
+  }
+  return GBS_OK;
+}
+
+// FP64 CG, and the solver left to the automatic choice: an explicit solver, plan or
+// single-reduction form is what the caller asked for.  team_tuned: the autotuner
+// measured the team fastest.
+static bool team_allowed(gbs_mat A, const ksp_opts &o) {
+  return o.method == GBS_KSP_CG && o.precision == GBS_FP64 && !o.host_loop &&
+         A->lanes == GBS_SPMV_SELL && A->nrows > 0 &&
+         (A->team_tuned ||
+          (A->solver == GBS_SOLVER_AUTO && A->cg_form == GBS_CG_TEXTBOOK && A->plan_auto));
+}
+
+// How a batch runs under the automatic choice (batch_choice), or, tuned for
+// teams, the better of theirs.
+int32_t batch_team(gbs_mat A, const ksp_opts &o) {
+  if (!team_allowed(A, o) || A->nsys < 2 || batch_choice(A) != GBS_OK) return BATCH_PHASES;
+  const int32_t e = A->team_tuned ? A->batch_team : A->batch_engine[0];
+  return e == BATCH_CLUSTER || e == BATCH_PARTS ? e : BATCH_PHASES;
+}
+bool batch_teams(gbs_mat A) {
+  return A->nsys >= 2 && batch_choice(A) == GBS_OK && A->batch_team != BATCH_PHASES;
+}
+
 bool use_team(gbs_mat A, bool per_system, const ksp_opts &o) {
-  if (per_system) return team_batch_size(A, o) > 1;
-  if (A->nsys != 1 || o.method != GBS_KSP_CG || o.precision != GBS_FP64 ||
-      o.host_loop || A->lanes != GBS_SPMV_SELL || A->nrows == 0)
-    return false;
-  return A->team_tuned || (A->solver == GBS_SOLVER_AUTO && A->cg_form == GBS_CG_TEXTBOOK &&
-                           A->plan_auto && team_suits(A));
+  if (per_system) return batch_team(A, o) != BATCH_PHASES;
+  return A->nsys == 1 && team_allowed(A, o) && (A->team_tuned || team_suits(A));
 }
 
 // The team of a solve on A: its CTAs, their threads and their shared memory.
@@ -862,43 +1093,81 @@ static TeamShape team_shape(gbs_mat A) {
   return T;
 }
 
-// FP64 CG on teams of CTAs; *ran stays false (and nothing has started) where
-// the device cannot hold a team at once.
-static int solve_team_batch(gbs_mat A, const double *b, double *x, const ksp_opts &o,
-                            cudaStream_t s, bool *ran) {
-  const int size = team_batch_size(A, o);
-  const int64_t per = (A->max_sys_rows / 32 + size) / size * 32;
-  const int tpb = per <= 1024 ? 512 : 1024;
-  void (*const kernel)(PcgArgs, int32_t, int32_t) =
-      tpb == 512 ? k_team_batch<512> : k_team_batch<1024>;
-  GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)TEAM_SMEM));
-  GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaLaunchConfig_t lc = {};
-  cudaLaunchAttribute at[1];
-  memset(at, 0, sizeof(at));
-  lc.gridDim = dim3((unsigned)(sm_count(A) / size * size));
-  lc.blockDim = dim3((unsigned)tpb);
-  lc.dynamicSmemBytes = TEAM_SMEM;
-  lc.stream = s;
-  lc.attrs = at;
-  lc.numAttrs = 1;
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)size;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  int fit = 0;  // clusters resident at once
-  if (cudaOccupancyMaxActiveClusters(&fit, kernel, &lc) != cudaSuccess || fit < 1) {
-    cudaGetLastError();
-    return GBS_OK;
-  }
-  lc.gridDim = dim3((unsigned)(std::min<int64_t>(fit, A->nsys) * size));
+// Batches on teams; *ran stays false (and nothing has started) where the device
+// cannot hold a team at once.
+static int solve_clusters(gbs_mat A, const double *b, double *x, const ksp_opts &o,
+                          cudaStream_t s, bool *ran) {
+  ClusterLaunch L;
+  GBS_TRY(cluster_launch(A, A->batch_cluster, L));
+  if (L.fit < 1) return GBS_OK;
+  L.lc.stream = s;
+  L.lc.gridDim = dim3((unsigned)(std::min<int64_t>(L.fit, A->nsys) * A->batch_cluster));
   PcgArgs a = make_args(A, true, false);
   a.stream_matrix = 0;  // (a system's matrix is read again by the same SMs, from L2)
   a.order = A->cta_order;
   a.cta_n = A->nsys;
   GBS_TRY_CUDA(cudaMemsetAsync(A->ctl, 0, sizeof(DevCtl), s));
   GBS_TRY(put_call(A->call, call_args(b, x, o), s, A->ctl));
-  GBS_TRY_CUDA(cudaLaunchKernelEx(&lc, kernel, a, A->col_span, (int32_t)TEAM_SMEM));
+  GBS_TRY_CUDA(cudaLaunchKernelEx(&L.lc, L.kernel, a, A->col_span, (int32_t)TEAM_SMEM));
+  count_launches(1);
+  *ran = true;
+  return GBS_OK;
+}
+
+static int solve_parts(gbs_mat A, const double *b, double *x, const ksp_opts &o,
+                       cudaStream_t s, bool *ran) {
+  TeamParts parts;
+  memset(&parts, 0, sizeof(parts));
+  // the largest part's rows, and whether every part keeps its matrix and vectors
+  int64_t rows = 0, bytes = 0;
+  const int64_t per_entry = A->sell_npat ? 8 : (A->col_span <= 32767 ? 10 : 12);
+  for (int32_t k = 0; k < A->nsys; ++k) {
+    parts.first[k] = A->batch_parts[k];
+    const int32_t q = A->cta_order_h[k];
+    const int64_t size = A->batch_parts[k + 1] - A->batch_parts[k];
+    const int64_t per = (A->sell_slice0_h[q + 1] - A->sell_slice0_h[q] + size - 1) / size;
+    const int64_t halo = std::min<int64_t>(A->col_span, A->row_off_h[q + 1] - A->row_off_h[q]);
+    rows = std::max(rows, 32 * per);
+    bytes = std::max(bytes, per * (32 * 5 * 8 + (A->slice_max_nnz * per_entry) * 9 / 8 + 136 +
+                                   (A->sell_npat ? 256 : 0)) + 16 * std::max(32 * per, halo));
+  }
+  parts.first[A->nsys] = A->batch_parts[A->nsys];
+  const bool streams = bytes > TEAM_SMEM - 16 * 512;
+  const int tpb = streams ? 1024 : 512;
+  const int64_t smem = streams ? 16 * tpb + std::min<int64_t>(4, TEAM_L1_SMEM / (8 * rows)) * 8 * rows
+                               : TEAM_SMEM;
+  void (*const kernel)(PcgArgs, TeamParts, int32_t, int32_t, int32_t, unsigned *, double *) =
+      streams ? k_team_parts<1024> : k_team_parts<512>;
+  GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)TEAM_SMEM));
+  cudaLaunchConfig_t lc;
+  cudaLaunchAttribute at[1];
+  memset(&lc, 0, sizeof(lc));
+  memset(at, 0, sizeof(at));
+  lc.gridDim = dim3((unsigned)parts.first[A->nsys]);
+  lc.blockDim = dim3((unsigned)tpb);
+  lc.dynamicSmemBytes = (size_t)smem;
+  lc.stream = s;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  PcgArgs a = make_args(A, true, false);
+  a.stream_matrix = stream_matrix(A, 8);
+  a.order = A->cta_order;
+  a.cta_n = A->nsys;
+  // slots: four doubles a CTA; then the teams' counters (ensure_solver_workspace)
+  unsigned *const ctr = reinterpret_cast<unsigned *>(A->part + 4 * sm_count(A));
+  GBS_TRY_CUDA(cudaMemsetAsync(ctr, 0, sizeof(unsigned) * TEAM_CTR_STRIDE * A->nsys, s));
+  GBS_TRY_CUDA(cudaMemsetAsync(A->ctl, 0, sizeof(DevCtl), s));
+  GBS_TRY(put_call(A->call, call_args(b, x, o), s, A->ctl));
+  const cudaError_t e = cudaLaunchKernelEx(&lc, kernel, a, parts, A->col_span, (int32_t)smem,
+                                           (int32_t)streams, ctr, A->part);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources) {
+    cudaGetLastError();
+    return GBS_OK;
+  }
+  GBS_TRY_CUDA(e);
   count_launches(1);
   *ran = true;
   return GBS_OK;
@@ -907,7 +1176,9 @@ static int solve_team_batch(gbs_mat A, const double *b, double *x, const ksp_opt
 int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool per_system,
                cudaStream_t s, bool *ran) {
   *ran = false;
-  if (per_system) return solve_team_batch(A, b, x, o, s, ran);
+  if (per_system)
+    return batch_team(A, o) == BATCH_PARTS ? solve_parts(A, b, x, o, s, ran)
+                                           : solve_clusters(A, b, x, o, s, ran);
   TeamShape T = team_shape(A);
   PcgArgs a = make_args(A, false, false);
   a.stream_matrix = stream_matrix(A, 8);
