@@ -1190,8 +1190,7 @@ cleanup:
 //      held the kernel; a counting sort over NUM_CLASSES length classes puts
 //      segments of about one length on a warp.
 //   3. The results in nonzero order, coalesced.
-// The lane a nonzero lands on depends on shared-memory atomics; its sum does
-// not.
+// The lane a nonzero lands on depends on its class's ballots; its sum does not.
 //
 // SLICES: the tile is a few whole slices of the sliced copy, whose values and
 // the rows' D^-1 are written from the same shared sums -- otherwise two more
@@ -1204,7 +1203,7 @@ cleanup:
 constexpr int NUM_TPB = 256, NUM_CLASSES = 5, NUM_BATCH = 4;
 constexpr int NUM_NZ = 1024;   // nonzeros of a tile, at most
 constexpr int NUM_E = 3072;    // COO entries of a tile that shared memory holds
-constexpr int NUM_TILE = 512;  // nonzeros of a tile that is not cut by slices
+constexpr int NUM_TILE = 512;  // nonzeros of a tile that is not cut by slices, at most
 constexpr int NUM_SLICES = 8;  // slices of a tile, at most
 constexpr int NUM_CTAS = 6;    // CTAs an SM (40 registers a thread)
 
@@ -1326,16 +1325,15 @@ __device__ __forceinline__ void numeric_tile(const NumShared &sh, int e_cap, int
   }
 }
 
-// Tiles of NUM_TILE nonzeros; the values only.
+// Tiles of `tile` nonzeros; the values only.
 __global__ void __launch_bounds__(NUM_TPB, NUM_CTAS)
-    k_coo_numeric(int64_t nnz, const int32_t *__restrict__ jmap,
+    k_coo_numeric(int64_t nnz, int32_t tile, const int32_t *__restrict__ jmap,
                   const int32_t *__restrict__ perm, const double *__restrict__ v, int mode,
                   double *__restrict__ val) {
   extern __shared__ __align__(16) unsigned char num_smem[];
   const NumShared sh = num_carve(num_smem, NUM_E, NUM_TILE);
-  for (int64_t t0 = (int64_t)blockIdx.x * NUM_TILE; t0 < nnz;
-       t0 += (int64_t)gridDim.x * NUM_TILE) {
-    const int nt = nnz - t0 < NUM_TILE ? (int)(nnz - t0) : NUM_TILE;
+  for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < nnz; t0 += (int64_t)gridDim.x * tile) {
+    const int nt = nnz - t0 < tile ? (int)(nnz - t0) : tile;
     numeric_tile(sh, NUM_E, t0, nt, jmap, perm, v, mode, val);
     __syncthreads();
     for (int i = threadIdx.x; i < nt; i += NUM_TPB) val[t0 + i] = sh.sum[i];
@@ -1407,6 +1405,20 @@ __global__ void k_jacobi(int64_t nrows, const int32_t *__restrict__ diag_pos,
   }
 }
 
+// The values of A, without its sliced copy.  A tile holds as many whole warps of
+// nonzeros as fit NUM_E entries at their mean length with a quarter to spare:
+// longer ones go a thread each, and fewer to a CTA keep more SMs at it (ms,
+// tiles of 512 -> this: 1000 sums of 3000 entries 1.22 -> 0.43, 10,000 of 300 0.141 ->
+// 0.057, 300 of 3333 1.17 -> 0.48).
+static int numeric_values(gbs_mat A, const double *v, int mode, cudaStream_t s) {
+  const int64_t fit = (int64_t)NUM_E * 3 / 4 * A->nnz / std::max<int64_t>(A->nkept, 1);
+  const int32_t tile = (int32_t)std::min<int64_t>(NUM_TILE, std::max<int64_t>(32, fit / 32 * 32));
+  k_coo_numeric<<<grid_for(A->nnz, tile), NUM_TPB, num_shared(NUM_E, NUM_TILE), s>>>(
+      A->nnz, tile, A->jmap, A->perm, v, mode, A->val);
+  GBS_LAUNCHED(1);
+  return GBS_OK;
+}
+
 int launch_set_values(gbs_mat A, const double *v, int mode, cudaStream_t s) {
   // slices a tile holds, where every tile of so many fits (their largest
   // counts are the shape's)
@@ -1423,12 +1435,7 @@ int launch_set_values(gbs_mat A, const double *v, int mode, cudaStream_t s) {
         A->diag_pos, A->dinv, A->sell_ptr, A->sell_npat ? A->sell_mask : nullptr, A->sell_val);
     GBS_LAUNCHED(1);
   } else {
-    if (A->nnz > 0) {
-      k_coo_numeric<<<grid_for((A->nnz + NUM_TILE - 1) / NUM_TILE, 1), NUM_TPB,
-                      num_shared(NUM_E, NUM_TILE), s>>>(
-          A->nnz, A->jmap, A->perm, v, mode, A->val);
-      GBS_LAUNCHED(1);
-    }
+    if (A->nnz > 0) GBS_TRY(numeric_values(A, v, mode, s));
     if (A->nrows > 0) {
       k_jacobi<<<grid_for(A->nrows, 256), 256, 0, s>>>(A->nrows, A->diag_pos, A->val, A->dinv);
       GBS_LAUNCHED(1);
@@ -1481,12 +1488,7 @@ __global__ void k_vec_scatter(int64_t n, const int32_t *__restrict__ row_ptr,
 // Vector numeric stage: the in-order sums of the n x 1 pattern (the matrix
 // numeric kernel, INSERT into val), then the scatter into y.
 int launch_vec_set_values(gbs_mat A, const double *v, int mode, double *y, cudaStream_t s) {
-  if (A->nnz > 0) {
-    k_coo_numeric<<<grid_for((A->nnz + NUM_TILE - 1) / NUM_TILE, 1), NUM_TPB,
-                      num_shared(NUM_E, NUM_TILE), s>>>(
-        A->nnz, A->jmap, A->perm, v, GBS_INSERT, A->val);
-    GBS_LAUNCHED(1);
-  }
+  if (A->nnz > 0) GBS_TRY(numeric_values(A, v, GBS_INSERT, s));
   if (A->nrows > 0) {
     k_vec_scatter<<<grid_for(A->nrows, 256), 256, 0, s>>>(A->nrows, A->row_ptr, A->val, mode, y);
     GBS_LAUNCHED(1);
