@@ -26,8 +26,9 @@
 //     memory: 0.2-0.3 us a barrier, 0.7-0.9 us a sum;
 //   - the whole grid, one CTA per SM, launched cooperatively, meets at a
 //     counter in global memory: 1.2 us a barrier, 1.9 us a sum (152 CTAs).
-// Every wait of the grid team is bounded (one second and 2^22 polls), after
-// which the solve ends with GBS_ERR_TIMEOUT.
+// Every wait of the grid team is bounded (over a second and 2^22 polls), after
+// which the solve ends with GBS_ERR_TIMEOUT.  (A wait lasts as long as the other
+// CTAs' longest run of rows takes: at most about a second for 2^31 entries on one SM.)
 //
 // Every CTA adds the team's partial sums itself, in rank order, and its thread
 // 0 runs the scalar recurrences on the same totals, so all CTAs take the same
@@ -51,6 +52,8 @@
 namespace gbs {
 
 constexpr int TEAM_MAX_CLUSTER = 16;
+constexpr int64_t TEAM_WAIT_NS = 1000000000;   // bounded waits: over a second and
+constexpr unsigned TEAM_WAIT_POLLS = 1u << 22;  // 2^22 polls
 
 // How a launch lays out its dynamic shared memory: the block sums' scratch,
 // the p window and (clusters) the halo of z, then nvec vectors of rows_cap
@@ -60,6 +63,10 @@ struct TeamCfg {
   int32_t halo, win_cap, zh_cap;
   int32_t nvec, rows_cap, mat_cap;
   unsigned *ctr;   // grid team: arrivals, zero at launch
+  // ... and how long one of its waits may last: both so many polls and so many ns
+  // (a process that the GPU sets aside for a while polls no more)
+  unsigned wait_polls;
+  int64_t wait_ns;
   double *slots;   // grid team: 2 parities x 2 values x CTAs
 };
 
@@ -146,7 +153,7 @@ struct Team {
       if ((polls & 1023u) == 1023u) {
         const uint64_t t = global_ns();
         if (t0 == 0) t0 = t;
-        else if (polls > (1u << 22) && t - t0 > 1000000000ull) {
+        else if (polls > cfg.wait_polls && t - t0 > (uint64_t)cfg.wait_ns) {
           sh.abort = 1;
           break;
         }
@@ -656,6 +663,8 @@ __device__ __forceinline__ TeamCfg team_layout(int n, int per_rows, int halo, in
   c.window = c.halo = c.win_cap = c.zh_cap = c.mat_cap = 0;
   c.ctr = nullptr;
   c.slots = nullptr;
+  c.wait_polls = TEAM_WAIT_POLLS;
+  c.wait_ns = TEAM_WAIT_NS;
   c.rows_cap = max(per_rows, 32);
   int room = smem / 8 - 2 * (int)blockDim.x;  // doubles
   const int h = min(halo, n), win = (min(n, c.rows_cap + 2 * h) + 31) & ~31;
@@ -738,7 +747,8 @@ struct TeamParts {
 template <int TPB>
 __global__ void __launch_bounds__(TPB, 1)
     k_team_parts(const __grid_constant__ PcgArgs a, const __grid_constant__ TeamParts parts,
-                 int32_t halo, int32_t smem, int32_t streams, unsigned *ctr, double *slots) {
+                 int32_t halo, int32_t smem, int32_t streams, unsigned *ctr, double *slots,
+                 unsigned wait_polls, int64_t wait_ns) {
   extern __shared__ __align__(16) unsigned char team_smem[];
   __shared__ TeamShared sh;
   int k = 0;
@@ -756,6 +766,8 @@ __global__ void __launch_bounds__(TPB, 1)
     }
     c.ctr = ctr + k * TEAM_CTR_STRIDE;
     c.slots = slots + 4 * first;
+    c.wait_polls = wait_polls;
+    c.wait_ns = wait_ns;
     sh.cfg = c;
   }
   __syncthreads();
@@ -1136,7 +1148,8 @@ static int solve_parts(gbs_mat A, const double *b, double *x, const ksp_opts &o,
   const int tpb = streams ? 1024 : 512;
   const int64_t smem = streams ? 16 * tpb + std::min<int64_t>(4, TEAM_L1_SMEM / (8 * rows)) * 8 * rows
                                : TEAM_SMEM;
-  void (*const kernel)(PcgArgs, TeamParts, int32_t, int32_t, int32_t, unsigned *, double *) =
+  void (*const kernel)(PcgArgs, TeamParts, int32_t, int32_t, int32_t, unsigned *, double *,
+                       unsigned, int64_t) =
       streams ? k_team_parts<1024> : k_team_parts<512>;
   GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)TEAM_SMEM));
@@ -1162,7 +1175,8 @@ static int solve_parts(gbs_mat A, const double *b, double *x, const ksp_opts &o,
   GBS_TRY_CUDA(cudaMemsetAsync(A->ctl, 0, sizeof(DevCtl), s));
   GBS_TRY(put_call(A->call, call_args(b, x, o), s, A->ctl));
   const cudaError_t e = cudaLaunchKernelEx(&lc, kernel, a, parts, A->col_span, (int32_t)smem,
-                                           (int32_t)streams, ctr, A->part);
+                                           (int32_t)streams, ctr, A->part, TEAM_WAIT_POLLS,
+                                           TEAM_WAIT_NS);
   if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources) {
     cudaGetLastError();
     return GBS_OK;
@@ -1184,6 +1198,8 @@ int solve_team(gbs_mat A, const double *b, double *x, const ksp_opts &o, bool pe
   a.stream_matrix = stream_matrix(A, 8);
   T.cfg.slots = A->part;
   T.cfg.ctr = reinterpret_cast<unsigned *>(&A->ctl->queue);
+  T.cfg.wait_polls = TEAM_WAIT_POLLS;
+  T.cfg.wait_ns = TEAM_WAIT_NS;
   void (*const kernel)(PcgArgs, TeamCfg) =
       T.cluster ? k_team<false, 512> : T.tpb <= 512 ? k_team<true, 512> : k_team<true, 1024>;
   GBS_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
