@@ -210,8 +210,9 @@ struct gbs_mat_s {
   // row-product kernel (0: sliced ELL; 1, 2, 4, 8, 32: CSR-vector with that
   // many lanes per row), CTAs per SM cap of the grids
   gbs::TableDev ta, te;
-  // CSR-vector plans: the rows of each 512-row chunk (MatMult) and of each block
-  // of table A by length, longest first (spmv.cu); one allocation (order_s)
+  // CSR-vector plans of ragged rows: the rows of each 512-row chunk (MatMult) and of each
+  // block of table A by length, longest first (spmv.cu); one allocation (order_s), used
+  // where order_a is set
   int32_t *order_s = nullptr, *order_a = nullptr;
   int32_t Ra = 256, Re = 512;   // rows per SpMV block / per update block
   int32_t lanes = 0;

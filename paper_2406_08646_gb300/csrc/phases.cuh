@@ -454,9 +454,10 @@ __device__ __forceinline__ T transpose_reduce(T (&acc)[L], int li) {
 // average: about 40 steps a warp in row order, 20 in length order).
 // AHEAD: the next step's columns and values are loaded before this step's
 // gathers are used, one round trip a step instead of two; it takes registers,
-// which the solves' one-wave phase kernels have to spare (graph of 300k rows,
-// product phase 26.8 us in row order, 24.0 in length order, 22.5 so) and
-// MatMult's many small CTAs do not (28.8, 26.7; 32.6 so).
+// which the solves' one-wave phase kernels have to spare at four lanes and more
+// (graph of 300k rows, product phase 26.8 us in row order, 24.0 in length order, 22.5
+// so; with two lanes 93 registers for 64 and one CTA an SM for two) and MatMult's
+// many small CTAs do not (28.8, 26.7; 32.6 so).
 template <typename T, int L, bool AHEAD, class F>
 __device__ __forceinline__ void csr_rows(const int32_t *__restrict__ row_ptr,
                                          const int32_t *__restrict__ col,
@@ -873,7 +874,7 @@ __device__ __forceinline__ void row_products(const PcgArgs &a, int b, int r0, in
     else
       sell_rows<T, false, GATHER_NC, false, NP>(a.sv, sell_val, x, s0, s1, f);
   } else
-    csr_rows<T, L, true>(a.row_ptr, a.col, csr_val, x, r0, r1, a.row_order, f);
+    csr_rows<T, L, (L >= 4)>(a.row_ptr, a.col, csr_val, x, r0, r1, a.row_order, f);
 }
 
 // The convergence threshold thr = rtol ||b_s|| and two bounds of thr^2

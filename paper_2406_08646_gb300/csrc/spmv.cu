@@ -179,12 +179,13 @@ int launch_spmv(gbs_mat A, const double *x, double *y, cudaStream_t s) {
   }
   const int64_t chunks = (A->nrows + SPMV_ROWS - 1) / SPMV_ROWS;
   const unsigned grid = (unsigned)std::min<int64_t>(chunks, 1 << 20);
+  const int32_t *const order = A->order_a ? A->order_s : nullptr;
   switch (A->lanes) {
-    case 1: k_spmv<1><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
-    case 2: k_spmv<2><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
-    case 8: k_spmv<8><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
-    case 32: k_spmv<32><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
-    default: k_spmv<4><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, A->order_s); break;
+    case 1: k_spmv<1><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, order); break;
+    case 2: k_spmv<2><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, order); break;
+    case 8: k_spmv<8><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, order); break;
+    case 32: k_spmv<32><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, order); break;
+    default: k_spmv<4><<<grid, PHASE_TPB, 0, s>>>(A->row_ptr, A->col, A->val, x, y, n, order); break;
   }
   GBS_LAUNCHED(1);
   return GBS_OK;
@@ -450,7 +451,14 @@ int build_plan(gbs_mat A, int32_t Ra, int32_t Re, int32_t kernel, int32_t ctas_p
   if (Ra == 0) Ra = auto_rows(cap_a);
   if (Re == 0) Re = auto_rows(cap_e);
   GBS_TRY(build_table(A, Ra, cap_a, A->ta, st));
-  if (kernel != GBS_SPMV_SELL && kernel != 32) GBS_TRY(build_row_orders(A, st));
+  // Rows in length order: for four and eight lanes a row on rows too uneven for the
+  // sliced copy.  Shorter rows (fewer lanes) waste little, and even ones lose the
+  // neighbours they share columns with: us a CG iteration in row order / so, rows
+  // drawn from 2 to 16 entries (two lanes) 100k 23.0 / 23.4, 1M 80.0 / 79.9, from 2 to 120
+  // (four) 100k 43.8 / 33.8, 300k 103 / 75, 2 to 40 1M 111 / 93; 3D 7-point 1M with one
+  // lane 61 / 68, two 62 / 69, four 67 / 70.
+  if ((kernel == 4 || kernel == 8) && (double)A->sell_nnz_rows > 1.2 * (double)A->nnz)
+    GBS_TRY(build_row_orders(A, st));
   halo_window(A, Ra, A->ta);
   GBS_TRY(build_table(A, Re, cap_e, A->te, st));
   GBS_TRY(build_cta_order(A, st));
