@@ -419,7 +419,8 @@ int mat_get_plan(gbs_mat A, int32_t *spmv_rows, int32_t *update_rows, int32_t *k
  *     PHASES.  With an automatic plan, the textbook form and no host_loop it
  *     also chooses among
  *       - CTA for refined solves of systems of at most 120000 such operations;
- *       - teams of CTAs for FP64 CG on one system of at most 3,145,728 rows:
+ *       - teams of CTAs for FP64 CG on one system of at most 3,145,728 rows
+ *         (1,835,008 where they hold fewer than four entries each on average):
  *         every iteration in one launch, on a thread-block cluster (up to
  *         160000 operations) or on one CTA per SM.  Systems whose rows' lengths
  *         differ much from place to place, or whose columns are scattered

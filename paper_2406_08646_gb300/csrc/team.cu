@@ -789,7 +789,10 @@ constexpr int64_t TEAM_CLUSTER_WORK = 160000;
 // Beyond this many rows the phase kernels take over: twice the threads an SM
 // hide HBM's latency better than the saved meetings are worth (3D 7-point,
 // us an iteration on team / phases: 128^3 70.4 / 72.9, 160^3 141.6 / 134.0).
-constexpr int64_t TEAM_GRID_ROWS = 3 << 20;
+// Rows of fewer than four entries are the vectors' traffic for the most part and
+// end sooner (tridiagonal, 1.5M 45.0 / 48.0, 1.75M 52.8 / 54.0, 2M 58.7 / 56.5, 2.8M 84.6 /
+// 75.3).
+constexpr int64_t TEAM_GRID_ROWS = 3 << 20, TEAM_SHORT_ROWS = 7 << 18;
 // A team's CTA owns one run of slices, alone on its SM, where the phase kernels'
 // four CTAs an SM take blocks from four places of the matrix: where the rows'
 // lengths differ from place to place the team waits for its longest run.  That
@@ -809,7 +812,7 @@ constexpr int64_t TEAM_EXCESS = 28000, TEAM_EXCESS_ROWS = 1 << 20;
 // 30.2, 450k 69.3 / 65.9; 3D edges 300k 20.0 / 25.0, 1M (110) 51.8 / 47.0, 3M 131 / 106.
 static bool team_suits(gbs_mat A) {
   const int64_t n = A->nrows, run = A->run_max_nnz, sms = sm_count(A);
-  if (n > TEAM_GRID_ROWS) return false;
+  if (n > (A->nnz < 4 * n ? TEAM_SHORT_ROWS : TEAM_GRID_ROWS)) return false;
   if (4 * run * sms > 5 * A->nnz &&
       (n > TEAM_EXCESS_ROWS || run - A->nnz / sms > TEAM_EXCESS))
     return false;
