@@ -906,7 +906,8 @@ def run_gpu(args, rank: int, world: int):
             "spmv": {"gbs": spmv_gbs, "frac": spmv_gbs / hbm, "us": spmv_s * 1e6,
                      "alg_bytes": spmv_alg_bytes(n, nnz)},
             "generate": s0_rows(med, args.ne, hbm),
-            "roofline": {"kernel": "k_spmv_sell (MatMult, sliced-ELL FP64 row product)",
+            "roofline": {"kernel": ("k_spmv_sell_deep" if args.ne == 96 else "k_spmv_sell")
+                         + " (MatMult, sliced-ELL FP64 row product)",
                          "bound": "hbm", "achieved": spmv_gbs, "peak": hbm, "unit": "GB/s",
                          "frac": spmv_gbs / hbm, "peak_kind": f"{peak_kind} (copy, burst)",
                          "traffic": traffic, "alg_bytes": spmv_alg_bytes(n, nnz),

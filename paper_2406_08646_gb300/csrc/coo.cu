@@ -436,9 +436,11 @@ static unsigned grid_for(int64_t n, int tpb) {
   return (unsigned)g;
 }
 
-// A grid that keeps every SM busy and no more: for kernels that end in one
-// atomic a CTA, or loop anyway.
-static unsigned wave_for(int64_t n, int tpb) { return std::min(grid_for(n, tpb), 8u * 160u); }
+// A grid that keeps every SM of A's device busy and no more: for kernels that
+// end in one atomic a CTA.
+static unsigned wave_for(gbs_mat A, int64_t n, int tpb) {
+  return std::min(grid_for(n, tpb), 8u * (unsigned)sm_count(A));
+}
 
 // Error exits of the symbolic stages: set status and jump to cleanup.
 #define SYM_CUDA(call)                                                            \
@@ -930,7 +932,7 @@ static int symbolic_rows(gbs_mat A, const int32_t *i, const int32_t *j,
     }
     SYM_TRY(exclusive_scan(cnt, rstart, n + 1, scan_tmp, &dctl->nkept, s));
     if (n > 0) {
-      k_max_row<<<wave_for(n, 256), 256, 0, s>>>(reinterpret_cast<const int32_t *>(rstart), n,
+      k_max_row<<<wave_for(A, n, 256), 256, 0, s>>>(reinterpret_cast<const int32_t *>(rstart), n,
                                                  &dctl->maxcnt);
       GBS_LAUNCHED(1);
     }
@@ -1153,7 +1155,7 @@ static int symbolic_radix(gbs_mat A, const int32_t *i, const int32_t *j,
       GBS_LAUNCHED(1);
     }
     if (nnz > 0) {
-      k_csr_cols<<<wave_for(nnz, 256), 256, 0, s>>>(ukey, nnz, A->ncols, A->col, A->diag_pos,
+      k_csr_cols<<<wave_for(A, nnz, 256), 256, 0, s>>>(ukey, nnz, A->ncols, A->col, A->diag_pos,
                                                     &dctl->span);
       GBS_LAUNCHED(1);
     }
