@@ -1407,16 +1407,21 @@ __global__ void k_jacobi(int64_t nrows, const int32_t *__restrict__ diag_pos,
   }
 }
 
-// The values of A, without its sliced copy.  A tile holds as many whole warps of
-// nonzeros as fit NUM_E entries at their mean length with a quarter to spare:
-// longer ones go a thread each, and fewer to a CTA keep more SMs at it (ms,
-// tiles of 512 -> this: 1000 sums of 3000 entries 1.22 -> 0.43, 10,000 of 300 0.141 ->
-// 0.057, 300 of 3333 1.17 -> 0.48).
+// The values of A, without its sliced copy, in tiles of 512 nonzeros.  Where a
+// tile's entries would not fit shared memory its nonzeros go a thread each (which
+// long segments want anyway: neighbours in the pattern are often neighbours in v),
+// and few nonzeros are then dealt out to two CTAs an SM, a warp of them or more
+// each, but no tile so small that it would fit again.  ms, tiles of 512 -> this: 1000
+// sums of 3000 entries 1.22 -> 0.43, 10,000 of 300 0.141 -> 0.057, 300 of 3333 1.17 -> 0.47.
+// (Tiles that fit, for every mean length: 912,673 sums of 8 entries 0.039 -> 0.048.)
 static int numeric_values(gbs_mat A, const double *v, int mode, cudaStream_t s) {
-  const int64_t fit = (int64_t)NUM_E * 3 / 4 * A->nnz / std::max<int64_t>(A->nkept, 1);
-  const int32_t tile = (int32_t)std::min<int64_t>(NUM_TILE, std::max<int64_t>(32, fit / 32 * 32));
-  k_coo_numeric<<<grid_for(A->nnz, tile), NUM_TPB, num_shared(NUM_E, NUM_TILE), s>>>(
-      A->nnz, tile, A->jmap, A->perm, v, mode, A->val);
+  int64_t tile = NUM_TILE;
+  if (NUM_TILE * A->nkept > NUM_E * A->nnz) {
+    const int64_t least = NUM_E * A->nnz / A->nkept + 1, share = A->nnz / (2 * sm_count(A));
+    tile = std::min<int64_t>(NUM_TILE, (std::max(least, share) + 31) / 32 * 32);
+  }
+  k_coo_numeric<<<grid_for(A->nnz, (int)tile), NUM_TPB, num_shared(NUM_E, NUM_TILE), s>>>(
+      A->nnz, (int32_t)tile, A->jmap, A->perm, v, mode, A->val);
   GBS_LAUNCHED(1);
   return GBS_OK;
 }

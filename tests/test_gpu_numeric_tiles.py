@@ -1,7 +1,7 @@
 """GPU numeric COO stage without a sliced copy: tiles from 512 nonzeros down to one warp's, by the
-mean number of entries of a nonzero, with lengths that vary around it (tiles that fit shared
-memory beside ones that do not); and patterns of few rows, whose entries cannot fit the row
-counts.  Bits of the oracle's sums in increasing COO index.
+number of nonzeros and the mean number of entries of one, with lengths that vary around it (tiles
+that fit shared memory beside ones that do not); and patterns of few rows, whose entries cannot
+fit the row counts.  Bits of the oracle's sums in increasing COO index.
 """
 import numpy as np
 import pytest
