@@ -433,7 +433,7 @@ int mat_get_plan(gbs_mat A, int32_t *spmv_rows, int32_t *update_rows, int32_t *k
  * (one system's, or a batch's shared grid) is launched cooperatively and takes
  * every SM until the solve ends: solves on several streams then run one after
  * another, where PHASES lets them overlap -- set it for handles that are solved
- * at the same time on streams of their own (four systems of 40,000 rows at once:
+ * at the same time on streams of their own (200 iterations of four systems of 40,000 rows:
  * 4.0 ms on PHASES, 7.3 on teams, which take 1.8 for one alone against 3.4).  Its
  * waits are bounded; should one last over a second the solve ends with
  * GBS_ERR_TIMEOUT, whatever timeout_ns, and x is undefined.

@@ -869,12 +869,21 @@ constexpr double UNLIKE = 0.57, UNLIKE_SHARE = 1.3, UNLIKE_SIZE = 0.8;
 constexpr int64_t TEAM_BATCH_ROWS = 10240;  // rows a CTA of an unlike batch's clusters,
 constexpr int64_t UNLIKE_ROWS = 40000;      // ... which take systems of up to so many
 
-// The makespan of the systems on k machines that take them in the solvers' order
-// as they fall free; us(q): system q's time on one.
+// The makespan of n systems on k machines that take them in the solvers' order as
+// they fall free; us(q): system q's time on one.  Where it cannot be below limit, a
+// lower bound that is not either.
 template <class F>
-static double makespan(int64_t n, int64_t k, F us) {
-  std::vector<double> busy((size_t)std::min(std::max<int64_t>(k, 1), n), 0.0);
-  double end = 0.0;  // (a heap: the machine that falls free first in front)
+static double makespan(int64_t n, int64_t k, double limit, F us) {
+  k = std::min(std::max<int64_t>(k, 1), n);
+  double sum = 0.0, most = 0.0;
+  for (int64_t q = 0; q < n; ++q) {
+    const double t = us(q);
+    sum += t;
+    most = std::max(most, t);
+  }
+  if (n <= k || std::max(most, sum / (double)k) >= limit) return std::max(most, sum / (double)k);
+  std::vector<double> busy((size_t)k, 0.0);  // a heap: the machine that falls free first in front
+  double end = 0.0;
   for (int64_t q = 0; q < n; ++q) {
     std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
     busy.back() += us(q);
@@ -991,11 +1000,12 @@ int batch_choice(gbs_mat A) {
       ClusterLaunch L;
       GBS_TRY(cluster_launch(A, size, L));
       if (L.fit < 1) continue;
-      const double us = makespan(n, L.fit, [&](int64_t q) {
+      const double below = (unlike && size > small ? UNLIKE_SIZE : 1.0) * team_us;
+      const double us = makespan(n, L.fit, below, [&](int64_t q) {
         return queued[q] * (CLUSTER_US + uneven * CLUSTER_US_PER_NZ *
                                              (double)system_cost(A, q, CLUSTER_ROW_NZ) / size);
       });
-      if (us >= (unlike && size > small ? UNLIKE_SIZE : 1.0) * team_us) continue;
+      if (us >= below) continue;
       team_us = us;
       A->batch_team = BATCH_CLUSTER;
       A->batch_cluster = size;
@@ -1019,7 +1029,7 @@ int batch_choice(gbs_mat A) {
       PHASES_US * most_its + op * work,
       most_its * (PHASES_US + (4.0 * (double)A->nnz + 44.0 * (double)A->nrows) / PHASES_BYTES_PER_US32)};
   for (int refined = 0; refined < 2; ++refined) {
-    const double cta = makespan(n, sm_count(A), [&](int64_t q) {
+    const double cta = makespan(n, sm_count(A), phases[refined], [&](int64_t q) {
       return queued[q] * (CTA_US + (refined ? CTA_US_PER_OP32 * (double)ops[q]
                                             : CTA_US_PER_NZ * (double)system_cost(A, q, CTA_ROW_NZ)));
     });
